@@ -1690,10 +1690,12 @@ void guess_reset_column(hdg_ctx* c, int j) {
 namespace {
 template <int DIM, int K>
 void launch_post(hdg_ctx* c, const double* u, const double* lam, double* pstar) {
+  using C = PostCfg<DIM, K>;
   const PostTabs P{c->d_post, c->d_post + c->post_k1};
   c->n_launch += 1;
-  post_kernel<DIM, K><<<grid_for(c, c->sk.ne * PostCfg<DIM, K>::NT, PostCfg<DIM, K>::NT), PostCfg<DIM, K>::NT, 0,
-                        c->stream>>>(devmesh(c), c->tabs, P, u, lam, pstar);
+  cudaFuncSetAttribute(post_kernel<DIM, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  post_kernel<DIM, K><<<(unsigned)std::min<int64_t>((c->sk.ne + C::EPW - 1) / C::EPW, 1 << 30), 32, C::SMEM, c->stream>>>(
+      devmesh(c), c->tabs, P, u, lam, pstar);
 }
 }  // namespace
 
@@ -2233,11 +2235,24 @@ hdg_status hdg_postprocess(hdg_ctx* c, const double* u, const double* lam, doubl
     } catch (const std::exception& ex) {
       return fail(c, HDG_EINVAL, std::string("post-processing tables: ") + ex.what());
     }
-    std::vector<double> tab(P.K1);
-    tab.insert(tab.end(), P.E1.begin(), P.E1.end());
+    // the layouts of PostTabs: packed lower triangles of the symmetric combinations of K1, and
+    // E1 transposed, both without the constant mode
+    const int d = c->dim, Np = c->Np, n1 = (int)std::lround(std::sqrt((double)P.K1.size() / (d * d)));
+    std::vector<double> tab;
+    auto k1 = [&](int r, int q, int i, int l) { return P.K1[(((size_t)r * d + q) * n1 + i) * n1 + l]; };
+    auto block = [&](int r, int q) {
+      for (int i = 1; i < n1; ++i)
+        for (int l = 1; l <= i; ++l) tab.push_back(r == q ? k1(r, r, i, l) : k1(r, q, i, l) + k1(q, r, i, l));
+    };
+    for (int r = 0; r < d; ++r) block(r, r);
+    for (int r = 0; r < d; ++r)
+      for (int q = r + 1; q < d; ++q) block(r, q);
+    c->post_k1 = (int64_t)tab.size();
+    for (int r = 0; r < d; ++r)
+      for (int l = 0; l < Np; ++l)
+        for (int i = 1; i < n1; ++i) tab.push_back(P.E1[((size_t)r * n1 + i) * Np + l]);
     hdg_status s;
     if ((s = dalloc(c, &c->d_post, tab.size()))) return s;
-    c->post_k1 = (int64_t)P.K1.size();
     CUDA_TRY(c, cudaMemcpyAsync(c->d_post, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));   // tab is released at return
   }

@@ -80,3 +80,23 @@ def test_postprocess_full_size_sampled():
     lam_sub = np.stack([lam[fid[tuple(f)]] for f in sub.sk.faces.tolist()])
     po = ac.postprocess_pressure(sub, u[sample], lam_sub)
     assert relerr(ps[sample], po) < 1e-12
+
+
+@pytest.mark.parametrize("dim,k", [(2, 1), (2, 4), (3, 1), (3, 3), (3, 4)])
+@pytest.mark.parametrize("ne", [1, 3, 5, 9])
+def test_postprocess_partial_element_groups_match_oracle(dim, k, ne):
+    """Element counts around the kernel's groups of four elements per warp (a last group with one
+    or three live elements), rows that do and do not fill the eight lanes of an element."""
+    import torch
+    from paper_1807_00086_gb300 import hdg
+    vert, elem = mesh(dim, 3)
+    elem = elem[:ne]
+    used, inv = np.unique(elem, return_inverse=True)
+    vert, elem = vert[used], inv.reshape(elem.shape).astype(np.int32)
+    c = inputs.loguniform(ne, 1.0, 3.0, 4)
+    s = hdg.Solver(vert, elem, k, 1.0, 1.0, c)
+    prob = ac.build_problem(vert, elem, k, 1.0, 1.0, c)
+    u = inputs.random_state(ne, s.n, 30 * dim + k)
+    lam = inputs.random_traces(s.n_faces, s.Nf, 40 * dim + k)
+    ps = s.hdg_postprocess(torch.tensor(u, device="cuda"), torch.tensor(lam, device="cuda")).cpu().numpy()
+    assert relerr(ps, ac.postprocess_pressure(prob, u, lam)) < 1e-12
