@@ -78,8 +78,8 @@ hdg_status svk_tables(hdg_ctx* c, Svk* v) {
   const double* b = v->d_tab;
   const float* bf = v->d_tabf - off[7];   // same offsets as the FP64 buffer
   v->tabs = SvkTabs{b + off[0], b + off[1], b + off[2], b + off[3], b + off[4], b + off[5], b + off[6], T.nqf};
-  v->tjd = SvkJT<double>{b + off[7], b + off[8], b + off[9], b + off[10]};
-  v->tjf = SvkJT<float>{bf + off[7], bf + off[8], bf + off[9], bf + off[10]};
+  v->tjd = SvkJT<double>{b + off[7], b + off[7], b + off[8], b + off[9], b + off[10]};
+  v->tjf = SvkJT<float>{bf + off[7], b + off[7], bf + off[8], bf + off[9], bf + off[10]};
   v->nqr = D::NQR;
   v->nqj = D::NQJ;
   CUDA_TRY(c, cudaFuncSetAttribute(svk_condense_kernel<K, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,

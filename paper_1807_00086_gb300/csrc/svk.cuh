@@ -55,7 +55,7 @@ struct SvkDims {
   static constexpr int PRE = 36 * NP + 108;
   static constexpr int CHJ = QC * (18 + 81 + 3 * NP + 4 * NFP + 1 + PRE);
   static constexpr int CHR = 9 * NQR;                 // P(F) at every residual point (double)
-  static constexpr int CHT = 9 * NQJ;                 // T-apply: values at the Jacobian points
+  static constexpr int CHT = 9 * NQJ + 9 * NP;        // T-apply: values at the Jacobian points, input in TJ
   // condensation kernel: double arena | scratch (double CHR or TJ chunk / T-apply) | TJ arena
   static constexpr int SMD = 32 + N + M + 3 * NP * NP + N + M + 4 * 9 * NP + 3 * NV;
   template <typename TJ>
@@ -91,6 +91,7 @@ struct SvkTabs {
 template <typename T>
 struct SvkJT {
   const T* phiJ;   // [NQJ][Np]
+  const double* phiD;   // the same in FP64
   const T* wJ;     // [NQJ]
   const T* GJ;     // [NQJ][3][Np]  sum_b Dr[r][a][b] phi_b(x_q)
   const T* PSJ;    // [NQJ][4][Nfp] sum_a Ff[f][a][m] phi_a(x_q)
@@ -152,14 +153,68 @@ __device__ __forceinline__ T svk_tangent_entry(const T* F, const T* S, const T* 
 }
 
 // F = I + H at a point with basis values phi [Np] (H: [9][Np] FP64 coefficients)
-template <int NP, typename PT>
-__device__ __forceinline__ void svk_deformation(const PT* __restrict__ phi, const double* H, double* F) {
+template <int NP>
+__device__ __forceinline__ void svk_deformation(const double* __restrict__ phi, const double* H, double* F) {
 #pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    double v = (c == 0 || c == 4 || c == 8) ? 1.0 : 0.0;
-    for (int a = 0; a < NP; ++a) v += H[c * NP + a] * (double)phi[a];
-    F[c] = v;
+  for (int c = 0; c < 9; ++c) F[c] = (c == 0 || c == 4 || c == 8) ? 1.0 : 0.0;
+  for (int a = 0; a < NP; ++a) {   // nine independent sums: the FP64 latency is off the path
+    const double ph = phi[a];
+#pragma unroll
+    for (int c = 0; c < 9; ++c) F[c] += H[c * NP + a] * ph;
   }
+}
+
+// w1 = L^{-1} b and zv = L^{-T} w1 for the lower factor L (row stride NV, shared memory) by warp
+// 0 of the block, lane l holding rows l + 32 t: column-oriented, so a step is one product, one
+// broadcast and one multiply-add per row block. Bounded by the FP64 latency of 2 NV such steps;
+// with one thread doing the NV^2 multiply-adds in sequence, a conversion of L in each, a DIRK3
+// step of the 1,536-tet plate (k = 2, FP32 Jacobian) took 43.9 ms instead of 34.3 ms.
+template <int NV, typename TJ>
+__device__ __forceinline__ void svk_factor_solve(const TJ* L, const double* b, double* w1, double* zv) {
+  constexpr int T = (NV + 31) / 32;
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  double x[T], rd[T];
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const int l = lane + 32 * t;
+    x[t] = l < NV ? b[l] : 0.0;
+    rd[t] = l < NV ? 1.0 / (double)L[l * NV + l] : 0.0;
+  }
+#pragma unroll
+  for (int t0 = 0; t0 < T; ++t0) {
+    const int n = NV - 32 * t0 < 32 ? NV - 32 * t0 : 32;
+    for (int li = 0; li < n; ++li) {
+      const int i = 32 * t0 + li;
+      const double wi = __shfl_sync(0xffffffffu, x[t0] * rd[t0], li);
+#pragma unroll
+      for (int t = t0; t < T; ++t) {
+        const int l = lane + 32 * t;
+        if (l == i) x[t] = wi;
+        else if (l > i && l < NV) x[t] -= (double)L[l * NV + i] * wi;
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (lane + 32 * t < NV) w1[lane + 32 * t] = x[t];
+#pragma unroll
+  for (int t0 = T - 1; t0 >= 0; --t0) {
+    const int n = NV - 32 * t0 < 32 ? NV - 32 * t0 : 32;
+    for (int li = n - 1; li >= 0; --li) {
+      const int i = 32 * t0 + li;
+      const double zi = __shfl_sync(0xffffffffu, x[t0] * rd[t0], li);
+#pragma unroll
+      for (int t = 0; t <= t0; ++t) {
+        const int l = lane + 32 * t;
+        if (l == i) x[t] = zi;
+        else if (l < i) x[t] -= (double)L[i * NV + l] * zi;
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (lane + 32 * t < NV) zv[lane + 32 * t] = x[t];
 }
 
 // y = T x (x, y: [9][Np] FP64 in shared memory) on the Jacobian rule in precision TJ; FJ
@@ -170,13 +225,17 @@ __device__ void svk_T_apply(const SvkJT<TJ>& tj, const TJ* FJ, TJ lam, TJ mu, TJ
   using D = SvkDims<K>;
   constexpr int NP = D::NP, NQJ = D::NQJ, NT = D::NT;
   const int tid = threadIdx.x;
+  // x in TJ, converted once: a conversion from FP64 issues at the FP64 rate
+  TJ* xj = scr + 9 * NQJ;
+  for (int t = tid; t < 9 * NP; t += NT) xj[t] = (TJ)x[t];
+  __syncthreads();
   for (int q = tid; q < NQJ; q += NT) {
     const TJ* ph = tj.phiJ + (int64_t)q * NP;
     TJ xv[9];
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
       TJ v = TJ(0);
-      for (int a = 0; a < NP; ++a) v += (TJ)x[c * NP + a] * ph[a];
+      for (int a = 0; a < NP; ++a) v += xj[c * NP + a] * ph[a];
       xv[c] = v;
     }
     const TJ* F = FJ + q * 9;
@@ -207,7 +266,7 @@ __device__ void svk_F_at_jac(const SvkJT<TJ>& tj, const double* H, TJ* FJ) {
   using D = SvkDims<K>;
   for (int q = threadIdx.x; q < D::NQJ; q += D::NT) {
     double F[9];
-    svk_deformation<D::NP, TJ>(tj.phiJ + (int64_t)q * D::NP, H, F);
+    svk_deformation<D::NP>(tj.phiD + (int64_t)q * D::NP, H, F);
 #pragma unroll
     for (int c = 0; c < 9; ++c) FJ[q * 9 + c] = (TJ)F[c];
   }
@@ -283,7 +342,7 @@ __global__ void __launch_bounds__(256, SvkMinBlocks<K, TJ>::value) svk_condense_
   // ---- residual (FP64): P(F) at the residual points, then the volume and face terms
   for (int q = tid; q < NQR; q += NT) {
     double F[9], S[9];
-    svk_deformation<NP, double>(tb.phiR + (int64_t)q * NP, Hc, F);
+    svk_deformation<NP>(tb.phiR + (int64_t)q * NP, Hc, F);
     svk_stress<double>(F, lam, mu, S, nullptr);
     const double w = tb.wR[q];
 #pragma unroll
@@ -327,9 +386,11 @@ __global__ void __launch_bounds__(256, SvkMinBlocks<K, TJ>::value) svk_condense_
       }
     } else {
       const int c = idx / NP - 12, aa = idx % NP;
-      double sq = 0.0;
-      for (int q = 0; q < NQR; ++q) sq += CHR[q * 9 + c] * tb.phiR[(int64_t)q * NP + aa];
-      v = dJ * (ue[idx] - sq);
+      double sq[4] = {0.0, 0.0, 0.0, 0.0};   // NQR = (2k + 2)^3 is a multiple of 4
+      for (int q = 0; q < NQR; q += 4)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) sq[b] += CHR[(q + b) * 9 + c] * tb.phiR[(int64_t)(q + b) * NP + aa];
+      v = dJ * (ue[idx] - ((sq[0] + sq[1]) + (sq[2] + sq[3])));
     }
     R[idx] = v;
   }
@@ -586,18 +647,7 @@ __global__ void __launch_bounds__(256, SvkMinBlocks<K, TJ>::value) svk_condense_
     rv[idx] = v;
   }
   __syncthreads();
-  if (tid == 0) {
-    for (int i = 0; i < NV; ++i) {
-      double v = rv[i];
-      for (int l = 0; l < i; ++l) v -= (double)Sv[i * NV + l] * w1[l];
-      w1[i] = v / (double)Sv[i * NV + i];
-    }
-    for (int i = NV - 1; i >= 0; --i) {
-      double v = w1[i];
-      for (int l = i + 1; l < NV; ++l) v -= (double)Sv[l * NV + i] * zv[l];
-      zv[i] = v / (double)Sv[i * NV + i];
-    }
-  }
+  svk_factor_solve<NV, TJ>(Sv, rv, w1, zv);
   __syncthreads();
   double* gK = a.slot + e * (int64_t)M;
   for (int idx = tid; idx < M; idx += NT) {
@@ -728,18 +778,7 @@ __global__ void __launch_bounds__(256, SvkMinBlocks<K, TJ>::value) svk_recover_k
     w1[idx] = v;
   }
   __syncthreads();
-  if (tid == 0) {
-    for (int i = 0; i < NV; ++i) {
-      double v = w1[i];
-      for (int l = 0; l < i; ++l) v -= (double)Ls[i * NV + l] * w1[l];
-      w1[i] = v / (double)Ls[i * NV + i];
-    }
-    for (int i = NV - 1; i >= 0; --i) {
-      double v = w1[i];
-      for (int l = i + 1; l < NV; ++l) v -= (double)Ls[l * NV + i] * zv[l];
-      zv[i] = v / (double)Ls[i * NV + i];
-    }
-  }
+  svk_factor_solve<NV, TJ>(Ls, w1, rv, zv);   // rv: L^{-1} of the right-hand side
   __syncthreads();
   for (int idx = tid; idx < 9 * NP; idx += NT) {
     const int c = idx / NP, aa = idx % NP, i = c / 3, J = c % 3;
