@@ -24,7 +24,12 @@
 //   A^{-1} R = (z_v, (R_H - Dx^T z_v) / (alpha d), (R_P + T z_H) / d),  z_v = S_v^{-1} (R_v + Dx y)
 //   C A^{-1} R = W^T z_v - BH^T y.
 // The three products Dx T Dx^T, Dx T BH and BH^T T BH are sums over the quadrature points of
-// outer products (one CTA per element, accumulators in registers); T is never formed.
+// outer products (one CTA per element); T is never formed. Each accumulation is cut into one
+// register tile per thread, so that a factor read from shared memory serves a row or a column of
+// products, and with an FP32 Jacobian all three share one pass over the points: bounded by the
+// FP64 residual and the barriers between the short phases. 1,536 tets, k = 2, FP32 Jacobian:
+// 0.97 ms (2.06 ms with one product per thread and read, three passes, three barriers per
+// Cholesky column and one thread's triangular solves).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -50,17 +55,33 @@ struct SvkDims {
   static constexpr int NQJ = QJ * QJ * QJ;
   static constexpr int QC = 8;                        // Jacobian points per chunk
   static constexpr int NT = 256;
-  // chunk area: per-point S and F F^T (18), tangent (81), g_J (3 N_p), psi_f (4 N_fp), weight,
-  // and the largest per-pass precompute (27 N_p, 36 N_p + 108 or 144 per point)
-  static constexpr int PRE = 36 * NP + 108;
-  static constexpr int CHJ = QC * (18 + 81 + 3 * NP + 4 * NFP + 1 + PRE);
+  // register tiles of the three accumulations, one tile per thread: (a) the 6 blocks i <= k of
+  // Np x Np, (b) the 36 blocks (i, i2, f) of Np x Nfp, (c) the 90 blocks (f <= f2, i, i2) of Nfp x Nfp
+  static constexpr int TAR = K == 1 ? 1 : (K == 2 ? 2 : 4), TAC = TAR;
+  static constexpr int TBR = K == 3 ? 4 : 2, TBC = K == 1 ? 1 : NFP;
+  static constexpr int TCR = K == 3 ? 5 : 3, TCC = NFP;
+  static constexpr int NTA = 6 * (NP / TAR) * (NP / TAC);
+  static constexpr int NTB = 36 * (NP / TBR) * (NFP / TBC);
+  static constexpr int NTC = 90 * (NFP / TCR) * (NFP / TCC);
+  static_assert(NP % TAR == 0 && NP % TBR == 0 && NFP % TBC == 0 && NFP % TCR == 0, "whole tiles");
+  static_assert(NTA <= NT && NTB <= NT && NTC <= NT, "one tile per thread");
+  // chunk area: stress and F F^T of two chunks (18 per point each), tangent (81), g_J (3 N_p),
+  // psi_f (4 N_fp), weight, and the precomputed factors of the passes that share a chunk:
+  // all three (FP32) or one at a time (FP64, whose registers and shared memory hold one)
+  template <typename TJ>
+  __host__ __device__ static constexpr bool fuse() { return sizeof(TJ) == 4; }
+  static constexpr int PA = 18 * NP, PB = 36 * NP, PN = 108, PC = 90;
+  template <typename TJ>
+  __host__ __device__ static constexpr int chj() {
+    return QC * (2 * 18 + 81 + 3 * NP + 4 * NFP + 1 + (fuse<TJ>() ? PA + PB + PN + PC : PB + PN));
+  }
   static constexpr int CHR = 9 * NQR;                 // P(F) at every residual point (double)
   static constexpr int CHT = 9 * NQJ + 9 * NP;        // T-apply: values at the Jacobian points, input in TJ
   // condensation kernel: double arena | scratch (double CHR or TJ chunk / T-apply) | TJ arena
   static constexpr int SMD = 32 + N + M + 3 * NP * NP + N + M + 4 * 9 * NP + 3 * NV;
   template <typename TJ>
   __host__ __device__ static constexpr size_t scr_bytes() {
-    const size_t a = sizeof(double) * CHR, b = sizeof(TJ) * (CHJ > CHT ? CHJ : CHT);
+    const size_t a = sizeof(double) * CHR, b = sizeof(TJ) * (chj<TJ>() > CHT ? chj<TJ>() : CHT);
     return ((a > b ? a : b) + 15) / 16 * 16;
   }
   template <typename TJ>
@@ -273,13 +294,6 @@ __device__ void svk_F_at_jac(const SvkJT<TJ>& tj, const double* H, TJ* FJ) {
   __syncthreads();
 }
 
-// upper-triangle index t -> (row, col) of an n x n matrix, row-major rows of n - r entries
-__device__ __forceinline__ void tri_decode(int t, int n, int& r, int& c) {
-  r = 0;
-  while (t >= n - r) { t -= n - r; ++r; }
-  c = r + t;
-}
-
 // CTAs per SM the register budget is cut for: two for the FP32 Jacobian up to k = 2
 template <int K, typename TJ>
 struct SvkMinBlocks { static constexpr int value = sizeof(TJ) == 4 && K <= 2 ? 2 : 1; };
@@ -409,88 +423,239 @@ __global__ void __launch_bounds__(256, SvkMinBlocks<K, TJ>::value) svk_condense_
   __syncthreads();   // the residual scratch is reused below
   svk_F_at_jac<K, TJ>(tj, Hc, FJ);   // barrier inside
   // chunk layout
-  TJ* cS = CH;                         // [QC][9]  S
-  TJ* cFF = cS + QC * 9;               // [QC][9]  F F^T
-  TJ* cA = cFF + QC * 9;               // [QC][81] tangent
+  constexpr bool FUSE = D::template fuse<TJ>();
+  TJ* cS = CH;                         // [2][QC][18]  S | F F^T of this chunk and the next
+  TJ* cA = cS + 2 * QC * 18;           // [QC][81] tangent
   TJ* cg = cA + QC * 81;               // [QC][3][Np] g_J
   TJ* cps = cg + QC * 3 * NP;          // [QC][4][Nfp] psi_f
-  TJ* cw = cps + QC * 4 * NFP;         // [QC] physical weights
-  TJ* cpre = cw + QC;                  // per-pass precompute
+  TJ* cw = cps + QC * 4 * NFP;         // [QC] physical weights (0 past the last point)
+  TJ* cn = cw + QC;                    // [QC][108] w sum_L A[iJ][i2 L] n_fL at (i, i2, f, J)
+  TJ* cb = cn + QC * D::PN;            // [QC][36][Np] factors of (b)
+  TJ* ca = FUSE ? cb + QC * D::PB : cn;            // [QC][6][3][Np] factors of (a)
+  TJ* cc = FUSE ? ca + QC * D::PA : cb;            // [QC][90] factors of (c)
   __shared__ TJ Jij[9], nj[12];   // J^{-1} and the normals in the Jacobian precision
   if (tid < 9) Jij[tid] = (TJ)Ji[tid];
   else if (tid < 21) nj[tid - 9] = (TJ)nrm[tid - 9];
-  __syncthreads();
-  // per chunk: S, F F^T, tangent, g_J, psi_f, weights of points q0 .. q0 + nq
-  auto load_chunk = [&](int q0, int nq) {
-    for (int t = tid; t < nq; t += NT) {
-      svk_stress<TJ>(FJ + (q0 + t) * 9, lamj, muj, cS + t * 9, cFF + t * 9);
-      cw[t] = tj.wJ[q0 + t] * dJj;
-    }
-    __syncthreads();
-    for (int t = tid; t < nq * 81; t += NT) {
+  // S and F F^T of chunk ch by the QC threads from t0 on
+  auto stress_chunk = [&](int ch, int t0) {
+    const int t = tid - t0;
+    if (t < 0 || t >= QC) return;
+    const int q = ch * QC + t < NQJ ? ch * QC + t : NQJ - 1;
+    TJ* d = cS + ((ch & 1) * QC + t) * 18;
+    svk_stress<TJ>(FJ + q * 9, lamj, muj, d, d + 9);
+  };
+  // tangent, g_J, psi_f and weights of a chunk; its stresses are in place. Points past the last
+  // one repeat it with weight zero, so every chunk has QC points.
+  auto load_chunk = [&](int ch) {
+    for (int t = tid; t < QC * 81; t += NT) {
       const int qq = t / 81, r = t % 81;
-      cA[t] = svk_tangent_entry<TJ>(FJ + (q0 + qq) * 9, cS + qq * 9, cFF + qq * 9, lamj, muj, r / 9, r % 9);
+      const int q = ch * QC + qq < NQJ ? ch * QC + qq : NQJ - 1;
+      const TJ* d = cS + ((ch & 1) * QC + qq) * 18;
+      cA[t] = svk_tangent_entry<TJ>(FJ + q * 9, d, d + 9, lamj, muj, r / 9, r % 9);
     }
-    for (int t = tid; t < nq * 3 * NP; t += NT) {
+    for (int t = tid; t < QC * 3 * NP; t += NT) {
       const int qq = t / (3 * NP), J = (t / NP) % 3, aa = t % NP;
-      const TJ* G = tj.GJ + (int64_t)(q0 + qq) * 3 * NP;
+      const int q = ch * QC + qq < NQJ ? ch * QC + qq : NQJ - 1;
+      const TJ* G = tj.GJ + (int64_t)q * 3 * NP;
       cg[t] = dJj * (Jij[J] * G[aa] + Jij[3 + J] * G[NP + aa] + Jij[6 + J] * G[2 * NP + aa]);
     }
-    for (int t = tid; t < nq * 4 * NFP; t += NT) {
+    for (int t = tid; t < QC * 4 * NFP; t += NT) {
       const int qq = t / (4 * NFP), f = (t / NFP) % 4;
-      cps[t] = (TJ)JF[f] * tj.PSJ[(int64_t)(q0 + qq) * 4 * NFP + t % (4 * NFP)];
+      const int q = ch * QC + qq < NQJ ? ch * QC + qq : NQJ - 1;
+      cps[t] = (TJ)JF[f] * tj.PSJ[(int64_t)q * 4 * NFP + t % (4 * NFP)];
     }
+    if (tid < QC) cw[tid] = ch * QC + tid < NQJ ? tj.wJ[ch * QC + tid] * dJj : TJ(0);
     __syncthreads();
   };
-  // ---- (a) Dx T Dx^T, upper triangle: [(i,a),(k,b)] = sum_q w sum_L t[i][k][L][a] g_L(q)_b,
-  //      t[i][k][L][a] = sum_J g_J(q)_a A[iJ][kL]
-  {
-    constexpr int NE = NV * (NV + 1) / 2, NS = (NE + NT - 1) / NT;
-    TJ acc[NS];
-    int rc[NS];
+  // Factors of a chunk; an item's decoding is shared by its HQ points.
+  constexpr int HQ = QC / 2;
+  auto factors_n = [&]() {   // the normals' contraction, used by (b) and (c)
+    for (int t = tid; t < 2 * D::PN; t += NT) {
+      const int r = t % D::PN, q0 = t / D::PN * HQ;
+      const int i = r / 36, i2 = (r / 12) % 3, f = (r / 3) % 4, J = r % 3;
+      const TJ n0 = nj[f * 3], n1 = nj[f * 3 + 1], n2 = nj[f * 3 + 2];
 #pragma unroll
-    for (int u = 0; u < NS; ++u) {
-      acc[u] = TJ(0);
-      const int t = tid + u * NT;
-      int r = 0, c = 0;
-      if (t < NE) tri_decode(t, NV, r, c);
-      rc[u] = (r << 16) | c;
-    }
-    for (int q0 = 0; q0 < NQJ; q0 += QC) {
-      const int nq = NQJ - q0 < QC ? NQJ - q0 : QC;
-      load_chunk(q0, nq);
-      for (int t = tid; t < nq * 27 * NP; t += NT) {
-        const int qq = t / (27 * NP), ikL = (t / NP) % 27, aa = t % NP;
-        const int i = ikL / 9, k = (ikL / 3) % 3, L = ikL % 3;
-        const TJ* A = cA + qq * 81;
-        const TJ* gg = cg + qq * 3 * NP;
-        cpre[t] = gg[aa] * A[(i * 3) * 9 + k * 3 + L] + gg[NP + aa] * A[(i * 3 + 1) * 9 + k * 3 + L] +
-                  gg[2 * NP + aa] * A[(i * 3 + 2) * 9 + k * 3 + L];
+      for (int qq = q0; qq < q0 + HQ; ++qq) {
+        const TJ* A = cA + qq * 81 + (i * 3 + J) * 9 + i2 * 3;
+        cn[qq * D::PN + r] = cw[qq] * (A[0] * n0 + A[1] * n1 + A[2] * n2);
       }
-      __syncthreads();
+    }
+  };
+  auto factors_a = [&]() {   // w sum_J g_J(q)_a A[iJ][kL] at (i <= k, L, a)
+    for (int t = tid; t < 2 * D::PA; t += NT) {
+      const int r = t % D::PA, q0 = t / D::PA * HQ;
+      const int p = r / (3 * NP), L = (r / NP) % 3, aa = r % NP;
+      const int i = p < 3 ? 0 : (p < 5 ? 1 : 2), k = p < 3 ? p : (p < 5 ? p - 2 : 2);
 #pragma unroll
-      for (int u = 0; u < NS; ++u) {
-        if (tid + u * NT < NE) {
-          const int r = rc[u] >> 16, c = rc[u] & 0xffff;
-          const int i = r / NP, aa = r % NP, k = c / NP, b = c % NP;
-          TJ v = acc[u];
-          for (int qq = 0; qq < nq; ++qq) {
-            const TJ* tt = cpre + ((qq * 27) + i * 9 + k * 3) * NP + aa;
-            const TJ* gg = cg + qq * 3 * NP + b;
-            v += cw[qq] * (tt[0] * gg[0] + tt[NP] * gg[NP] + tt[2 * NP] * gg[2 * NP]);
-          }
-          acc[u] = v;
+      for (int qq = q0; qq < q0 + HQ; ++qq) {
+        const TJ* A = cA + qq * 81 + (i * 3) * 9 + k * 3 + L;
+        const TJ* gg = cg + qq * 3 * NP + aa;
+        ca[qq * D::PA + r] = cw[qq] * (gg[0] * A[0] + gg[NP] * A[9] + gg[2 * NP] * A[18]);
+      }
+    }
+  };
+  auto factors_b = [&]() {   // sum_J g_J(q)_a cn at (i, i2, f, a)
+    for (int t = tid; t < 2 * D::PB; t += NT) {
+      const int r = t % D::PB, q0 = t / D::PB * HQ;
+      const int c36 = r / NP, aa = r % NP;
+#pragma unroll
+      for (int qq = q0; qq < q0 + HQ; ++qq) {
+        const TJ* cj = cn + qq * D::PN + c36 * 3;
+        const TJ* gg = cg + qq * 3 * NP + aa;
+        cb[qq * D::PB + r] = gg[0] * cj[0] + gg[NP] * cj[1] + gg[2 * NP] * cj[2];
+      }
+    }
+  };
+  // block pair index 0..9 -> (f <= f2)
+  auto pair_f = [](int p, int& f, int& f2) {
+    f = p < 4 ? 0 : (p < 7 ? 1 : (p < 9 ? 2 : 3));
+    f2 = p < 4 ? p : (p < 7 ? p - 3 : (p < 9 ? p - 5 : 3));
+  };
+  auto factors_c = [&]() {   // n_f^T A^{(i, i2)} n_f2 with the weight, at (f <= f2, i, i2)
+    for (int t = tid; t < 2 * D::PC; t += NT) {
+      const int r = t % D::PC, q0 = t / D::PC * HQ;
+      int f, f2;
+      pair_f(r / 9, f, f2);
+      const int i = (r / 3) % 3, i2 = r % 3;
+      const TJ n0 = nj[f * 3], n1 = nj[f * 3 + 1], n2 = nj[f * 3 + 2];
+#pragma unroll
+      for (int qq = q0; qq < q0 + HQ; ++qq) {
+        const TJ* cj = cn + qq * D::PN + ((i * 3 + i2) * 4 + f2) * 3;
+        cc[qq * D::PC + r] = n0 * cj[0] + n1 * cj[1] + n2 * cj[2];
+      }
+    }
+  };
+  // this thread's tiles
+  constexpr int TAR = D::TAR, TAC = D::TAC, TBR = D::TBR, TBC = D::TBC, TCR = D::TCR, TCC = D::TCC;
+  const bool hasA = tid < D::NTA, hasB = tid < D::NTB, hasC = tid < D::NTC;
+  const int pa = hasA ? tid / ((NP / TAR) * (NP / TAC)) : 0;
+  const int a0 = hasA ? (tid / (NP / TAC)) % (NP / TAR) * TAR : 0, b0 = hasA ? tid % (NP / TAC) * TAC : 0;
+  const int ia = pa < 3 ? 0 : (pa < 5 ? 1 : 2), ka = pa < 3 ? pa : (pa < 5 ? pa - 2 : 2);
+  const int pb = hasB ? tid / ((NP / TBR) * (NFP / TBC)) : 0;
+  const int br0 = hasB ? (tid / (NFP / TBC)) % (NP / TBR) * TBR : 0, bc0 = hasB ? tid % (NFP / TBC) * TBC : 0;
+  const int pc = hasC ? tid / ((NFP / TCR) * (NFP / TCC)) : 0;
+  const int cr0 = hasC ? (tid / (NFP / TCC)) % (NFP / TCR) * TCR : 0, cc0 = hasC ? tid % (NFP / TCC) * TCC : 0;
+  int cf, cf2;
+  pair_f(pc / 9, cf, cf2);
+  const int ci = (pc / 3) % 3, ci2 = pc % 3;
+  TJ accA[TAR][TAC], accB[TBR][TBC], accC[TCR][TCC];
+#pragma unroll
+  for (int x = 0; x < TAR; ++x)
+#pragma unroll
+    for (int z = 0; z < TAC; ++z) accA[x][z] = TJ(0);
+#pragma unroll
+  for (int x = 0; x < TBR; ++x)
+#pragma unroll
+    for (int z = 0; z < TBC; ++z) accB[x][z] = TJ(0);
+#pragma unroll
+  for (int x = 0; x < TCR; ++x)
+#pragma unroll
+    for (int z = 0; z < TCC; ++z) accC[x][z] = TJ(0);
+  // ---- (a) Dx T Dx^T: [(i,a),(k,b)] = sum_q sum_L ca[i][k][L][a] g_L(q)_b
+  auto sum_a = [&]() {
+    if (!hasA) return;
+#pragma unroll 2
+    for (int qq = 0; qq < QC; ++qq)
+#pragma unroll
+      for (int L = 0; L < 3; ++L) {
+        const TJ* tt = ca + qq * D::PA + (pa * 3 + L) * NP + a0;
+        const TJ* gg = cg + (qq * 3 + L) * NP + b0;
+        TJ gv[TAC];
+#pragma unroll
+        for (int z = 0; z < TAC; ++z) gv[z] = gg[z];
+#pragma unroll
+        for (int x = 0; x < TAR; ++x)
+#pragma unroll
+          for (int z = 0; z < TAC; ++z) accA[x][z] += tt[x] * gv[z];
+      }
+  };
+  // ---- (b) Dx T BH: [(i,a),(f,i2,m)] = -sum_q cb[i][i2][f][a] psi_f(q)_m
+  auto sum_b = [&]() {
+    if (!hasB) return;
+#pragma unroll 2
+    for (int qq = 0; qq < QC; ++qq) {
+      const TJ* tt = cb + qq * D::PB + pb * NP + br0;
+      const TJ* ps = cps + (qq * 4 + pb % 4) * NFP + bc0;
+      TJ pv[TBC];
+#pragma unroll
+      for (int z = 0; z < TBC; ++z) pv[z] = ps[z];
+#pragma unroll
+      for (int x = 0; x < TBR; ++x)
+#pragma unroll
+        for (int z = 0; z < TBC; ++z) accB[x][z] += tt[x] * pv[z];
+    }
+  };
+  // ---- (c) BH^T T BH: [(f,i,m),(f2,i2,m2)] = sum_q cc[f][f2][i][i2] psi_f(q)_m psi_f2(q)_m2
+  auto sum_c = [&]() {
+    if (!hasC) return;
+#pragma unroll 2
+    for (int qq = 0; qq < QC; ++qq) {
+      const TJ w = cc[qq * D::PC + pc];
+      const TJ* p1 = cps + (qq * 4 + cf) * NFP + cr0;
+      const TJ* p2 = cps + (qq * 4 + cf2) * NFP + cc0;
+      TJ pv[TCC];
+#pragma unroll
+      for (int z = 0; z < TCC; ++z) pv[z] = p2[z];
+#pragma unroll
+      for (int x = 0; x < TCR; ++x) {
+        const TJ wx = w * p1[x];
+#pragma unroll
+        for (int z = 0; z < TCC; ++z) accC[x][z] += wx * pv[z];
+      }
+    }
+  };
+  constexpr int NCH = (NQJ + QC - 1) / QC;
+  if constexpr (FUSE) {
+    // the stresses of the next chunk are formed by the last warp, which holds few tiles, while
+    // the others accumulate
+    stress_chunk(0, 0);
+    __syncthreads();
+    for (int ch = 0; ch < NCH; ++ch) {
+      load_chunk(ch);
+      factors_n();
+      factors_a();
+      __syncthreads();
+      factors_b();
+      factors_c();
+      __syncthreads();
+      if (ch + 1 < NCH) stress_chunk(ch + 1, NT - 32);
+      sum_a();
+      sum_b();
+      sum_c();
+      __syncthreads();
+    }
+  } else {
+    // one pass over the points per accumulation
+    for (int pass = 0; pass < 3; ++pass)
+      for (int ch = 0; ch < NCH; ++ch) {
+        stress_chunk(ch, 0);
+        __syncthreads();
+        load_chunk(ch);
+        if (pass == 0) {
+          factors_a();
+          __syncthreads();
+          sum_a();
+        } else {
+          factors_n();
+          __syncthreads();
+          if (pass == 1) factors_b();
+          else factors_c();
+          __syncthreads();
+          if (pass == 1) sum_b();
+          else sum_c();
         }
+        __syncthreads();
       }
-      __syncthreads();
-    }
+  }
+  if (hasA) {
 #pragma unroll
-    for (int u = 0; u < NS; ++u) {
-      if (tid + u * NT < NE) {
-        const int r = rc[u] >> 16, c = rc[u] & 0xffff;
-        const int i = r / NP, aa = r % NP, k = c / NP, b = c % NP;
-        double v = iad2 * (double)acc[u];
-        if (i == k) {
+    for (int x = 0; x < TAR; ++x)
+#pragma unroll
+      for (int z = 0; z < TAC; ++z) {
+        const int aa = a0 + x, b = b0 + z, r = ia * NP + aa, c = ka * NP + b;
+        if (r > c) continue;   // the diagonal blocks' lower half is the mirror of the upper one
+        double v = iad2 * (double)accA[x][z];
+        if (ia == ka) {
           double ev = 0.0;
           for (int f = 0; f < 4; ++f) ev += JF[f] * tb.Ef[(f * NP + aa) * NP + b];
           v += s * ev + (aa == b ? alpha * rho * dJ : 0.0);
@@ -498,142 +663,88 @@ __global__ void __launch_bounds__(256, SvkMinBlocks<K, TJ>::value) svk_condense_
         Sv[r * NV + c] = (TJ)v;
         Sv[c * NV + r] = (TJ)v;
       }
-    }
   }
-  // ---- (b) Dx T BH: [(i,a),(f,i2,m)] = -sum_q w u[i][i2][f][a] psi_f(q)_m,
-  //      u[i][i2][f][a] = sum_J g_J(q)_a sum_L A[iJ][i2 L] n_fL;   W = Bv + Dx T BH / (alpha d^2)
-  {
-    constexpr int NE = NV * M, NS = (NE + NT - 1) / NT;
-    TJ acc[NS];
+  if (hasB) {   // W = Bv + Dx T BH / (alpha d^2)
+    const int i = pb / 12, i2 = (pb / 4) % 3, f = pb % 4;
 #pragma unroll
-    for (int u = 0; u < NS; ++u) acc[u] = TJ(0);
-    for (int q0 = 0; q0 < NQJ; q0 += QC) {
-      const int nq = NQJ - q0 < QC ? NQJ - q0 : QC;
-      load_chunk(q0, nq);
-      // c_J[i][i2][f] = sum_L A[iJ][i2 L] n_fL, then u = sum_J g_J c_J
-      TJ* ccj = cpre + QC * 36 * NP;
-      for (int t = tid; t < nq * 108; t += NT) {
-        const int qq = t / 108, r = t % 108;
-        const int i = r / 36, i2 = (r / 12) % 3, f = (r / 3) % 4, J = r % 3;
-        const TJ* A = cA + qq * 81 + (i * 3 + J) * 9 + i2 * 3;
-        ccj[t] = A[0] * nj[f * 3] + A[1] * nj[f * 3 + 1] + A[2] * nj[f * 3 + 2];
-      }
-      __syncthreads();
-      for (int t = tid; t < nq * 36 * NP; t += NT) {
-        const int qq = t / (36 * NP), c36 = (t / NP) % 36, aa = t % NP;
-        const TJ* cj = ccj + qq * 108 + c36 * 3;
-        const TJ* gg = cg + qq * 3 * NP + aa;
-        cpre[t] = gg[0] * cj[0] + gg[NP] * cj[1] + gg[2 * NP] * cj[2];
-      }
-      __syncthreads();
+    for (int x = 0; x < TBR; ++x)
 #pragma unroll
-      for (int u = 0; u < NS; ++u) {
-        const int t = tid + u * NT;
-        if (t < NE) {
-          const int r = t / M, col = t % M;
-          const int i = r / NP, aa = r % NP, f = col / NF, i2 = (col % NF) / NFP, m = col % NFP;
-          TJ v = acc[u];
-          for (int qq = 0; qq < nq; ++qq)
-            v += cw[qq] * cpre[((qq * 36) + i * 12 + i2 * 4 + f) * NP + aa] * cps[(qq * 4 + f) * NFP + m];
-          acc[u] = v;
-        }
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < NS; ++u) {
-      const int t = tid + u * NT;
-      if (t < NE) {
-        const int r = t / M, col = t % M;
-        const int i = r / NP, aa = r % NP, f = col / NF, i2 = (col % NF) / NFP, m = col % NFP;
-        double v = -iad2 * (double)acc[u];
+      for (int z = 0; z < TBC; ++z) {
+        const int aa = br0 + x, m = bc0 + z;
+        double v = -iad2 * (double)accB[x][z];
         if (i == i2) v -= s * JF[f] * tb.Ff[(f * NP + aa) * NFP + m];
-        W[t] = (TJ)v;
+        W[(i * NP + aa) * M + f * NF + i2 * NFP + m] = (TJ)v;
       }
-    }
   }
+  // ---- Cholesky S_v = L L^T with W's rows carried along: column j leaves the trailing block and
+  // W through its unscaled entries over the pivot (one barrier a column), and the scalings of L
+  // and of Z = L^{-1} W follow in one pass
+  __shared__ TJ rdv[NV];   // 1 / pivot
   __syncthreads();
-  // ---- Cholesky S_v = L L^T (in place, lower), then Z = L^{-1} W
-  for (int j = 0; j < NV; ++j) {
-    if (tid == 0) {
-      TJ dd = Sv[j * NV + j];
-      if (!(dd > TJ(0))) { atomicExch(a.err, 1); dd = TJ(1); }
-      Sv[j * NV + j] = tsqrt(dd);
-    }
+  auto pivot = [&](int j) {
+    TJ dd = Sv[j * NV + j];
+    if (!(dd > TJ(0))) { atomicExch(a.err, 1); dd = TJ(1); Sv[j * NV + j] = dd; }
+    rdv[j] = TJ(1) / dd;
+  };
+  if (tid == 0) pivot(0);
+  for (int j = 0; j < NV - 1; ++j) {
     __syncthreads();
-    for (int i = j + 1 + tid; i < NV; i += NT) Sv[i * NV + j] /= Sv[j * NV + j];
-    __syncthreads();
+    const TJ rd = rdv[j];
     const int w = NV - j - 1;
     for (int idx = tid; idx < w * w; idx += NT) {
       const int i = j + 1 + idx / w, l = j + 1 + idx % w;
-      if (l <= i) Sv[i * NV + l] -= Sv[i * NV + j] * Sv[l * NV + j];
+      if (l <= i) Sv[i * NV + l] -= Sv[i * NV + j] * rd * Sv[l * NV + j];
     }
-    __syncthreads();
-  }
-  for (int col = tid; col < M; col += NT) {
-    for (int i = 0; i < NV; ++i) {
-      TJ v = W[i * M + col];
-      for (int l = 0; l < i; ++l) v -= Sv[i * NV + l] * W[l * M + col];
-      W[i * M + col] = v / Sv[i * NV + i];
+    for (int idx = tid; idx < w * M; idx += NT) {
+      const int l = j + 1 + idx / M, col = idx % M;
+      W[l * M + col] -= Sv[l * NV + j] * rd * W[j * M + col];
     }
+    if (tid == 0) pivot(j + 1);   // thread 0 updated this entry itself
   }
   __syncthreads();
-  // ---- (c) BH^T T BH, upper triangle: [(f,i,m),(f2,i2,m2)] = sum_q w c[f][i][f2][i2] psi_f(q)_m psi_f2(q)_m2,
-  //      c = n_f^T A^{(i,i2)} n_f2;   S_K = D - Z^T Z + BH^T T BH / (alpha d^2)
-  {
-    constexpr int NE = M * (M + 1) / 2, NS = (NE + NT - 1) / NT;
-    TJ acc[NS];
-    int rc[NS];
-#pragma unroll
-    for (int u = 0; u < NS; ++u) {
-      acc[u] = TJ(0);
-      const int t = tid + u * NT;
-      int r = 0, c = 0;
-      if (t < NE) tri_decode(t, M, r, c);
-      rc[u] = (r << 16) | c;
-    }
-    for (int q0 = 0; q0 < NQJ; q0 += QC) {
-      const int nq = NQJ - q0 < QC ? NQJ - q0 : QC;
-      load_chunk(q0, nq);
-      for (int t = tid; t < nq * 144; t += NT) {
-        const int qq = t / 144, c144 = t % 144;
-        const int f = c144 / 36, i = (c144 / 12) % 3, f2 = (c144 / 3) % 4, i2 = c144 % 3;
-        const TJ* A = cA + qq * 81;
-        TJ v = TJ(0);
-#pragma unroll
-        for (int J = 0; J < 3; ++J)
-#pragma unroll
-          for (int L = 0; L < 3; ++L) v += nj[f * 3 + J] * A[(i * 3 + J) * 9 + i2 * 3 + L] * nj[f2 * 3 + L];
-        cpre[t] = cw[qq] * v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < NS; ++u) {
-        if (tid + u * NT < NE) {
-          const int c1 = rc[u] >> 16, c2 = rc[u] & 0xffff;
-          const int f = c1 / NF, i = (c1 % NF) / NFP, m = c1 % NFP;
-          const int f2 = c2 / NF, i2 = (c2 % NF) / NFP, m2 = c2 % NFP;
-          TJ v = acc[u];
-          for (int qq = 0; qq < nq; ++qq)
-            v += cpre[qq * 144 + f * 36 + i * 12 + f2 * 3 + i2] * cps[(qq * 4 + f) * NFP + m] * cps[(qq * 4 + f2) * NFP + m2];
-          acc[u] = v;
-        }
-      }
-      __syncthreads();
-    }
+  if (tid < NV) {   // diagonal of L, 1 / L_jj for the scalings
+    const TJ l = tsqrt(Sv[tid * NV + tid]);
+    Sv[tid * NV + tid] = l;
+    rdv[tid] = TJ(1) / l;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < NV * NV; idx += NT) {
+    const int i = idx / NV, j = idx % NV;
+    if (j < i) Sv[idx] *= rdv[j];
+  }
+  for (int idx = tid; idx < NV * M; idx += NT) W[idx] *= rdv[idx / M];
+  __syncthreads();
+  // ---- S_K = D - Z^T Z + BH^T T BH / (alpha d^2)
+  if (hasC) {
     double* Se = a.S + e * (int64_t)(M * M);
+    const int r0 = cf * NF + ci * NFP + cr0, c0 = cf2 * NF + ci2 * NFP + cc0;
+    TJ zz[TCR][TCC];
 #pragma unroll
-    for (int u = 0; u < NS; ++u) {
-      if (tid + u * NT < NE) {
-        const int c1 = rc[u] >> 16, c2 = rc[u] & 0xffff;
-        TJ zz = TJ(0);
-        for (int r = 0; r < NV; ++r) zz += W[r * M + c1] * W[r * M + c2];
-        double v = iad2 * (double)acc[u] - (double)zz;
-        if (c1 == c2) v += s * JF[c1 / NF];
+    for (int x = 0; x < TCR; ++x)
+#pragma unroll
+      for (int z = 0; z < TCC; ++z) zz[x][z] = TJ(0);
+    for (int r = 0; r < NV; ++r) {
+      TJ zv2[TCC];
+#pragma unroll
+      for (int z = 0; z < TCC; ++z) zv2[z] = W[r * M + c0 + z];
+#pragma unroll
+      for (int x = 0; x < TCR; ++x) {
+        const TJ z1 = W[r * M + r0 + x];
+#pragma unroll
+        for (int z = 0; z < TCC; ++z) zz[x][z] += z1 * zv2[z];
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < TCR; ++x)
+#pragma unroll
+      for (int z = 0; z < TCC; ++z) {
+        const int c1 = r0 + x, c2 = c0 + z;
+        if (c1 > c2) continue;   // same face: the lower half is the mirror of the upper one
+        double v = iad2 * (double)accC[x][z] - (double)zz[x][z];
+        if (c1 == c2) v += s * JF[cf];
         Se[c1 * M + c2] = v;
         Se[c2 * M + c1] = v;
       }
-    }
   }
   // ---- condensed right-hand side and A^{-1} R (FP64 vectors; the Jacobian factors in TJ)
   svk_T_apply<K, TJ>(tj, FJ, lamj, muj, dJj, R + 3 * NP, t1, CH);           // T R_H
