@@ -13,6 +13,7 @@
 
 #include "../../include/hdg.h"
 #include "kernels.cuh"
+#include "condense.cuh"
 #include "post.cuh"
 #include "dflocal.cuh"
 #include "multi.cuh"
@@ -31,7 +32,6 @@ namespace {
 
 template <int DIM, int K>
 void launch_condense(hdg_ctx* c) {
-  constexpr int NT = 128;
   c->n_launch += 2;
   if (c->phys == HDG_ELASTIC) {
     const size_t smem = CondElCfg<DIM, K>::SMEM;
@@ -41,8 +41,11 @@ void launch_condense(hdg_ctx* c) {
     diag_kernel<ElDims<DIM, K>><<<grid_for(c, c->sk.nf * c->Nf), 256, 0, c->stream>>>(devmesh(c), c->d_S, c->sgn, c->d_dinv);
     return;
   }
-  condense_kernel<DIM, K, NT><<<(unsigned)c->sk.ne, NT, 0, c->stream>>>(devmesh(c), c->tabs, c->alpha, c->tau, c->d_S,
-                                                                       c->d_Hinv, c->d_err);
+  using C = CondCfg<DIM, K>;
+  cudaFuncSetAttribute(condense_kernel<DIM, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  condense_kernel<DIM, K><<<(unsigned)((c->sk.ne + C::EPW - 1) / C::EPW), 32, C::SMEM, c->stream>>>(
+      devmesh(c), CondTabs{c->d_condtab, c->tabs.Ff, c->tabs.DFrf, c->tabs.Pfg}, c->alpha, c->tau, c->d_S, c->d_Hinv,
+      c->d_err);
   diag_kernel<Dims<DIM, K>><<<grid_for(c, c->sk.nf * c->Nf), 256, 0, c->stream>>>(devmesh(c), c->d_S, c->sgn, c->d_dinv);
 }
 
@@ -100,14 +103,6 @@ void launch_apply(hdg_ctx* c, const double* x, double* zslot, const int* done, i
 }
 
 template <int DIM, int K>
-void launch_pack32(hdg_ctx* c) {
-  using PK = Packed<DIM, K>;
-  const int64_t n = ((c->sk.ne + 31) / 32) * PK::P4 * 128;
-  c->n_launch += 1;
-  pack32_kernel<DIM, K><<<grid_for(c, n), 256, 0, c->stream>>>(c->sk.ne, c->d_S, c->d_S32);
-}
-
-template <int DIM, int K>
 void launch_face_q64(hdg_ctx* c) {
   if (c->phys == HDG_ELASTIC)
     cg_face_q_kernel<ElDims<DIM, K>><<<c->nb_red, 256, 0, c->stream>>>((int)c->sk.nf, c->sgn, c->d_face_slot, c->d_face_bnd,
@@ -147,22 +142,27 @@ void launch_face_q32(hdg_ctx* c) {
                                                                        c->d_part, c->d_sc);
 }
 
+// every FP32 / FP16 / double-float copy of S_K that the context's solves read
 template <int DIM, int K>
-void launch_packdf(hdg_ctx* c) {
-  using PK = Packed<DIM, K>;
-  const int64_t n = c->sk.ne * PK::P4 * 4;
+void launch_pack(hdg_ctx* c) {
+  using C = PackCfg<DIM, K>;
+  PackOut o{};
+  if (c->R == 1) {
+    o.Sdf = c->d_Sdf; o.S32 = c->d_S32; o.S16 = c->d_S16; o.sc16 = c->d_sc16;
+  } else {
+    (c->R >= 32 ? o.S32m : o.S32) = c->d_S32;
+    o.Shi = c->d_mShi; o.Slo = c->d_mSlo;
+  }
   c->n_launch += 1;
-  packdf_kernel<DIM, K><<<grid_for(c, n), 256, 0, c->stream>>>(c->sk.ne, c->d_S, c->d_Sdf);
+  cudaFuncSetAttribute(pack_kernel<DIM, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  // whole 32-element groups
+  pack_kernel<DIM, K><<<(unsigned)((c->sk.ne + 31) / 32 * (32 / C::EPB)), 256, C::SMEM, c->stream>>>(c->sk.ne, c->d_S, o);
 }
 
+// gather table, shared memory and resident CTAs of the FP16 apply
 template <int DIM, int K>
-void launch_pack16(hdg_ctx* c) {
-  using PK = Packed16<DIM, K>;
+void prepare_apply16(hdg_ctx* c) {
   const int64_t ne = c->sk.ne;
-  c->n_launch += 2;
-  scale16_kernel<DIM, K><<<grid_for(c, ne * 32), 256, 0, c->stream>>>(ne, c->d_S, c->d_sc16);
-  pack16_kernel<DIM, K><<<grid_for(c, ((ne + 31) / 32) * PK::P8 * 256), 256, 0, c->stream>>>(ne, c->d_S, c->d_sc16,
-                                                                                               c->d_S16);
   using C = Apply16Cfg<DIM, K>;
   const int64_t ng = ((ne + 31) / 32) * 32 * Dims<DIM, K>::NFC;
   c->n_launch += 1;
@@ -228,14 +228,6 @@ void attr_apply_tc(hdg_ctx* c) {
       per_sm < 1)
     per_sm = 1;
   c->tcp_per_sm = per_sm;
-}
-
-template <int DIM, int K>
-void launch_pack32m(hdg_ctx* c) {
-  using PK = Packed<DIM, K>;
-  const int64_t n = c->sk.ne * PK::P4 * 4;
-  c->n_launch += 1;
-  pack32m_kernel<DIM, K><<<grid_for(c, n), 256, 0, c->stream>>>(c->sk.ne, c->d_S, c->d_S32);
 }
 
 template <int DIM, int K>
@@ -316,24 +308,14 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
       const int64_t nS = c->sk.ne * (int64_t)c->m * c->m;
       c->n_launch += 1;
       to32_copy_kernel<<<grid_for(c, nS), 256, 0, c->stream>>>(nS, c->d_S, c->d_S32);
-    } else if (c->R > 1) {
-      if (c->R >= 32) {
-        HDG_DISPATCH(c, launch_pack32m, c);
-        HDG_DISPATCH(c, attr_apply_tc, c);
-      } else {
-        HDG_DISPATCH(c, launch_pack32, c);   // group layout, read by the narrow multi-column apply
-      }
-      const int64_t nS = c->sk.ne * (int64_t)c->m * c->m;
-      c->n_launch += 1;
-      split_df_kernel<<<grid_for(c, nS), 256, 0, c->stream>>>(nS, c->d_S, c->d_mShi, c->d_mSlo);
-      const int64_t nH = c->sk.ne * (int64_t)c->nv * c->nv;
-      c->n_launch += 1;
-      to_df_kernel<<<grid_for(c, nH), 256, 0, c->stream>>>(nH, c->d_Hinv, c->d_Hinvdf);
     } else {
-      HDG_DISPATCH(c, launch_pack32, c);
-      HDG_DISPATCH(c, launch_packdf, c);
-      HDG_DISPATCH(c, attr_apply_df, c);
-      if (c->d_S16) HDG_DISPATCH(c, launch_pack16, c);
+      HDG_DISPATCH(c, launch_pack, c);
+      if (c->R >= 32) {
+        HDG_DISPATCH(c, attr_apply_tc, c);
+      } else if (c->R == 1) {
+        HDG_DISPATCH(c, attr_apply_df, c);
+        if (c->d_S16) HDG_DISPATCH(c, prepare_apply16, c);
+      }
       const int64_t nH = c->sk.ne * (int64_t)c->nv * c->nv;
       c->n_launch += 1;
       to_df_kernel<<<grid_for(c, nH), 256, 0, c->stream>>>(nH, c->d_Hinv, c->d_Hinvdf);
@@ -1953,6 +1935,23 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   CUDA_TRY(c, cudaMemcpyAsync(c->d_tab, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, c->stream));
   c->tabs.Dr = c->d_tab + off[0]; c->tabs.Ff = c->d_tab + off[1]; c->tabs.Ef = c->d_tab + off[2];
   c->tabs.Trs = c->d_tab + off[3]; c->tabs.DFrf = c->d_tab + off[4]; c->tabs.Pfg = c->d_tab + off[5];
+  if (c->phys == HDG_ACOUSTIC) {
+    // lower triangles, packed by rows, of the terms of the local pressure block H (CondTabs::HP)
+    const int Np = c->T.Np, d = c->dim;
+    std::vector<double> hp;
+    auto tri = [&](const double* A, const double* B) {
+      for (int i = 0; i < Np; ++i)
+        for (int l = 0; l <= i; ++l) hp.push_back(A[(size_t)i * Np + l] + (B ? B[(size_t)i * Np + l] : 0.0));
+    };
+    const size_t blk = (size_t)Np * Np;
+    for (int f = 0; f <= d; ++f) tri(&c->T.Ef[f * blk], nullptr);
+    for (int r = 0; r < d; ++r) tri(&c->T.Trs[(size_t)(r * d + r) * blk], nullptr);
+    for (int r = 0; r < d; ++r)
+      for (int q = r + 1; q < d; ++q) tri(&c->T.Trs[(size_t)(r * d + q) * blk], &c->T.Trs[(size_t)(q * d + r) * blk]);
+    if ((s = dalloc(c, &c->d_condtab, hp.size()))) return s;
+    CUDA_TRY(c, cudaMemcpyAsync(c->d_condtab, hp.data(), hp.size() * 8, cudaMemcpyHostToDevice, c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));   // hp is released here
+  }
   if ((s = dalloc(c, &c->d_qv_w, c->T.qv_w.size()))) return s;
   if ((s = dalloc(c, &c->d_qv_phi, c->T.qv_phi.size()))) return s;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_qv_w, c->T.qv_w.data(), c->T.qv_w.size() * 8, cudaMemcpyHostToDevice, c->stream));

@@ -43,6 +43,7 @@ struct hdg_ctx {
   int32_t *d_elem_face = nullptr, *d_face_slot = nullptr, *d_face_bnd = nullptr;
   int64_t* d_bnd_faces = nullptr;
   Tabs tabs{};
+  double* d_condtab = nullptr;   // packed tables of the acoustic condensation (CondTabs::HP)
   double *d_qv_w = nullptr, *d_qv_phi = nullptr;
   // condensed operators
   double *d_S = nullptr, *d_Hinv = nullptr, *d_dinv = nullptr;

@@ -54,12 +54,6 @@ struct LocalDfCfg {
   static constexpr int NT = EPB * NP;
 };
 
-// Double-float copy of an FP64 array (H^{-1} after each condensation, the element geometry).
-static __global__ void to_df_kernel(int64_t n, const double* __restrict__ a, df2* __restrict__ out) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-    out[t] = df_from(a[t]);
-}
-
 // EPB elements per CTA, one thread per (element, row i < NP). geo: double-float copy of the
 // element geometry; Hinv: double-float H^{-1} [ne][NP][NP] (symmetric, read as columns).
 template <int DIM, int K, int MODE>

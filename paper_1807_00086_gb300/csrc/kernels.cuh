@@ -66,118 +66,6 @@ struct Dims {
   static constexpr int ON = 1 + DIM * DIM + DIM + 1;
 };
 
-// ---------------------------------------------------------------- condensation (a)(b)(c)
-// One CTA per element: assemble H, Cholesky H = L L^T, W = L^{-1} Bt, S = W^T W + ...,
-// H^{-1} = L^{-T} L^{-1}. Writes S [ne][M][M] and Hinv [ne][NP][NP].
-template <int DIM, int K, int NT>
-__global__ void __launch_bounds__(NT) condense_kernel(DevMesh mesh, Tabs T, double alpha, double tau,
-                                                      double* __restrict__ S, double* __restrict__ Hinv,
-                                                      int* __restrict__ err) {
-  using D = Dims<DIM, K>;
-  constexpr int NP = D::NP, NF = D::NF, M = D::M, NFC = D::NFC;
-  __shared__ double H[NP * NP];
-  __shared__ double W[NP * M];
-  __shared__ double Li[NP * NP];
-  __shared__ double g[GEO_STRIDE];
-  __shared__ double Grs[DIM * DIM], Bfr[NFC * DIM], nn[NFC * NFC];
-  const int64_t e = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (tid < GEO_STRIDE) g[tid] = mesh.geo[e * GEO_STRIDE + tid];
-  __syncthreads();
-  const double dJ = g[0];
-  const double rho = mesh.rho[e], cc = mesh.c[e];
-  const double a = alpha / (rho * cc * cc), b = alpha * rho;
-  if (tid < DIM * DIM) {
-    int r = tid / DIM, s = tid % DIM;
-    double v = 0.0;
-    for (int j = 0; j < DIM; ++j) v += g[1 + r * DIM + j] * g[1 + s * DIM + j];
-    Grs[tid] = v;
-  } else if (tid < DIM * DIM + NFC * DIM) {
-    int t = tid - DIM * DIM, f = t / DIM, r = t % DIM;
-    double v = 0.0;
-    for (int j = 0; j < DIM; ++j) v += g[D::ON + f * DIM + j] * g[1 + r * DIM + j];
-    Bfr[t] = v;
-  } else if (tid < DIM * DIM + NFC * DIM + NFC * NFC) {
-    int t = tid - DIM * DIM - NFC * DIM, f = t / NFC, h = t % NFC;
-    double v = 0.0;
-    for (int j = 0; j < DIM; ++j) v += g[D::ON + f * DIM + j] * g[D::ON + h * DIM + j];
-    nn[t] = v;
-  }
-  __syncthreads();
-  for (int idx = tid; idx < NP * NP; idx += NT) {
-    const int i = idx / NP, l = idx % NP;
-    double v = (i == l) ? a * dJ : 0.0;
-    double fe = 0.0;
-    for (int f = 0; f < NFC; ++f) fe += g[D::OJF + f] * T.Ef[(f * NP + i) * NP + l];
-    double dd = 0.0;
-    for (int rs = 0; rs < DIM * DIM; ++rs) dd += Grs[rs] * T.Trs[(rs * NP + i) * NP + l];
-    H[idx] = v + tau * fe + (dJ / b) * dd;
-    Li[idx] = (i == l) ? 1.0 : 0.0;
-  }
-  for (int idx = tid; idx < NP * M; idx += NT) {
-    const int i = idx / M, col = idx % M, f = col / NF, mm = col % NF;
-    double v = tau * T.Ff[(f * NP + i) * NF + mm];
-    double d2 = 0.0;
-    for (int r = 0; r < DIM; ++r) d2 += Bfr[f * DIM + r] * T.DFrf[((r * NFC + f) * NP + i) * NF + mm];
-    W[idx] = -g[D::OJF + f] * (v + d2 / b);
-  }
-  __syncthreads();
-  // Cholesky, right-looking, lower triangle in place
-  for (int j = 0; j < NP; ++j) {
-    if (tid == 0) {
-      double d = H[j * NP + j];
-      if (!(d > 0.0)) { atomicExch(err, 1); d = 1.0; }
-      H[j * NP + j] = sqrt(d);
-    }
-    __syncthreads();
-    for (int i = j + 1 + tid; i < NP; i += NT) H[i * NP + j] /= H[j * NP + j];
-    __syncthreads();
-    const int w = NP - j - 1;
-    for (int idx = tid; idx < w * w; idx += NT) {
-      const int i = j + 1 + idx / w, l = j + 1 + idx % w;
-      if (l <= i) H[i * NP + l] -= H[i * NP + j] * H[l * NP + j];
-    }
-    __syncthreads();
-  }
-  // forward substitution, one column per thread: W <- L^{-1} Bt, Li <- L^{-1}
-  for (int col = tid; col < M + NP; col += NT) {
-    if (col < M) {
-      for (int i = 0; i < NP; ++i) {
-        double s = W[i * M + col];
-        for (int l = 0; l < i; ++l) s -= H[i * NP + l] * W[l * M + col];
-        W[i * M + col] = s / H[i * NP + i];
-      }
-    } else {
-      const int c2 = col - M;
-      for (int i = c2; i < NP; ++i) {
-        double s = (i == c2) ? 1.0 : 0.0;
-        for (int l = c2; l < i; ++l) s -= H[i * NP + l] * Li[l * NP + c2];
-        Li[i * NP + c2] = s / H[i * NP + i];
-      }
-    }
-  }
-  __syncthreads();
-  double* Se = S + e * (int64_t)(M * M);
-  const double ib = 1.0 / (b * dJ);
-  for (int idx = tid; idx < M * M; idx += NT) {
-    const int ra = idx / M, cb = idx % M;
-    const int f = ra / NF, aa = ra % NF, h = cb / NF, bb = cb % NF;
-    double s = 0.0;
-    for (int i = 0; i < NP; ++i) s += W[i * M + ra] * W[i * M + cb];
-    if (ra == cb) s -= tau * g[D::OJF + f];
-    s -= ib * g[D::OJF + f] * g[D::OJF + h] * nn[f * NFC + h] * T.Pfg[((f * NFC + h) * NF + aa) * NF + bb];
-    Se[idx] = s;
-  }
-  double* He = Hinv + e * (int64_t)(NP * NP);
-  for (int idx = tid; idx < NP * NP; idx += NT) {
-    const int i = idx / NP, l = idx % NP;
-    const int q0 = i > l ? i : l;
-    double s = 0.0;
-    for (int q = q0; q < NP; ++q) s += Li[q * NP + i] * Li[q * NP + l];
-    He[idx] = s;
-  }
-}
-
 // Jacobi preconditioner: dinv = sgn / (sum over the face's slots of diag S_K), sgn = -1 for the
 // acoustic convention (K negative definite), +1 for the elastic one (K positive definite).
 template <class D>
@@ -746,31 +634,6 @@ struct Packed {
 
 __host__ __device__ constexpr int packed_index(int M, int r, int c) { return r * M - r * (r - 1) / 2 + (c - r); }
 
-template <int DIM, int K>
-__global__ void pack32_kernel(int64_t ne, const double* __restrict__ S, float* __restrict__ S32) {
-  using PK = Packed<DIM, K>;
-  constexpr int M = PK::M, P4 = PK::P4;
-  const int64_t ngroups = (ne + 31) / 32;
-  const int64_t n = ngroups * P4 * 32 * 4;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int j = (int)(t & 3);
-    const int lane = (int)((t >> 2) & 31);
-    const int64_t q = (t >> 7) % P4;
-    const int64_t g = (t >> 7) / P4;
-    const int64_t e = g * 32 + lane;
-    const int p = (int)(q * 4 + j);
-    float v = 0.f;
-    if (e < ne && p < PK::P) {
-      // invert the packed index: row r holds entries [packed_index(r, r), packed_index(r, M-1)]
-      int r = 0;
-      while (packed_index(M, r, M - 1) < p) ++r;
-      const int c = r + (p - packed_index(M, r, r));
-      v = (float)S[e * (int64_t)(M * M) + r * M + c];
-    }
-    S32[t] = v;
-  }
-}
-
 // p.q of the Krylov iteration, formed inside the element apply: with q = sgn K p and K the
 // sum of the element blocks, p.q = sgn sum_K p_K . (S_K p_K) (boundary entries of p are zero
 // on both sides). Each 4-warp block writes its partial; the last block to finish (ticket
@@ -908,46 +771,6 @@ struct Packed16 {
   static constexpr int P = M * (M + 1) / 2;
   static constexpr int P8 = (P + 7) / 8;
 };
-
-template <int DIM, int K>
-__global__ void scale16_kernel(int64_t ne, const double* __restrict__ S, float* __restrict__ sc16) {
-  constexpr int M = Dims<DIM, K>::M;
-  const int lane = threadIdx.x & 31;
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t e = w; e < ne; e += nw) {
-    double m = 0.0;
-    for (int i = lane; i < M * M; i += 32) m = fmax(m, fabs(S[e * (int64_t)(M * M) + i]));
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    // round the scale up so that |S / sc| <= 1 holds after the FP32 rounding of sc
-    if (lane == 0) sc16[e] = m > 0.0 ? __double2float_ru(m) : 1.f;
-  }
-}
-
-template <int DIM, int K>
-__global__ void pack16_kernel(int64_t ne, const double* __restrict__ S, const float* __restrict__ sc16,
-                              __half* __restrict__ S16) {
-  using PK = Packed16<DIM, K>;
-  constexpr int M = PK::M, P8 = PK::P8;
-  const int64_t ngroups = (ne + 31) / 32;
-  const int64_t n = ngroups * P8 * 32 * 8;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int j = (int)(t & 7);
-    const int lane = (int)((t >> 3) & 31);
-    const int64_t q = (t >> 8) % P8;
-    const int64_t g = (t >> 8) / P8;
-    const int64_t e = g * 32 + lane;
-    const int p = (int)(q * 8 + j);
-    float v = 0.f;
-    if (e < ne && p < PK::P) {
-      int r = 0;
-      while (packed_index(M, r, M - 1) < p) ++r;
-      const int c = r + (p - packed_index(M, r, r));
-      v = (float)(S[e * (int64_t)(M * M) + r * M + c] / (double)sc16[e]);
-    }
-    S16[t] = __float2half_rn(v);
-  }
-}
 
 // Trace gather table of the FP16 apply: gface[e][f] = the id of face f of element e where it
 // carries trace unknowns (an interior face), else -1; rows past the last element are -1
@@ -1406,28 +1229,6 @@ struct DfAcc {
 // off(s) + r with off(s) = packed_index(M, s, s) (the s-th superdiagonal follows the first s
 // ones). hi = fl32(S), lo = fl32(S - hi).
 __host__ __device__ constexpr int diag_off(int M, int s) { return packed_index(M, s, s); }
-
-template <int DIM, int K>
-__global__ void packdf_kernel(int64_t ne, const double* __restrict__ S, float* __restrict__ Sdf) {
-  using PK = Packed<DIM, K>;
-  constexpr int M = PK::M, PD = PK::P4 * 4;
-  const int64_t n = ne * PD;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = t / PD;
-    const int pos = (int)(t - e * PD);
-    float hi = 0.f, lo = 0.f;
-    if (pos < PK::P) {
-      int s = 0;
-      while (s < M - 1 && diag_off(M, s + 1) <= pos) ++s;
-      const int r = pos - diag_off(M, s);
-      const double v = S[e * (int64_t)(M * M) + r * M + r + s];
-      hi = __double2float_rn(v);
-      lo = __double2float_rn(v - (double)hi);
-    }
-    Sdf[e * 2 * PD + pos] = hi;
-    Sdf[e * 2 * PD + PD + pos] = lo;
-  }
-}
 
 // FP64-accurate refinement apply on the FP32 pipe: zslot[e][r] = sum_c S_K[r][c] x_K[c] with
 // S_K = hi + lo from the diagonal-major copy and x split into double-floats. CTA = EPB

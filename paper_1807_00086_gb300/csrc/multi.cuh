@@ -270,37 +270,6 @@ __global__ void __launch_bounds__(32 * ApplyDfMCfg<DIM, K>::WPB) apply_df_multi_
   }
 }
 
-// hi = fl32(S), lo = fl32(S - hi), full [e][m][m]
-static __global__ void split_df_kernel(int64_t n, const double* __restrict__ S, float* __restrict__ hi,
-                                       float* __restrict__ lo) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const float h = __double2float_rn(S[t]);
-    hi[t] = h;
-    lo[t] = __double2float_rn(S[t] - (double)h);
-  }
-}
-
-// FP32 S for the multi-column path: element-major packed upper triangles [e][P4] float4, so a
-// CTA streams its elements' blocks contiguously into shared memory.
-template <int DIM, int K>
-__global__ void pack32m_kernel(int64_t ne, const double* __restrict__ S, float* __restrict__ S32m) {
-  using PK = Packed<DIM, K>;
-  constexpr int M = PK::M, P4 = PK::P4;
-  const int64_t n = ne * P4 * 4;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = t / (P4 * 4);
-    const int p = (int)(t % (P4 * 4));
-    float v = 0.f;
-    if (p < PK::P) {
-      int r = 0;
-      while (packed_index(M, r, M - 1) < p) ++r;
-      const int c = r + (p - packed_index(M, r, r));
-      v = (float)S[e * (int64_t)(M * M) + r * M + c];
-    }
-    S32m[t] = v;
-  }
-}
-
 // CTA = EPB elements x all column groups (CG = R/32 warps per element); the elements' packed
 // S_K are staged once in shared memory and read by every warp as broadcasts.
 template <int DIM, int K>
