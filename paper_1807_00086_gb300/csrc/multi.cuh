@@ -231,8 +231,11 @@ __global__ void __launch_bounds__(128) apply_multi_kernel(int64_t ne, int R, con
 
 // FP64-accurate R-column apply on the FP32 pipe (the refinement residual of the mixed
 // multi-column path): S_K = hi + lo as full row-major FP32 pairs [e][m][m], x split into
-// double-floats and staged lane-contiguous in shared memory, one compensated accumulator per
-// (row, lane). Warp = 32 / CWN elements x CWN columns.
+// double-floats and staged lane-contiguous in shared memory. Warp = 32 / CWN elements x CWN columns.
+// Four rows (three where M is no multiple of four) share each x from shared memory, and four
+// entries of a row one 16-byte load, so that the kernel is bounded by its FP32 instructions (11 per
+// product) and not by the load unit: one row and one entry at a time took
+// 1.81 ms for 24,576 tets x 64 columns (k = 3), against 1.29 ms; R = 4, 16,464 tets: 0.255 -> 0.173 ms.
 template <int DIM, int K>
 struct ApplyDfMCfg {   // warps per block: the staged x (M x 32 double-floats per warp) stays under 48 KB
   static constexpr int WPB = Dims<DIM, K>::M * 32 * 8 * 4 <= 48 * 1024 ? 4 : 2;
@@ -262,11 +265,43 @@ __global__ void __launch_bounds__(32 * ApplyDfMCfg<DIM, K>::WPB) apply_df_multi_
   if (!live) return;
   const float* Sh = Shi + e * (int64_t)(M * M);
   const float* Sl = Slo + e * (int64_t)(M * M);
-  for (int r = 0; r < M; ++r) {
-    DfAcc acc;
-#pragma unroll 8
-    for (int c = 0; c < M; ++c) acc.fma(df2{__ldg(Sh + r * M + c), __ldg(Sl + r * M + c)}, xs[w][c][lane]);
-    slot[(e * M + r) * R + j] = acc.value();
+  double* out = slot + e * (int64_t)M * R + j;
+  if constexpr (M % 4 == 0) {
+    for (int r = 0; r < M; r += 4) {
+      DfAcc acc[4];
+#pragma unroll 2
+      for (int c = 0; c < M; c += 4) {
+        float h[4][4], l[4][4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float4 u = __ldg(reinterpret_cast<const float4*>(Sh + (r + b) * M + c));
+          const float4 v = __ldg(reinterpret_cast<const float4*>(Sl + (r + b) * M + c));
+          h[b][0] = u.x; h[b][1] = u.y; h[b][2] = u.z; h[b][3] = u.w;
+          l[b][0] = v.x; l[b][1] = v.y; l[b][2] = v.z; l[b][3] = v.w;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const df2 xc = xs[w][c + k][lane];
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[b].fma(df2{h[b][k], l[b][k]}, xc);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b) out[(int64_t)(r + b) * R] = acc[b].value();
+    }
+  } else {
+    static_assert(M % 3 == 0, "rows in threes");
+    for (int r = 0; r < M; r += 3) {
+      DfAcc acc[3];
+#pragma unroll
+      for (int c = 0; c < M; ++c) {
+        const df2 xc = xs[w][c][lane];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) acc[b].fma(df2{__ldg(Sh + (r + b) * M + c), __ldg(Sl + (r + b) * M + c)}, xc);
+      }
+#pragma unroll
+      for (int b = 0; b < 3; ++b) out[(int64_t)(r + b) * R] = acc[b].value();
+    }
   }
 }
 
