@@ -1590,7 +1590,7 @@ hdg_status guess_before_v(hdg_ctx* c, int64_t n, const double* b, double* x, con
   const int nb = c->nb_red;
   c->n_launch += 3;
   gdots_kernel<<<nb, 256, 0, c->stream>>>(n, c->d_gd, c->d_gb, b, c->d_gpart);
-  gsolve_kernel<<<1, 256, 0, c->stream>>>(nb, c->d_gpart, c->d_gd);
+  gsolve_kernel<<<1, kGsolveThreads, 0, c->stream>>>(nb, c->d_gpart, c->d_gd);
   glincomb_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(n, c->d_gd, c->d_gl, mask, x);
   return check_launch(c, "guess");
 }
