@@ -947,17 +947,6 @@ void mlaunch_local_cw(hdg_ctx* c, int mode, const double* F, const double* hist,
                       double* out) {
   using L = LocalMultiCfg<DIM, K, CWW>;
   dim3 grid((unsigned)c->sk.ne, (unsigned)((c->R + L::CW - 1) / L::CW));
-  if (c->d_Hinvdf) {   // mixed precision: double-float on the FP32 pipe
-    const float th = (float)c->tau;
-    const df2 tau{th, (float)(c->tau - (double)th)};
-    if (mode == 0)
-      local_df_multi_kernel<DIM, K, 0, CWW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf,
-                                                                           c->alpha, tau, c->R, F, hist, sa, lam, out);
-    else
-      local_df_multi_kernel<DIM, K, 1, CWW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf,
-                                                                           c->alpha, tau, c->R, F, hist, sa, lam, out);
-    return;
-  }
   if (mode == 0)
     local_multi_kernel<DIM, K, 0, CWW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabs, c->d_Hinv, c->alpha, c->tau,
                                                                        c->R, F, hist, sa, lam, out);
@@ -966,16 +955,38 @@ void mlaunch_local_cw(hdg_ctx* c, int mode, const double* F, const double* hist,
                                                                        c->R, F, hist, sa, lam, out);
 }
 
+// mixed precision: double-float on the FP32 pipe
+template <int DIM, int K, int CW>
+void mlaunch_local_df(hdg_ctx* c, int mode, const double* F, const double* hist, const SrcArgs& sa, const double* lam,
+                      double* out) {
+  using L = LocalDfMCfg<DIM, K, CW>;
+  const dim3 grid((unsigned)((c->sk.ne + L::EPB - 1) / L::EPB), (unsigned)(c->R / CW));
+  const float th = (float)c->tau;
+  const df2 tau{th, (float)(c->tau - (double)th)};
+  if (mode == 0)
+    local_df_multi_kernel<DIM, K, 0, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf,
+                                                                        c->alpha, tau, c->R, F, hist, sa, lam, out);
+  else
+    local_df_multi_kernel<DIM, K, 1, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf,
+                                                                        c->alpha, tau, c->R, F, hist, sa, lam, out);
+}
+
 template <int DIM, int K>
 void mlaunch_local(hdg_ctx* c, int mode, const double* F, const double* hist, double t, const double* lam, double* out) {
   const SrcArgs sa = srcargs(c, t);
   c->n_launch += 1;
   // as many columns per CTA as the batch has (up to the kernel's width)
-  // (the double-float kernels of the mixed path take at most 16, for three CTAs per SM)
+  if (c->d_Hinvdf) {
+    if (c->R <= 2) mlaunch_local_df<DIM, K, 2>(c, mode, F, hist, sa, lam, out);
+    else if (c->R <= 4) mlaunch_local_df<DIM, K, 4>(c, mode, F, hist, sa, lam, out);
+    else if (c->R <= 8) mlaunch_local_df<DIM, K, 8>(c, mode, F, hist, sa, lam, out);
+    else mlaunch_local_df<DIM, K, 16>(c, mode, F, hist, sa, lam, out);
+    return;
+  }
   if (c->R <= 2) mlaunch_local_cw<DIM, K, 2>(c, mode, F, hist, sa, lam, out);
   else if (c->R <= 4) mlaunch_local_cw<DIM, K, 4>(c, mode, F, hist, sa, lam, out);
   else if (c->R <= 8) mlaunch_local_cw<DIM, K, 8>(c, mode, F, hist, sa, lam, out);
-  else if (c->R <= 16 || c->d_Hinvdf) mlaunch_local_cw<DIM, K, 16>(c, mode, F, hist, sa, lam, out);
+  else if (c->R <= 16) mlaunch_local_cw<DIM, K, 16>(c, mode, F, hist, sa, lam, out);
   else mlaunch_local_cw<DIM, K, 32>(c, mode, F, hist, sa, lam, out);
 }
 

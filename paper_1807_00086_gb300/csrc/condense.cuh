@@ -207,26 +207,6 @@ __global__ void __launch_bounds__(32) condense_kernel(DevMesh mesh, CondTabs T, 
   }
 }
 
-// hi = fl32(v), lo = fl32(v - hi), bit for bit as the FP64 conversions give them, on the integer
-// pipe: the four FP64 instructions of the other route cost a copy kernel more than its bytes do
-// (to_df_kernel on 33 M entries: 0.234 -> 0.090 ms).
-__device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
-  const unsigned hw = (unsigned)__double2hiint(v), lw = (unsigned)__double2loint(v);
-  const int ex = (int)((hw >> 20) & 0x7ffu);
-  if (ex < 960 || ex > 1140) {   // zero, tiny, huge, infinite: by conversion
-    hi = __double2float_rn(v);
-    lo = __double2float_rn(v - (double)hi);
-    return;
-  }
-  const unsigned m = ((hw & 0xfffffu) << 3) | (lw >> 29), rem = lw & 0x1fffffffu;
-  const unsigned up = rem > 0x10000000u || (rem == 0x10000000u && (m & 1u)) ? 1u : 0u;   // nearest, ties to even
-  const unsigned sign = hw & 0x80000000u;
-  hi = __uint_as_float(sign | ((((unsigned)(ex - 896) << 23) | m) + up));
-  // the signed remainder in units of the last FP64 place, rounded once
-  const float rl = (float)((int)rem - (int)(up << 29)) * __uint_as_float((unsigned)(ex - 948) << 23);
-  lo = sign ? -rl : rl;
-}
-
 // Double-float copy of an FP64 array (H^{-1} after each condensation, the element geometry).
 static __global__ void to_df_kernel(int64_t n, const double* __restrict__ a, df2* __restrict__ out) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
