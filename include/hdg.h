@@ -401,10 +401,10 @@ hdg_status hdg_trace_apply_noalloc(int32_t dim, int32_t k, int64_t n_elem, int64
 
 /* Tiles of the per-element-degree (elastic, elem_k) kernels, chosen by the library's
  * autotuner on the context's own data: at the first hdg_condense it times each candidate tile
- * of the matrix-free apply (warps per block in {4, 8} x columns in flight in {4, 8, 16}) on
- * the condensed operator: apply64 is the FP64-accurate apply (the FP64 kernel, or with mixed
- * precision the double-float refinement-residual kernel), apply32 the FP32 inner apply
- * (mixed precision). At the first local solve of
+ * of the FP64 matrix-free apply (warps per block in {4, 8} x columns in flight in {4, 8, 16})
+ * on the condensed operator: apply64. With mixed precision the applies (apply64: the
+ * double-float refinement-residual kernel, apply32: the inner apply) read packed copies of S_K
+ * and have one tile, 4 warps x 8 entries per lane. At the first local solve of
  * each kind it times the block size of the one-launch element-local solve (64, 128 or 256
  * threads per element). tuned = 0 before the first condensation; local_threads are 0 until
  * the first condensed right-hand side (index 0) / recovery (index 1). HDG_EINVAL for a

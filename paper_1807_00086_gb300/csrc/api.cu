@@ -122,24 +122,38 @@ hdg_status reset_dev_timing(hdg_ctx* c) {
 // p.q reduction target of the single-column FP32/FP16 applies, with the launch-timing slot
 PqOut pq_out(hdg_ctx* c, DevTiming* timing) { return PqOut{c->d_pqpart, c->d_ticket, c->d_pq, (float)c->sgn, timing}; }
 
-template <int DIM, int K>
-void launch_update_f32(hdg_ctx* c, int par) {
-  cg32_update_f_kernel<Dims<DIM, K>><<<c->nb_red, 256, 0, c->stream>>>(
-      c->nfe4 / 4, c->sk.nf * c->Nf, (float)c->sgn, par, c->d_face_slot, c->d_face_bnd, c->d_slot32,
-      (const float4*)c->d_p32, (const float4*)c->d_dinv32, (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-      c->d_pq, c->d_part + c->nb_red, c->d_sc);
+// CTAs of kernel A of the two-kernel iteration
+inline int two_na(const hdg_ctx* c) {
+  if (c->phys == HDG_ELASTIC) return (int)std::max<int64_t>(1, std::min<int64_t>((c->sk.ne + 3) / 4, (int64_t)c->sms * 16));
+  return (int)(((c->sk.ne + 31) / 32 + 3) / 4);
+}
+// dev != 0: device-driven loop with condition h
+Cg2Args two_args(hdg_ctx* c, int par, int dev, cudaGraphConditionalHandle h) {
+  return Cg2Args{c->d_sc, c->d_two, c->d_twoA, c->d_twoB, two_na(c), c->nb_red, par, c->opt.maxit, dev, (float)c->sgn, h};
 }
 
+// vector update with p.q from the FP16 apply (three-kernel iteration), or kernel B of the two-kernel one
 template <int DIM, int K>
-void launch_face_q32(hdg_ctx* c) {
-  if (c->phys == HDG_ELASTIC)
-    cg32_face_q_kernel<ElDims<DIM, K>><<<c->nb_red, 256, 0, c->stream>>>((int)c->sk.nf, (float)c->sgn, c->d_face_slot,
-                                                                         c->d_face_bnd, c->d_slot32, c->d_p32, c->d_q32,
-                                                                         c->d_part, c->d_sc);
-  else
-    cg32_face_q_kernel<Dims<DIM, K>><<<c->nb_red, 256, 0, c->stream>>>((int)c->sk.nf, (float)c->sgn, c->d_face_slot,
-                                                                       c->d_face_bnd, c->d_slot32, c->d_p32, c->d_q32,
-                                                                       c->d_part, c->d_sc);
+void launch_update_f32(hdg_ctx* c, int par) {
+  using Q = QFaces<Dims<DIM, K>>;
+  cg32_update_f_kernel<Q, false><<<c->nb_red, 256, 0, c->stream>>>(
+      c->nfe4 / 4, (float)c->sgn, par, Q{c->sk.nf * c->Nf, (const int2*)c->d_face_slot, c->d_face_bnd}, c->d_slot32,
+      (float4*)c->d_p32,
+      (const float4*)c->d_dinv32, (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32, c->d_pq, c->d_part + c->nb_red,
+      c->d_sc, Cg2Args{});
+}
+template <class L>
+void launch_update_two_l(hdg_ctx* c, const Cg2Args& o) {
+  using Q = QFaces<L>;
+  cg32_update_f_kernel<Q, true><<<c->nb_red, 256, 0, c->stream>>>(
+      c->nfe4 / 4, (float)c->sgn, o.parity, Q{c->sk.nf * c->Nf, (const int2*)c->d_face_slot, c->d_face_bnd}, c->d_slot32,
+      (float4*)c->d_p32,
+      (const float4*)c->d_dinv32, (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32, nullptr, nullptr, c->d_sc, o);
+}
+template <int DIM, int K>
+void launch_update_two(hdg_ctx* c, const Cg2Args& o) {
+  if (c->phys == HDG_ELASTIC) launch_update_two_l<ElDims<DIM, K>>(c, o);
+  else launch_update_two_l<Dims<DIM, K>>(c, o);
 }
 
 // every FP32 / FP16 / double-float copy of S_K that the context's solves read
@@ -235,16 +249,42 @@ void launch_apply32(hdg_ctx* c, const float* x, float* slot, const int* done, in
   const int64_t ngroups = (c->sk.ne + 31) / 32;
   c->n_launch += 1;
   cudaEvent_t stop = apply_begin(c, 1, iter);
-  if (c->phys == HDG_ELASTIC) {
-    apply32f_kernel<ElDims<DIM, K>><<<(unsigned)((c->sk.ne + 3) / 4), 128, 0, c->stream>>>(
-        c->sk.ne, c->d_elem_face, c->d_face_bnd, c->d_S32, x, slot, done);
-    apply_end(c, stop);
+  apply32_kernel<DIM, K, false><<<(unsigned)((ngroups + 3) / 4), 128, 0, c->stream>>>(
+      c->sk.ne, c->d_elem_face, c->d_face_bnd, c->d_S32, x, nullptr, slot, done, pq_out(c, c->d_dtime), Cg2Args{});
+  apply_end(c, stop);
+}
+
+// kernel A of the two-kernel FP32 iteration
+template <int DIM, int K>
+void launch_apply_two(hdg_ctx* c, const Cg2Args& o, int iter) {
+  c->n_launch += 1;
+  cudaEvent_t stop = apply_begin(c, 1, iter);
+  if (c->phys == HDG_ELASTIC)
+    apply32f_kernel<ElDims<DIM, K>><<<(unsigned)o.na, 128, 0, c->stream>>>(c->sk.ne, c->d_elem_face, c->d_face_bnd, c->d_S32,
+                                                                           c->d_z32, c->d_p32, c->d_slot32, o);
+  else
+    apply32_kernel<DIM, K, true><<<(unsigned)o.na, 128, 0, c->stream>>>(c->sk.ne, c->d_elem_face, c->d_face_bnd, c->d_S32,
+                                                                        c->d_z32, c->d_p32, c->d_slot32, nullptr,
+                                                                        pq_out(c, c->d_dtime), o);
+  apply_end(c, stop);
+}
+
+// one iteration of the FP32 inner PCG on the context's FP32 vectors: apply and update with the FP32
+// copy of S_K; apply, update and direction with the FP16 copy, whose gather is staged by
+// asynchronous copies and has no room for a second vector. dev != 0: loop condition h
+void inner32_iter(hdg_ctx* c, bool use16, int par, int dev, cudaGraphConditionalHandle h, int iter) {
+  if (!use16) {
+    const Cg2Args o = two_args(c, par, dev, h);
+    HDG_DISPATCH(c, launch_apply_two, c, o, iter);
+    c->n_launch += 1;
+    HDG_DISPATCH(c, launch_update_two, c, o);
     return;
   }
-  apply32_kernel<DIM, K><<<(unsigned)((ngroups + 3) / 4), 128, 0, c->stream>>>(c->sk.ne, c->d_elem_face, c->d_face_bnd,
-                                                                              c->d_S32, x, slot, done,
-                                                                              pq_out(c, c->d_dtime));
-  apply_end(c, stop);
+  HDG_DISPATCH(c, launch_apply16, c, c->d_p32, c->d_slot32, &c->d_sc->done, iter);
+  c->n_launch += 2;
+  HDG_DISPATCH(c, launch_update_f32, c, par);
+  cg32_direction_kernel<<<c->nb_red, 256, 0, c->stream>>>(c->nfe4 / 4, c->nb_red, par, iter, c->d_part + c->nb_red,
+                                                          (const float4*)c->d_z32, (float4*)c->d_p32, c->d_sc, c->opt.maxit, h);
 }
 
 // ---- continuous traces (IEDG / EDG): expansion lam = R mu and restriction R^T (face weights)
@@ -356,8 +396,8 @@ hdg_status cg32_inner(hdg_ctx* c, int* iters, double tol, int* last, bool use16)
   const int64_t n4 = c->nfe4 / 4;
   c->n_launch += 2;
   cg32_init_kernel<<<nb, 256, 0, c->stream>>>(n4, (const float4*)c->d_b32, (const float4*)c->d_dinv32, (float4*)c->d_x32,
-                                              (float4*)c->d_r32, (float4*)c->d_z32, (float4*)c->d_p32, c->d_part);
-  cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, tol, c->d_sc, nullptr);
+                                              (float4*)c->d_r32, (float4*)c->d_z32, (float4*)c->d_p32, c->d_twoB);
+  cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_twoB, tol, c->d_sc, c->d_two, nullptr);
   hdg_status s = check_launch(c, "cg32_init");
   if (s) return s;
   int it = 0;
@@ -365,32 +405,13 @@ hdg_status cg32_inner(hdg_ctx* c, int* iters, double tol, int* last, bool use16)
   const int chk = std::max(1, c->opt.check_every);
   c->h_sc->done = 0;
   const int first = std::max(2, std::min(chk, *last - 1));   // first poll near the last solve's count
-  while (!c->h_sc->done && it < maxit) {
+  // the two-kernel iteration tests an update at the start of the next one: one more than maxit ends it
+  const int end = use16 ? maxit : maxit + 1;
+  while (!c->h_sc->done && it < end) {
     // with statistics on, poll at check_every: a poll idles the GPU until the host enqueues the
     // next apply, and that gap would land inside the apply's event pair
-    const int upto = std::min(maxit, it + (it == 0 ? first : (c->stats_on ? chk : std::min(chk, 3))));
-    for (; it < upto; ++it) {
-      const int par = it & 1;
-      if (use16) {
-        HDG_DISPATCH(c, launch_apply16, c, c->d_p32, c->d_slot32, &c->d_sc->done, it);
-      } else {
-        HDG_DISPATCH(c, launch_apply32, c, c->d_p32, c->d_slot32, &c->d_sc->done, it);
-      }
-      if (c->phys == HDG_ELASTIC) {
-        c->n_launch += 3;
-        HDG_DISPATCH(c, launch_face_q32, c);
-        cg32_update_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, c->d_part, (const float4*)c->d_p32,
-                                                      (const float4*)c->d_q32, (const float4*)c->d_dinv32,
-                                                      (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                      c->d_part + nb, c->d_sc);
-      } else {
-        // p.q comes from the apply; the update forms q from the slots
-        c->n_launch += 2;
-        HDG_DISPATCH(c, launch_update_f32, c, par);
-      }
-      cg32_direction_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, it, c->d_part + nb, (const float4*)c->d_z32,
-                                                       (float4*)c->d_p32, c->d_sc, maxit, 0);
-    }
+    const int upto = std::min(end, it + (it == 0 ? first : (c->stats_on ? chk : std::min(chk, 3))));
+    for (; it < upto; ++it) inner32_iter(c, use16, it & 1, 0, 0, it);
     if ((s = check_launch(c, "cg32_iter"))) return s;
     CUDA_TRY(c, cudaMemcpyAsync(c->h_sc, c->d_sc, sizeof(CgScal), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -513,26 +534,7 @@ hdg_status solve_mixed_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solv
   const bool from_guess = c->guess_x && c->g_q && c->d_Sdf && c->phys == HDG_ACOUSTIC && c->R == 1;
   const int* skip = from_guess ? &c->d_lc->skip_res : nullptr;
   auto inner = [&](bool use16, cudaGraphConditionalHandle h) {
-    for (int par = 0; par < 2; ++par) {
-      if (use16) {
-        HDG_DISPATCH(c, launch_apply16, c, c->d_p32, c->d_slot32, &c->d_sc->done, -1);
-      } else {
-        HDG_DISPATCH(c, launch_apply32, c, c->d_p32, c->d_slot32, &c->d_sc->done, -1);
-      }
-      if (c->phys == HDG_ELASTIC) {
-        c->n_launch += 3;
-        HDG_DISPATCH(c, launch_face_q32, c);
-        cg32_update_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, c->d_part, (const float4*)c->d_p32,
-                                                      (const float4*)c->d_q32, (const float4*)c->d_dinv32,
-                                                      (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                      c->d_part + nb, c->d_sc);
-      } else {
-        c->n_launch += 2;
-        HDG_DISPATCH(c, launch_update_f32, c, par);
-      }
-      cg32_direction_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, -1, c->d_part + nb, (const float4*)c->d_z32,
-                                                       (float4*)c->d_p32, c->d_sc, maxit, h);
-    }
+    for (int par = 0; par < 2; ++par) inner32_iter(c, use16, par, 1, h, -1);
   };
   auto build = [&](GraphBuild& gb, cudaGraph_t G, hdg_ctx::DevGraph& dg) {
     std::vector<cudaGraphNode_t> deps, bd, d16, d32;
@@ -566,8 +568,8 @@ hdg_status solve_mixed_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solv
       to32_scaled_kernel<<<grid_for(c, nfe), 256, 0, c->stream>>>(nfe, c->d_res, c->d_rs, c->d_b32);
       cg32_init_kernel<<<nb, 256, 0, c->stream>>>(n4, (const float4*)c->d_b32, (const float4*)c->d_dinv32,
                                                   (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                  (float4*)c->d_p32, c->d_part);
-      cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, 0.5, c->d_sc, &c->d_lc->tol);
+                                                  (float4*)c->d_p32, c->d_twoB);
+      cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_twoB, 0.5, c->d_sc, c->d_two, &c->d_lc->tol);
     });
     const int64_t n2 = c->n_launch;
     if (has16) {
@@ -694,8 +696,8 @@ hdg_status edg_mixed_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solve_
       to32_scaled_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(n, c->d_res, c->d_rs, c->d_b32);
       cg32_init_kernel<<<nb, 256, 0, c->stream>>>(n4, (const float4*)c->d_b32, (const float4*)c->d_dinv32,
                                                   (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                  (float4*)c->d_p32, c->d_part);
-      cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, 0.5, c->d_sc, &c->d_lc->tol);
+                                                  (float4*)c->d_p32, c->d_twoB);
+      cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_twoB, 0.5, c->d_sc, c->d_two, &c->d_lc->tol);
     });
     const int64_t n2 = c->n_launch;
     if (has16) {
@@ -1153,13 +1155,33 @@ void mrefine_update_cols(hdg_ctx* c, int64_t n, double* lam) {
 
 // One FP32 iteration of the inner column-block PCG on the context's FP32 vectors (p32, x32,
 // r32, slots32), iteration parity par. R = 32 or 64: the persistent tensor-core apply forms
-// (p, q) and alpha in its epilogue and the update reads q from the slots (4 launches). Other R:
+// (p, q) and alpha in its epilogue and the update reads q from the slots (4 launches). R = 4, 8, 16:
+// the two-kernel iteration (Cg2MState). Other R:
 // apply, face pass with (p, q), alpha, update (6 launches). dev != 0: the beta kernel also sets
 // the device-driven loop's condition h.
+template <int DIM, int K, int CWN>
+void m_iter_two(hdg_ctx* c, int par, int maxit, int dev, cudaGraphConditionalHandle h, int iter) {
+  constexpr int EPB = 4 * (32 / CWN);   // elements per 4-warp CTA and pass
+  const int na = (int)std::max<int64_t>(1, std::min<int64_t>((c->sk.ne + EPB - 1) / EPB, (int64_t)c->sms * two_ctas(Dims<DIM, K>::M)));
+  const int nb = std::min(c->nb_red, 2 * c->sms);   // every CTA of the apply reads their partials
+  const Cg2MArgs o{mscal(c), c->d_twom, c->d_twoA, c->d_twoB, na, nb, CWN, par, maxit, dev, h};
+  c->n_launch += 2;
+  cudaEvent_t stop = apply_begin(c, 1, iter);
+  apply_multi_two_kernel<DIM, K, CWN><<<na, 128, 0, c->stream>>>(c->sk.ne, c->d_elem_face, c->d_face_bnd, c->d_S32, c->d_z32,
+                                                                c->d_p32, c->d_mslot32, o);
+  apply_end(c, stop);
+  mupdate_two_kernel<DIM, K><<<nb, 256, 0, c->stream>>>((int)c->sk.nf, (const int2*)c->d_face_slot, c->d_face_bnd,
+                                                        (const float4*)c->d_mslot32, (float4*)c->d_p32, c->d_dinv32,
+                                                        (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32, o);
+}
+
 template <int DIM, int K>
 void m_iter32(hdg_ctx* c, int par, int maxit, int dev, cudaGraphConditionalHandle h, int iter) {
   const int64_t n = c->sk.nf * c->Nf * (int64_t)c->R;
   const int nb = c->nb_red, R = c->R;
+  if (R == 4) return m_iter_two<DIM, K, 4>(c, par, maxit, dev, h, iter);
+  if (R == 8) return m_iter_two<DIM, K, 8>(c, par, maxit, dev, h, iter);
+  if (R == 16) return m_iter_two<DIM, K, 16>(c, par, maxit, dev, h, iter);
   if (R == 32 || R == 64) {
     using CP = ApplyTcPCfg<DIM, K>;
     const int64_t nq = (c->sk.ne + CP::WPB - 1) / CP::WPB;
@@ -1216,7 +1238,7 @@ hdg_status mcg(hdg_ctx* c, const TV* b, TV* x, TV* r, TV* z, TV* p, TV* q, TV* s
   }
   if (sizeof(TV) == 4)   // inner solve of a refinement sweep: per-column relaxed tolerance
     mcols_init<<<1, 256, 0, c->stream>>>(nb, c->R, rtol, x0_zero ? 1 : 0, c->d_part, mscal(c), c->d_mrr2, c->d_mbb2,
-                                         c->opt.rtol);
+                                         c->opt.rtol, c->d_twom);
   else
     mcols_init<<<1, 256, 0, c->stream>>>(nb, c->R, rtol, x0_zero ? 1 : 0, c->d_part, mscal(c));
   if ((s = check_launch(c, "mcg_init"))) return s;
@@ -1269,13 +1291,15 @@ hdg_status mcg(hdg_ctx* c, const TV* b, TV* x, TV* r, TV* z, TV* p, TV* q, TV* s
       c->graphs.push_back({key, gexec});
     }
   }
-  while (!c->h_mint[0] && it < maxit) {
+  // the two-kernel iteration tests an update at the start of the next one: one more than maxit ends it
+  const int end = sizeof(TV) == 4 && two_cols(c->R) ? maxit + 1 : maxit;
+  while (!c->h_mint[0] && it < end) {
     if (gexec) {
       const int reps = it == 0 ? std::max(1, (first + GCH - 1) / GCH) : 1;
       for (int rr = 0; rr < reps; ++rr) CUDA_TRY(c, cudaGraphLaunch(gexec, c->stream));
       it += reps * GCH;
     } else {
-      const int upto = std::min(maxit, it + (it == 0 ? first : std::min(chk, 3)));
+      const int upto = std::min(end, it + (it == 0 ? first : std::min(chk, 3)));
       issue(it, upto - it);
       it = upto;
     }
@@ -1356,7 +1380,7 @@ hdg_status msolve_graph(hdg_ctx* c, const double* b, double* x, hdg_solve_info* 
       HDG_DISPATCH(c, mlaunch_init32, c, (const float*)nullptr, (const float*)c->d_b32, (const float*)c->d_dinv32,
                    c->d_r32, c->d_z32, c->d_p32);
       mcols_init<<<1, 256, 0, c->stream>>>(nb, R, c->opt.inner_rtol, 1, c->d_part, mscal(c), c->d_mrr2, c->d_mbb2,
-                                           c->opt.rtol);
+                                           c->opt.rtol, c->d_twom);
     });
     const int64_t n2 = c->n_launch;
     cudaGraph_t BI = gb.loop(B, bd, h_in);
@@ -1890,11 +1914,9 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   CUDA_TRY(c, cudaGetDevice(&dev));
   CUDA_TRY(c, cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev));
   {
-    // reduction grid = one resident wave of the heaviest vector kernel (no partial second wave)
-    int per_sm = 4;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg32_update_kernel, 256, 0) != cudaSuccess || per_sm < 1)
-      per_sm = 4;
-    c->nb_red = std::max(1, std::min(per_sm * c->sms, (int)((c->sk.nf * c->Nf + 255) / 256)));
+    // reduction grid = one resident wave of the heaviest vector kernel (no partial second wave), three
+    // CTAs of 256 threads per SM
+    c->nb_red = std::max(1, std::min(3 * c->sms, (int)((c->sk.nf * c->Nf + 255) / 256)));
   }
   const int64_t ne = c->sk.ne, nf = c->sk.nf, nb = c->sk.nb, nc = c->nfc;
   // element vertex coordinates in sorted order (host, for quadrature points and point location)
@@ -2020,6 +2042,15 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
     if ((s = dalloc(c, &c->d_pq, 1))) return s;
     if ((s = dalloc(c, &c->d_ticket, 1))) return s;
     CUDA_TRY(c, cudaMemsetAsync(c->d_ticket, 0, sizeof(unsigned), c->stream));
+    if (c->R == 1) {
+      if ((s = dalloc(c, &c->d_two, 1))) return s;
+      if ((s = dalloc(c, &c->d_twoA, (size_t)std::max<int64_t>((ngroups + 3) / 4, (int64_t)c->sms * 16)))) return s;
+      if ((s = dalloc(c, &c->d_twoB, (size_t)2 * c->nb_red))) return s;
+    } else if (two_cols(c->R)) {
+      if ((s = dalloc(c, &c->d_twom, 1))) return s;
+      if ((s = dalloc(c, &c->d_twoA, (size_t)c->sms * 8 * c->R))) return s;
+      if ((s = dalloc(c, &c->d_twoB, (size_t)4 * c->sms * c->R))) return s;
+    }
     if ((s = dalloc(c, &c->d_dtime, 2))) return s;
     if ((s = reset_dev_timing(c))) return s;
     if (c->R == 1 && c->phys == HDG_ACOUSTIC) {

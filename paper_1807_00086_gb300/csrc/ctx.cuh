@@ -14,10 +14,15 @@
 #include "kernels.cuh"
 #include "devloop.cuh"
 #include "dflocal.cuh"
+#include "multi.cuh"
 #include "mesh.h"
 #include "reftab.h"
 
 using namespace hdg;
+
+namespace hdg {
+struct Cg2MState;   // multi.cuh
+}
 
 struct VarDeg;   // variable-degree (per-element k) data of an elastic context
 struct Svk;      // nonlinear (Saint Venant-Kirchhoff) elastodynamics data
@@ -72,6 +77,9 @@ struct hdg_ctx {
   double *d_pqpart = nullptr, *d_pq = nullptr;   // p.q block partials and result of the FP32/FP16 apply
   unsigned* d_ticket = nullptr;                   // last-block counter of that reduction
   DevTiming* d_dtime = nullptr;   // device-side launch timing: [0] FP32 apply, [1] FP16 apply
+  Cg2State* d_two = nullptr;    // two-kernel FP32 iteration: state, and the partials of its kernels
+  float2 *d_twoA = nullptr, *d_twoB = nullptr;
+  Cg2MState* d_twom = nullptr;  // the same for a narrow column block
   float *d_r32 = nullptr, *d_z32 = nullptr, *d_p32 = nullptr, *d_q32 = nullptr, *d_x32 = nullptr, *d_b32 = nullptr;
   double* d_res = nullptr;   // FP64 refinement residual
   int64_t nfe4 = 0;          // FP32 face vectors padded to a multiple of 4 entries

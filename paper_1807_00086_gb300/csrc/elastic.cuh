@@ -394,44 +394,69 @@ __global__ void __launch_bounds__(128) local_el_kernel(DevMesh mesh, Tabs T, con
 
 // ------------------------------------------------------------------ FP32 apply for large blocks
 // warp per element, full FP32 S_K [e][M][M]; lane handles rows lane + 32 q; column c of the
-// symmetric S_K is read as row c (coalesced).
+// symmetric S_K is read as row c (coalesced). Kernel A of the two-kernel iteration (Cg2State).
 template <class L>
 __global__ void __launch_bounds__(128) apply32f_kernel(int64_t ne, const int32_t* __restrict__ elem_face,
                                                        const int32_t* __restrict__ face_bnd, const float* __restrict__ S32,
-                                                       const float* __restrict__ x, float* __restrict__ slot,
-                                                       const int* __restrict__ done) {
+                                                       const float* __restrict__ z, const float* __restrict__ p,
+                                                       float* __restrict__ slot, Cg2Args o2) {
   constexpr int NF = L::NF, M = L::M, NFC = L::NFC;
   constexpr int RPL = (M + 31) / 32;
   __shared__ float lx[4][M];
-  if (done && *done) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t e = (int64_t)blockIdx.x * 4 + w;
-  if (e < ne) {
-    for (int r = lane; r < M; r += 32) {
-      const int f = elem_face[e * NFC + r / NF];
-      lx[w][r] = face_bnd[f] < 0 ? x[(int64_t)f * NF + r % NF] : 0.f;
-    }
-  }
-  __syncwarp();
-  if (e >= ne) return;
-  float acc[RPL];
-#pragma unroll
-  for (int q = 0; q < RPL; ++q) acc[q] = 0.f;
-  const float* Se = S32 + e * (int64_t)(M * M);
-#pragma unroll 4
-  for (int c = 0; c < M; ++c) {
-    const float xc = lx[w][c];
+  int64_t e = (int64_t)blockIdx.x * 4 + w;
+  float zr[RPL], pr[RPL];
+  auto gather = [&] {
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
       const int r = lane + 32 * q;
-      if (r < M) acc[q] = fmaf(__ldcs(Se + c * M + r), xc, acc[q]);
+      zr[q] = pr[q] = 0.f;
+      if (e < ne && r < M) {
+        const int f = elem_face[e * NFC + r / NF];
+        const int64_t t = (int64_t)f * NF + r % NF;
+        if (face_bnd[f] < 0) {
+          zr[q] = z[t];
+          pr[q] = p[t];
+        }
+      }
     }
-  }
+  };
+  gather();
+  float beta;
+  bool first;
+  if (!cg2_begin_a<4>(o2, beta, first)) return;   // while the gather is in flight
+  Acc2 pq;
+  while (e < ne) {
+    __syncwarp();
 #pragma unroll
-  for (int q = 0; q < RPL; ++q) {
-    const int r = lane + 32 * q;
-    if (r < M) slot[e * M + r] = acc[q];
+    for (int q = 0; q < RPL; ++q)
+      if (lane + 32 * q < M) lx[w][lane + 32 * q] = cg2_dir(first, beta, pr[q], zr[q]);
+    __syncwarp();
+    float acc[RPL];
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) acc[q] = 0.f;
+    const float* Se = S32 + e * (int64_t)(M * M);
+#pragma unroll 8
+    for (int c = 0; c < M; ++c) {
+      const float xc = lx[w][c];
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) {
+        const int r = lane + 32 * q;
+        if (r < M) acc[q] = fmaf(__ldcs(Se + c * M + r), xc, acc[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+      const int r = lane + 32 * q;
+      if (r < M) {
+        slot[e * M + r] = acc[q];
+        pq.dot(lx[w][r], acc[q]);
+      }
+    }
+    e += (int64_t)gridDim.x * 4;
+    gather();
   }
+  cg2_end_a<4>(o2, pq);
 }
 
 static __global__ void to32_copy_kernel(int64_t n, const double* __restrict__ a, float* __restrict__ b) {

@@ -345,7 +345,66 @@ struct Acc2 {
   }
   __device__ __forceinline__ void dot4(float4 a, float4 b) { dot(a.x, b.x); dot(a.y, b.y); dot(a.z, b.z); dot(a.w, b.w); }
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+  // both pairs' sum: the heads by TwoSum, as in add; symmetric in its operands
+  __device__ __forceinline__ void merge(float s2, float c2) {
+    const float t = s + s2;
+    const float bb = t - s;
+    c = (c + c2) + ((s - (t - bb)) + (s2 - bb));
+    s = t;
+  }
+  // sum over the lanes that differ in the bits lo, 2 lo, .. 16 of their index (every lane: the same)
+  __device__ __forceinline__ void warp_merge(int lo = 1) {
+    for (int o = 16; o >= lo; o >>= 1) merge(__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
+  }
 };
+
+// a / b of two compensated pairs, rounded to FP32 once (one Newton correction of the heads' quotient)
+__device__ __forceinline__ float pair_ratio(float2 a, float2 b) {
+  const float q = a.x / b.x;
+  const float r = (fmaf(-q, b.x, a.x) + a.y) - q * b.y;
+  return q + r / b.x;
+}
+
+// Sums of NQ pairs per thread over the CTA (NW warps), to every thread. On the FP32 pipe: an FP64
+// instruction holds an SM partition for about 64 cycles, so widening each thread's pairs and adding
+// doubles in the tree made the reductions the longest part of the small vector kernels.
+template <int NQ, int NW>
+__device__ __forceinline__ void block_pairs(Acc2 (&a)[NQ]) {
+  __shared__ float2 red[NQ][NW];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __syncthreads();   // an earlier sum's readers are done
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    a[q].warp_merge();
+    if (lane == 0) red[q][w] = make_float2(a[q].s, a[q].c);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    a[q] = Acc2();
+#pragma unroll
+    for (int i = 0; i < NW; ++i) a[q].merge(red[q][i].x, red[q][i].y);
+  }
+}
+// sums of the partials part[q n + i], i < n, to every thread
+template <int NQ, int NW>
+__device__ __forceinline__ void sum_pairs(const float2* __restrict__ part, int n, Acc2 (&a)[NQ]) {
+  constexpr int U = 4;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) a[q] = Acc2();
+  for (int i = threadIdx.x; i < n; i += U * 32 * NW) {
+    float2 v[NQ][U];   // all loads of a trip before its sums
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[q][u] = i + u * 32 * NW < n ? part[q * n + i + u * 32 * NW] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) a[q].merge(v[q][u].x, v[q][u].y);
+  }
+  block_pairs<NQ, NW>(a);
+}
 
 // Deterministic sum of a partials array (same order in every block); result in all threads.
 __device__ __forceinline__ double reduce_partials(const double* __restrict__ part, int n, int stride, double* red) {
@@ -357,6 +416,21 @@ __device__ __forceinline__ double reduce_partials(const double* __restrict__ par
   __syncthreads();
   return bc;
 }
+
+// Scalars of an FP32 inner solve whose iteration is two kernels: A multiplies every element block by
+// its direction p_K = z_K + beta p_K, formed in the gather, and leaves block partials of (p, S p);
+// B forms alpha from them, advances p, x, r, z and leaves partials of (r, z) and (r, r), from which
+// the next A takes beta and the convergence test. Every CTA of a kernel sums the partials it needs
+// itself, in the same order, as compensated FP32 pairs; CTA 0 alone records the state, in the slot
+// of the other iteration parity, so that no CTA reads what it writes. A small system's iteration is
+// bounded by the latency of its dependent kernels and of their sums: 16,562 triangles, k = 3: 9.2 us
+// (21.0 us as apply, update and direction with FP64 sums).
+struct Cg2State {
+  float2 rho[2];     // (r, z) of the iteration with this parity
+  float2 tol2;
+  float beta;        // of the running iteration
+  int it[2];         // updates completed before the iteration with this parity
+};
 
 // sum of the two slot contributions of each face entry (interior faces), 0 on boundary.
 __device__ __forceinline__ double face_sum(const int32_t* __restrict__ face_slot, const double* __restrict__ zslot,
@@ -666,6 +740,20 @@ __device__ __forceinline__ void timing_start(const PqOut& o) {
   if (o.timing && o.part && threadIdx.x == 0) atomicMin(&o.timing->start_ns, global_ns());
 }
 
+// A kernel that leaves its partials to the next one still counts its CTAs for the launch timing.
+__device__ __forceinline__ void timing_end(const PqOut& o) {
+  if (!o.timing || threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(o.ticket, 1u) != gridDim.x - 1) return;
+  const unsigned long long t1 = global_ns(), t0 = *(volatile unsigned long long*)&o.timing->start_ns;
+  if (t1 > t0) {
+    o.timing->ms += 1e-6 * (double)(t1 - t0);
+    o.timing->count += 1;
+  }
+  o.timing->start_ns = ~0ull;
+  *o.ticket = 0u;
+}
+
 __device__ __forceinline__ void pq_epilogue(const PqOut& o, double v) {
   __shared__ double wsum[4];
   __shared__ bool last;
@@ -701,33 +789,105 @@ __device__ __forceinline__ void pq_epilogue(const PqOut& o, double v) {
   }
 }
 
+// What kernels A and B of a two-kernel iteration share (see Cg2State)
+struct Cg2Args {
+  CgScal* sc;
+  Cg2State* st;
+  float2 *partA, *partB;   // partials of A [na], of B [2][nb]
+  int na, nb;
+  int parity, maxit, dev;
+  float sgn;
+  cudaGraphConditionalHandle h;
+};
+
+// Start of A: beta, or false when the solve is finished (recorded by CTA 0). first: p is still z.
+template <int NW>
+__device__ __forceinline__ bool cg2_begin_a(const Cg2Args& o, float& beta, bool& first) {
+  // everything is loaded before any of it is tested: at k = 0 the partials are loaded for nothing
+  const int over = o.sc->done, k = o.st->it[o.parity];
+  const float2 rho = o.st->rho[o.parity], t2 = o.st->tol2;
+  Acc2 a[2];
+  sum_pairs<2, NW>(o.partB, o.nb, a);
+  if (over) {
+    if (o.dev && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(o.h, 0u);
+    return false;
+  }
+  first = k == 0;
+  beta = 0.f;
+  float2 rz = rho;
+  int done = 0;
+  if (!first) {
+    rz = make_float2(a[0].s, a[0].c);
+    beta = pair_ratio(rz, rho);
+    done = (a[1].s - t2.x) + (a[1].c - t2.y) <= 0.f ? 1 : (k >= o.maxit ? 2 : 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) o.sc->rr = a[1].value();
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    o.st->rho[o.parity ^ 1] = rz;
+    o.st->it[o.parity ^ 1] = k + 1;
+    o.st->beta = beta;
+    o.sc->iters = k;
+    if (done) o.sc->done = done;
+    if (o.dev) cudaGraphSetConditional(o.h, done ? 0u : 1u);
+  }
+  return done == 0;
+}
+
+// End of A: this CTA's partial of (p, S p)
+template <int NW>
+__device__ __forceinline__ void cg2_end_a(const Cg2Args& o, Acc2 pq) {
+  Acc2 a[1] = {pq};
+  block_pairs<1, NW>(a);
+  if (threadIdx.x == 0) o.partA[blockIdx.x] = make_float2(a[0].s, a[0].c);
+}
+
+// direction entry of a two-kernel iteration: one multiply-add wherever it is formed, so both
+// elements of a face and the owner of the entry hold the same bits
+__device__ __forceinline__ float cg2_dir(bool first, float beta, float p, float z) { return first ? z : fmaf(beta, p, z); }
+
 // slot32 layout: [e][M] floats (element-major, like the FP64 slots); the warp transposes
 // its 32 x M products through shared memory so that the stores are contiguous float4s.
-template <int DIM, int K>
+// TWO: kernel A of a two-kernel iteration (x = z, the direction from z and p, partials left in o2);
+// else x is the direction and the epilogue completes (p, q).
+template <int DIM, int K, bool TWO>
 __global__ void __launch_bounds__(128, 4) apply32_kernel(int64_t ne, const int32_t* __restrict__ elem_face,
                                                       const int32_t* __restrict__ face_bnd,
                                                       const float* __restrict__ S32, const float* __restrict__ x,
-                                                      float* __restrict__ slot, const int* __restrict__ done, PqOut pqo) {
+                                                      const float* __restrict__ p, float* __restrict__ slot,
+                                                      const int* __restrict__ done, PqOut pqo, Cg2Args o2) {
   using D = Dims<DIM, K>;
   using PK = Packed<DIM, K>;
   constexpr int NF = D::NF, M = D::M, NFC = D::NFC, P4 = PK::P4;
   constexpr int MP = M + 1;   // padded row: conflict-free transposed writes
   __shared__ float tr[4][32 * MP];
-  if (done && *done) return;
+  if constexpr (!TWO) {
+    if (done && *done) return;
+  }
   timing_start(pqo);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t g0 = (int64_t)blockIdx.x * 4 + wid;
   const bool wact = g0 * 32 < ne;                 // the last block may hold idle warps
   const int64_t g = wact ? g0 : 0;
   const int64_t e = g0 * 32 + lane;
-  float xl[M], y[M];
+  float xl[M], y[M];   // TWO: y holds p until the direction is formed
 #pragma unroll
   for (int f = 0; f < NFC; ++f) {
     int fid = -1;
     if (e < ne) fid = elem_face[e * NFC + f];
     const bool use = fid >= 0 && face_bnd[fid] < 0;
 #pragma unroll
-    for (int mm = 0; mm < NF; ++mm) xl[f * NF + mm] = use ? x[(int64_t)fid * NF + mm] : 0.f;
+    for (int mm = 0; mm < NF; ++mm) {
+      const int64_t t = (int64_t)fid * NF + mm;
+      xl[f * NF + mm] = use ? x[t] : 0.f;
+      if constexpr (TWO) y[f * NF + mm] = use ? p[t] : 0.f;
+    }
+  }
+  if constexpr (TWO) {
+    float beta;
+    bool first;
+    if (!cg2_begin_a<4>(o2, beta, first)) return;   // while the gather is in flight
+#pragma unroll
+    for (int r = 0; r < M; ++r) xl[r] = cg2_dir(first, beta, y[r], xl[r]);
   }
 #pragma unroll
   for (int r = 0; r < M; ++r) y[r] = 0.f;
@@ -753,10 +913,13 @@ __global__ void __launch_bounds__(128, 4) apply32_kernel(int64_t ne, const int32
     float* dst = slot + g * 32 * (int64_t)M;
     for (int idx = lane; idx < nvalid * M; idx += 32) dst[idx] = t[(idx / M) * MP + idx % M];
   }
-  if (pqo.part) {
-    Acc2 a;
+  Acc2 a;
 #pragma unroll
-    for (int r = 0; r < M; ++r) a.dot(xl[r], y[r]);
+  for (int r = 0; r < M; ++r) a.dot(xl[r], y[r]);
+  if constexpr (TWO) {
+    cg2_end_a<4>(o2, a);
+    timing_end(pqo);
+  } else if (pqo.part) {
     pq_epilogue(pqo, a.value());
   }
 }
@@ -896,38 +1059,6 @@ __global__ void __launch_bounds__(128, 4) apply16_kernel(int64_t ne, const int32
   if (pqo.part) pq_epilogue(pqo, a.value());
 }
 
-// q = sgn K32 p on faces; partial p.q in FP64. NF is compile-time (no integer division).
-template <class LD>
-__global__ void __launch_bounds__(256) cg32_face_q_kernel(int nf, float sgn, const int32_t* __restrict__ face_slot,
-                                                          const int32_t* __restrict__ face_bnd,
-                                                          const float* __restrict__ slot, const float* __restrict__ p,
-                                                          float* __restrict__ q, double* __restrict__ part,
-                                                          const CgScal* __restrict__ sc) {
-  constexpr int NF = LD::NF;
-  if (sc->done) return;
-  __shared__ double red[8];
-  Acc2 pq;
-  for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
-    float qv[NF];
-    if (face_bnd[f] < 0) {
-      const float* s0 = slot + (int64_t)face_slot[2 * f] * NF;
-      const float* s1 = slot + (int64_t)face_slot[2 * f + 1] * NF;
-#pragma unroll
-      for (int mm = 0; mm < NF; ++mm) qv[mm] = sgn * (s0[mm] + s1[mm]);
-    } else {
-#pragma unroll
-      for (int mm = 0; mm < NF; ++mm) qv[mm] = 0.f;
-    }
-#pragma unroll
-    for (int mm = 0; mm < NF; ++mm) {
-      q[(int64_t)f * NF + mm] = qv[mm];
-      pq.dot(p[(int64_t)f * NF + mm], qv[mm]);
-    }
-  }
-  const double s = block_sum256(pq.value(), red);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
 // FP32 vectors are padded to a multiple of 4 entries (padding: zero, dinv = 0) and
 // processed as float4.
 __device__ __forceinline__ float4 f4fma(float a, float4 x, float4 y) {
@@ -939,72 +1070,34 @@ __device__ __forceinline__ float4 f4mul(float4 a, float4 b) { return make_float4
 // inner solve start from x = 0: r = b, z = Dinv r, p = z; partials (rz, rr)
 static __global__ void cg32_init_kernel(int64_t n4, const float4* __restrict__ b, const float4* __restrict__ dinv,
                                  float4* __restrict__ x, float4* __restrict__ r, float4* __restrict__ z,
-                                 float4* __restrict__ p, double* __restrict__ part) {
-  __shared__ double red[8];
-  Acc2 rz, rr;
+                                 float4* __restrict__ p, float2* __restrict__ part) {
+  Acc2 a[2];   // (r, z), (r, r)
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
     const float4 rv = b[t];
     const float4 zv = f4mul(dinv[t], rv);
     x[t] = make_float4(0.f, 0.f, 0.f, 0.f); r[t] = rv; z[t] = zv; p[t] = zv;
-    rz.dot4(rv, zv); rr.dot4(rv, rv);
+    a[0].dot4(rv, zv); a[1].dot4(rv, rv);
   }
-  double s;
-  s = block_sum256(rz.value(), red); if (threadIdx.x == 0) part[blockIdx.x * 2 + 0] = s;
-  s = block_sum256(rr.value(), red); if (threadIdx.x == 0) part[blockIdx.x * 2 + 1] = s;
+  block_pairs<2, 8>(a);
+  if (threadIdx.x < 2) part[threadIdx.x * gridDim.x + blockIdx.x] = make_float2(a[threadIdx.x].s, a[threadIdx.x].c);
 }
 
 // rtol_dev (may be null): the relative tolerance read on the device instead of rtol
-static __global__ void cg32_init_scalars(int nb, const double* __restrict__ part, double rtol, CgScal* sc,
+static __global__ void cg32_init_scalars(int nb, const float2* __restrict__ part, double rtol, CgScal* sc, Cg2State* st,
                                          const double* __restrict__ rtol_dev) {
-  __shared__ double red[8];
-  const double rz = reduce_partials(part + 0, nb, 2, red);
-  const double rr = reduce_partials(part + 1, nb, 2, red);
+  Acc2 a[2];
+  sum_pairs<2, 8>(part, nb, a);
   if (threadIdx.x == 0) {
-    const double tol = rtol_dev ? *rtol_dev : rtol;
-    sc->rho[0] = rz; sc->rho[1] = 0; sc->bb = rr; sc->rr = rr;
-    sc->tol2 = tol * tol * rr;
+    const double tol = rtol_dev ? *rtol_dev : rtol, rr = a[1].value(), t2 = tol * tol * rr;
+    sc->rho[0] = a[0].value(); sc->rho[1] = 0; sc->bb = rr; sc->rr = rr;
+    sc->tol2 = t2;
     sc->iters = 0;
     sc->done = (rr == 0.0) ? 1 : 0;
+    st->rho[0] = st->rho[1] = make_float2(a[0].s, a[0].c);
+    st->tol2 = make_float2((float)t2, (float)(t2 - (double)(float)t2));
+    st->beta = 0.f;
+    st->it[0] = st->it[1] = 0;
   }
-}
-
-static __global__ void cg32_update_kernel(int64_t n4, int nb, int parity, const double* __restrict__ part_pq,
-                                   const float4* __restrict__ p, const float4* __restrict__ q,
-                                   const float4* __restrict__ dinv, float4* __restrict__ x, float4* __restrict__ r,
-                                   float4* __restrict__ z, double* __restrict__ part, const CgScal* __restrict__ sc) {
-  if (sc->done) return;
-  __shared__ double red[8];
-  const double pq = reduce_partials(part_pq, nb, 1, red);
-  const float al = (float)(sc->rho[parity] / pq);
-  Acc2 rz, rr;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (; t + 3 * stride < n4; t += 4 * stride) {
-    float4 pv[4], qv[4], xv[4], rv[4], dv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      pv[u] = p[t + u * stride]; qv[u] = q[t + u * stride]; xv[u] = x[t + u * stride];
-      rv[u] = r[t + u * stride]; dv[u] = dinv[t + u * stride];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      x[t + u * stride] = f4fma(al, pv[u], xv[u]);
-      const float4 rn = f4fma(-al, qv[u], rv[u]);
-      const float4 zn = f4mul(dv[u], rn);
-      r[t + u * stride] = rn; z[t + u * stride] = zn;
-      rz.dot4(rn, zn); rr.dot4(rn, rn);
-    }
-  }
-  for (; t < n4; t += stride) {
-    x[t] = f4fma(al, p[t], x[t]);
-    const float4 rv1 = f4fma(-al, q[t], r[t]);
-    const float4 zv1 = f4mul(dinv[t], rv1);
-    r[t] = rv1; z[t] = zv1;
-    rz.dot4(rv1, zv1); rr.dot4(rv1, rv1);
-  }
-  double s;
-  s = block_sum256(rz.value(), red); if (threadIdx.x == 0) part[blockIdx.x * 2 + 0] = s;
-  s = block_sum256(rr.value(), red); if (threadIdx.x == 0) part[blockIdx.x * 2 + 1] = s;
 }
 
 // The update of the Krylov iteration with q = sgn K p formed from the slots (the face pass
@@ -1047,49 +1140,103 @@ __device__ __forceinline__ float4 q_entries4(int64_t t, int64_t nfe, float sgn, 
   return make_float4(q[0], q[1], q[2], q[3]);
 }
 
+// where q's four entries of a float4 come from: the two slots of an interior face, or slot positions
+// per entry (dslot[2 t], dslot[2 t + 1]; -1: boundary)
 template <class LD>
-__global__ void __launch_bounds__(256) cg32_update_f_kernel(int64_t n4, int64_t nfe, float sgn, int parity,
-                                                            const int32_t* __restrict__ face_slot,
-                                                            const int32_t* __restrict__ face_bnd,
-                                                            const float* __restrict__ slot,
-                                                            const float4* __restrict__ p,
-                                                            const float4* __restrict__ dinv, float4* __restrict__ x,
-                                                            float4* __restrict__ r, float4* __restrict__ z,
-                                                            const double* __restrict__ pq_in,
-                                                            double* __restrict__ part, const CgScal* __restrict__ sc) {
-  constexpr int U = 2;
-  if (sc->done) return;
-  __shared__ double red[8];
-  const float al = (float)(sc->rho[parity] / *pq_in);
-  const int2* face_slot2 = reinterpret_cast<const int2*>(face_slot);
-  Acc2 rz, rr;
+struct QFaces {
+  int64_t nfe;
+  const int2* face_slot2;
+  const int32_t* face_bnd;
+  __device__ __forceinline__ float4 at(int64_t t, float sgn, const float* slot) const {
+    return q_entries4<LD>(t, nfe, sgn, face_slot2, face_bnd, slot);
+  }
+};
+struct QSlots {
+  int64_t n;
+  const int32_t* dslot;
+  __device__ __forceinline__ float4 at(int64_t t, float sgn, const float* slot) const {
+    float q[4];
+    int2 d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = 4 * t + i < n ? reinterpret_cast<const int2*>(dslot)[4 * t + i] : make_int2(-1, -1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = d[i].x >= 0 ? sgn * (slot[d[i].x] + slot[d[i].y]) : 0.f;
+    return make_float4(q[0], q[1], q[2], q[3]);
+  }
+};
+
+// TWO: kernel B of a two-kernel iteration (alpha from A's partials, p advanced here); else p is the
+// direction and (p, q) complete in pq_in.
+// (The first trip's loads are issued before alpha is formed.)
+template <class Q, bool TWO>
+__global__ void __launch_bounds__(256, 3) cg32_update_f_kernel(int64_t n4, float sgn, int parity, Q qsrc,
+                                                               const float* __restrict__ slot, float4* __restrict__ p,
+                                                               const float4* __restrict__ dinv, float4* __restrict__ x,
+                                                               float4* __restrict__ r, float4* __restrict__ z,
+                                                               const double* __restrict__ pq_in,
+                                                               double* __restrict__ part, const CgScal* __restrict__ sc,
+                                                               Cg2Args o2) {
+  constexpr int U = TWO ? 1 : 2;
+  if constexpr (!TWO) {
+    if (sc->done) return;
+  }
+  float4 pv[U], xv[U], rv[U], dv[U], qv[U], zv[U];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += U * stride) {
-    float4 pv[U], xv[U], rv[U], dv[U], qv[U];
+  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  auto load = [&] {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t tu = t + u * stride;
       if (tu < n4) {
-        pv[u] = p[tu]; xv[u] = x[tu]; rv[u] = r[tu]; dv[u] = dinv[tu];
-        qv[u] = q_entries4<LD>(tu, nfe, sgn, face_slot2, face_bnd, slot);
+        pv[u] = p[tu];
+        if constexpr (TWO) zv[u] = z[tu];
+        xv[u] = x[tu]; rv[u] = r[tu]; dv[u] = dinv[tu];
+        qv[u] = qsrc.at(tu, sgn, slot);
       }
     }
+  };
+  float al, beta = 0.f;
+  bool first = true;
+  if constexpr (TWO) {
+    load();
+    const int over = sc->done, k = o2.st->it[parity];
+    const float2 rho = o2.st->rho[parity ^ 1];
+    beta = o2.st->beta;
+    Acc2 pq[1];
+    sum_pairs<1, 8>(o2.partA, o2.na, pq);
+    if (over) return;
+    al = pair_ratio(rho, make_float2(sgn * pq[0].s, sgn * pq[0].c));
+    first = k == 0;
+  } else {
+    al = (float)(sc->rho[parity] / *pq_in);
+    load();
+  }
+  Acc2 a[2];   // (r, z), (r, r)
+  while (t < n4) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t tu = t + u * stride;
       if (tu >= n4) break;
+      if constexpr (TWO) {
+        pv[u] = first ? zv[u] : f4fma(beta, pv[u], zv[u]);
+        p[tu] = pv[u];
+      }
       x[tu] = f4fma(al, pv[u], xv[u]);
       const float4 rn = f4fma(-al, qv[u], rv[u]);
       const float4 zn = f4mul(dv[u], rn);
       r[tu] = rn;
       z[tu] = zn;
-      rz.dot4(rn, zn);
-      rr.dot4(rn, rn);
+      a[0].dot4(rn, zn);
+      a[1].dot4(rn, rn);
     }
+    t += U * stride;
+    load();
   }
-  double s;
-  s = block_sum256(rz.value(), red); if (threadIdx.x == 0) part[blockIdx.x * 2 + 0] = s;
-  s = block_sum256(rr.value(), red); if (threadIdx.x == 0) part[blockIdx.x * 2 + 1] = s;
+  block_pairs<2, 8>(a);
+  if (threadIdx.x < 2) {
+    if constexpr (TWO) o2.partB[threadIdx.x * gridDim.x + blockIdx.x] = make_float2(a[threadIdx.x].s, a[threadIdx.x].c);
+    else part[blockIdx.x * 2 + threadIdx.x] = a[threadIdx.x].value();
+  }
 }
 
 // as cg_direction_kernel, FP32 vectors (float4)

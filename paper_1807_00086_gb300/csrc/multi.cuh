@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(LocalMultiCfg<DIM, K, CWW>::NT)
 
 // ------------------------------------------------------------------ trace apply, R columns
 // warp = (element, 32-column group); lane = column. S_K entries are warp-uniform loads.
-// FP32: S from the packed group layout of pack32_kernel. FP64: S from [e][M][M].
+// FP32: S from the packed group layout of pack_kernel. FP64: S from [e][M][M].
 // Warp = 32 / CWN elements x CWN columns (CWN = min(R, 32)); the FP32 S_K is read from the
 // 32-element group layout of the single-column path (consecutive elements of a warp read
 // consecutive float4s), the FP64 S_K from [e][m][m].
@@ -731,6 +731,278 @@ __global__ void __launch_bounds__(256) mdirection_kernel(int64_t n, int R, const
   for (int64_t t = blockIdx.x * 256 + threadIdx.x; t < n; t += (int64_t)gridDim.x * 256) p[t] = z[t] + be * p[t];
 }
 
+// ---- two-kernel iteration of narrow FP32 column blocks (R = 4, 8, 16), as Cg2State per column: A
+// multiplies every element block by its direction p_K = z_K + beta p_K, formed in the gather, and
+// leaves partials of (p, S p); B forms alpha, advances p, x, r, z and leaves partials of (r, z) and
+// (r, r); the next A takes beta and the convergence tests from them. Sums are compensated FP32 pairs,
+// added by every CTA of the consuming kernel in the same order; CTA 0 alone records the state.
+// Wider blocks keep one-block scalar kernels: their partials are too many to be read by every CTA.
+// Triangles, k = 2, R = 4: 9 us an iteration (32 us as apply, face pass, alpha, update, beta and
+// direction); 16,464 tets, k = 3, R = 4: 37 us (88 us).
+constexpr int kTwoR = 16;
+struct Cg2MState {
+  float2 rho[2][kTwoR], tol2[kTwoR];
+  float beta[kTwoR];
+  int conv[2][kTwoR];
+  int it[2];
+};
+struct Cg2MArgs {
+  MScal sc;
+  Cg2MState* st;
+  float2 *partA, *partB;   // [na][R], [2][nb][R]
+  int na, nb, R;
+  int parity, maxit, dev;
+  cudaGraphConditionalHandle h;
+};
+__host__ __device__ constexpr bool two_cols(int R) { return R % 4 == 0 && R <= kTwoR; }
+// CTAs of A per SM (its grid is one wave): the element block and its product stay in registers
+__host__ __device__ constexpr int two_ctas(int M) { return M <= 16 ? 8 : M <= 24 ? 6 : M <= 40 ? 4 : 3; }
+
+// Column sums of part[(q n + i) R + j], i < n, by a CTA of NW warps; thread j < R receives column j
+template <int NQ, int NW>
+__device__ __forceinline__ void sum_pairs_cols(const float2* __restrict__ part, int n, int R, Acc2 (&a)[NQ]) {
+  __shared__ float2 red[NQ][NW][kTwoR];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = threadIdx.x & (R - 1), G = 32 * NW / R;
+  constexpr int U = 4;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) a[q] = Acc2();
+  for (int i = threadIdx.x / R; i < n; i += U * G) {
+    float2 v[NQ][U];   // all loads of a trip before its sums
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        v[q][u] = i + u * G < n ? part[((int64_t)q * n + i + u * G) * R + j] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) a[q].merge(v[q][u].x, v[q][u].y);
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    a[q].warp_merge(R);
+    if (lane < R) red[q][w][lane] = make_float2(a[q].s, a[q].c);
+  }
+  __syncthreads();
+  if (threadIdx.x < R)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      a[q] = Acc2();
+#pragma unroll
+      for (int i = 0; i < NW; ++i) a[q].merge(red[q][i][threadIdx.x].x, red[q][i][threadIdx.x].y);
+    }
+}
+
+// Start of A: the columns' betas in be[R], or false when the solve is finished
+template <int NW>
+__device__ __forceinline__ bool cg2m_begin_a(const Cg2MArgs& o, float* be, bool& first) {
+  __shared__ int running;
+  // loaded before any of it is tested, as in cg2_begin_a
+  const int over = *o.sc.done, k = o.st->it[o.parity], j = threadIdx.x;
+  first = k == 0;
+  if (j == 0) running = 0;
+  Acc2 a[2];
+  sum_pairs_cols<2, NW>(o.partB, o.nb, o.R, a);
+  if (over) {
+    if (o.dev && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(o.h, 0u);
+    return false;
+  }
+  if (j < o.R) {
+    float2 rz = o.st->rho[o.parity][j];
+    int conv = o.st->conv[o.parity][j];
+    float beta = 0.f;
+    if (!first) {
+      const float2 t2 = o.st->tol2[j], rn = make_float2(a[0].s, a[0].c);
+      conv = conv || (a[1].s - t2.x) + (a[1].c - t2.y) <= 0.f;
+      if (!conv) beta = pair_ratio(rn, rz);
+      rz = rn;
+      if (blockIdx.x == 0) o.sc.rr[j] = a[1].value();
+    }
+    be[j] = beta;
+    if (!conv) running = 1;   // any column: the same value from every writer
+    if (blockIdx.x == 0) {
+      o.st->rho[o.parity ^ 1][j] = rz;
+      o.st->conv[o.parity ^ 1][j] = conv;
+      o.st->beta[j] = beta;
+      o.sc.conv[j] = conv;
+    }
+  }
+  __syncthreads();
+  const int done = running == 0 ? 1 : (k >= o.maxit ? 2 : 0);
+  if (blockIdx.x == 0 && j == 0) {
+    o.st->it[o.parity ^ 1] = k + 1;
+    *o.sc.iters = k;
+    if (done) *o.sc.done = done;
+    if (o.dev) cudaGraphSetConditional(o.h, done ? 0u : 1u);
+  }
+  return done == 0;
+}
+
+// Kernel A: the work split of apply_multi_kernel (a lane holds one column of one element), CTAs
+// stride over the elements
+template <int DIM, int K, int CWN>
+__global__ void __launch_bounds__(128, two_ctas(Dims<DIM, K>::M)) apply_multi_two_kernel(
+    int64_t ne, const int32_t* __restrict__ elem_face, const int32_t* __restrict__ face_bnd, const float* __restrict__ S32,
+    const float* __restrict__ z, const float* __restrict__ p, float* __restrict__ slot, Cg2MArgs o) {
+  using Dm = Dims<DIM, K>;
+  using PK = Packed<DIM, K>;
+  constexpr int NF = Dm::NF, M = Dm::M, NFC = Dm::NFC, P4 = PK::P4, EPW = 32 / CWN, R = CWN;
+  __shared__ float be[R];
+  __shared__ float2 red[4][R];
+  bool first;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = lane % CWN;
+  int64_t e = ((int64_t)blockIdx.x * 4 + w) * EPW + lane / CWN;
+  float xl[M], y[M];   // y holds p until the direction is formed
+  auto gather = [&] {
+#pragma unroll
+    for (int f = 0; f < NFC; ++f) {
+      const int fid = e < ne ? elem_face[e * NFC + f] : 0;
+      const bool use = e < ne && face_bnd[fid] < 0;
+#pragma unroll
+      for (int mm = 0; mm < NF; ++mm) {
+        const int64_t t = ((int64_t)fid * NF + mm) * R + j;
+        xl[f * NF + mm] = use ? z[t] : 0.f;
+        y[f * NF + mm] = use ? p[t] : 0.f;
+      }
+    }
+  };
+  gather();
+  if (!cg2m_begin_a<4>(o, be, first)) return;   // while the gather is in flight
+  const float beta = be[j];
+  Acc2 pq;
+  while (e < ne) {
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+      xl[r] = cg2_dir(first, beta, y[r], xl[r]);
+      y[r] = 0.f;
+    }
+    const float4* Sg = reinterpret_cast<const float4*>(S32) + (e >> 5) * (int64_t)P4 * 32 + (e & 31);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+#pragma unroll
+      for (int c = r; c < M; ++c) {
+        const int q = packed_index(M, r, c);
+        if ((q & 3) == 0) v = __ldg(Sg + (q >> 2) * 32);
+        const float s = (q & 3) == 0 ? v.x : (q & 3) == 1 ? v.y : (q & 3) == 2 ? v.z : v.w;
+        y[r] = fmaf(s, xl[c], y[r]);
+        if (c != r) y[c] = fmaf(s, xl[r], y[c]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+      slot[(e * M + r) * R + j] = y[r];
+      pq.dot(xl[r], y[r]);
+    }
+    e += (int64_t)gridDim.x * 4 * EPW;
+    gather();
+  }
+  __syncwarp();
+  pq.warp_merge(CWN);
+  if (lane < R) red[w][lane] = make_float2(pq.s, pq.c);
+  __syncthreads();
+  if (threadIdx.x < R) {
+    Acc2 s;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s.merge(red[i][threadIdx.x].x, red[i][threadIdx.x].y);
+    o.partA[(int64_t)blockIdx.x * R + threadIdx.x] = make_float2(s.s, s.c);
+  }
+}
+
+// Kernel B, four columns per thread: q = -K p from the two slots of each interior entry
+template <int DIM, int K>
+__global__ void __launch_bounds__(256, 3) mupdate_two_kernel(int nf, const int2* __restrict__ face_slot2,
+                                                             const int32_t* __restrict__ face_bnd,
+                                                             const float4* __restrict__ slot, float4* __restrict__ p,
+                                                             const float* __restrict__ dinv, float4* __restrict__ x,
+                                                             float4* __restrict__ r, float4* __restrict__ z, Cg2MArgs o) {
+  constexpr int NF = Dims<DIM, K>::NF, U = 1;
+  const int R = o.R, R4 = R >> 2, lg = __ffs(R4) - 1, jq = threadIdx.x & (R4 - 1);
+  __shared__ float als[kTwoR];
+  __shared__ float2 red[2][8][kTwoR];
+  const int64_t n4 = (int64_t)nf * NF * R4, S = (int64_t)gridDim.x * 256;
+  int64_t t = blockIdx.x * 256 + threadIdx.x;
+  float4 pv[U], zv[U], s0[U], s1[U], xv[U], rv[U];
+  float d[U];
+  auto load = [&] {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t tu = t + u * S;
+      s0[u] = s1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (tu < n4) {
+        const uint32_t fe = (uint32_t)(tu >> lg);
+        const uint32_t f = fe / NF;
+        const int mm = (int)(fe - f * NF);
+        const int fb = face_bnd[f];
+        const int2 fs = face_slot2[f];
+        pv[u] = p[tu]; zv[u] = z[tu]; xv[u] = x[tu]; rv[u] = r[tu]; d[u] = dinv[fe];
+        if (fb < 0) {
+          s0[u] = slot[((int64_t)fs.x * NF + mm) * R4 + jq];
+          s1[u] = slot[((int64_t)fs.y * NF + mm) * R4 + jq];
+        }
+      }
+    }
+  };
+  load();   // the first trip's, while alpha is formed
+  const int over = *o.sc.done;
+  const bool first = o.st->it[o.parity] == 0;
+  {
+    Acc2 a[1];
+    sum_pairs_cols<1, 8>(o.partA, o.na, R, a);
+    if (threadIdx.x < R) {
+      const int j = threadIdx.x;
+      als[j] = o.st->conv[o.parity ^ 1][j] || a[0].s == 0.f ? 0.f
+                                                            : pair_ratio(o.st->rho[o.parity ^ 1][j], make_float2(-a[0].s, -a[0].c));
+    }
+    __syncthreads();
+  }
+  if (over) return;
+  float al[4], be[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) { al[c] = als[4 * jq + c]; be[c] = o.st->beta[4 * jq + c]; }
+  Acc2 acc[2][4];
+  while (t < n4) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t tu = t + u * S;
+      if (tu >= n4) break;
+      const float4 pn = make_float4(cg2_dir(first, be[0], pv[u].x, zv[u].x), cg2_dir(first, be[1], pv[u].y, zv[u].y),
+                                    cg2_dir(first, be[2], pv[u].z, zv[u].z), cg2_dir(first, be[3], pv[u].w, zv[u].w));
+      const float4 qv = make_float4(-(s0[u].x + s1[u].x), -(s0[u].y + s1[u].y), -(s0[u].z + s1[u].z), -(s0[u].w + s1[u].w));
+      p[tu] = pn;
+      x[tu] = make_float4(fmaf(al[0], pn.x, xv[u].x), fmaf(al[1], pn.y, xv[u].y), fmaf(al[2], pn.z, xv[u].z),
+                          fmaf(al[3], pn.w, xv[u].w));
+      const float4 rn = make_float4(fmaf(-al[0], qv.x, rv[u].x), fmaf(-al[1], qv.y, rv[u].y), fmaf(-al[2], qv.z, rv[u].z),
+                                    fmaf(-al[3], qv.w, rv[u].w));
+      r[tu] = rn;
+      const float4 zn = make_float4(__fmul_rn(d[u], rn.x), __fmul_rn(d[u], rn.y), __fmul_rn(d[u], rn.z), __fmul_rn(d[u], rn.w));
+      z[tu] = zn;
+      acc[0][0].dot(rn.x, zn.x); acc[1][0].dot(rn.x, rn.x);
+      acc[0][1].dot(rn.y, zn.y); acc[1][1].dot(rn.y, rn.y);
+      acc[0][2].dot(rn.z, zn.z); acc[1][2].dot(rn.z, rn.z);
+      acc[0][3].dot(rn.w, zn.w); acc[1][3].dot(rn.w, rn.w);
+    }
+    t += U * S;
+    load();
+  }
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      acc[q][c].warp_merge(R4);
+      if (lane < R4) red[q][w][4 * lane + c] = make_float2(acc[q][c].s, acc[q][c].c);
+    }
+  __syncthreads();
+  if (threadIdx.x < 2 * R) {
+    const int q = threadIdx.x / R, j = threadIdx.x % R;
+    Acc2 s;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s.merge(red[q][i][j].x, red[q][i][j].y);
+    o.partB[((int64_t)q * gridDim.x + blockIdx.x) * R + j] = make_float2(s.s, s.c);
+  }
+}
+
 // ---- column-block Krylov kernels with NV columns per thread (R a multiple of NV)
 // Vectors are read NV columns at a time (float4 for the FP32 inner solve, double2 for the FP64
 // refinement residual): thread t holds entry t >> lg and columns NV (t & (R/NV - 1)) + 0..NV-1.
@@ -1267,7 +1539,8 @@ __global__ void __launch_bounds__(256) minit_kernel(int nf, int R, const int32_t
 // min(0.5, max(rtol, 0.25 outer_rtol / |r|/|b|)): the last sweep gains only what is left.
 static __global__ void mcols_init(int nb, int R, double rtol, int tol_from_rr, const double* __restrict__ part, MScal sc,
                                   const double* __restrict__ outer_rr = nullptr,
-                                  const double* __restrict__ outer_bb = nullptr, double outer_rtol = 0.0) {
+                                  const double* __restrict__ outer_bb = nullptr, double outer_rtol = 0.0,
+                                  Cg2MState* st = nullptr) {
   __shared__ int notconv;
   if (threadIdx.x == 0) notconv = 0;
   __syncthreads();
@@ -1287,6 +1560,14 @@ static __global__ void mcols_init(int nb, int R, double rtol, int tol_from_rr, c
     const int c = rr <= sc.tol2[j];
     sc.conv[j] = c;
     if (!c) atomicAdd(&notconv, 1);
+    if (st) {
+      const double t2 = sc.tol2[j];
+      st->rho[0][j] = st->rho[1][j] = make_float2((float)rz, (float)(rz - (double)(float)rz));
+      st->tol2[j] = make_float2((float)t2, (float)(t2 - (double)(float)t2));
+      st->conv[0][j] = st->conv[1][j] = c;
+      st->beta[j] = 0.f;
+      if (j == 0) st->it[0] = st->it[1] = 0;
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) {

@@ -9,6 +9,7 @@
 
 #include "ctx.cuh"
 #include "vardeg.cuh"
+#include "symapply.cuh"
 
 using namespace hdg;
 
@@ -21,13 +22,14 @@ struct VarDeg {
   std::vector<Cls> cls;
   int32_t* d_elist = nullptr;
   int64_t *d_u_off = nullptr, *d_h_off = nullptr, *d_s_off = nullptr, *d_sdiag = nullptr;
+  int64_t* d_p_off = nullptr;     // first unit of an element in the packed copies (symapply.cuh)
   int32_t *d_m_off = nullptr, *d_gidx = nullptr, *d_gint = nullptr, *d_dslot = nullptr;
   int16_t* d_pidx = nullptr;
   double* d_tab = nullptr;
   double* d_scr = nullptr;
   int64_t scr_blocks = 0;
-  int64_t m_tot = 0, s_tot = 0, h_tot = 0;
-  float* d_S32 = nullptr;
+  int64_t m_tot = 0, s_tot = 0, h_tot = 0, p_tot = 0;
+  float* d_S32 = nullptr;         // packed FP32 copy
   float* d_S32lo = nullptr;       // remainder of S_K beyond its FP32 copy (double-float residual apply)
   __half* d_S16 = nullptr;        // FP16 copy (HDG_MIXED16 inner operator) and its per-element scales
   float* d_sc16 = nullptr;
@@ -42,7 +44,7 @@ struct VarDeg {
   // one-launch local solves and the autotuned tiles
   VdClassTable table{};
   size_t local_smem = 0;
-  int tile32 = -1, tile64 = -1, tiledf = -1, tile16 = -1;   // index into kApplyTiles (-1: not tuned yet)
+  int tile64 = -1;                // index into kApplyTiles (-1: not tuned yet)
   int local_nth[2] = {0, 0};      // threads per element of the MODE 0 / MODE 1 launch (0: not tuned)
 };
 
@@ -102,41 +104,24 @@ void vd_launch_condense(hdg_ctx* c, const VarDeg::Cls& k) {
 constexpr int kApplyTiles[6][2] = {{4, 4}, {4, 8}, {4, 16}, {8, 4}, {8, 8}, {8, 16}};   // (warps, unroll)
 constexpr int kLocalThreads[3] = {64, 128, 256};
 
-template <typename TV, typename ST, int WPB, int UNR>
-void vd_apply_tile(hdg_ctx* c, const ST* S, const float* sc, const TV* x, TV* slot, const int* done) {
-  apply_vd_kernel<TV, ST, VD_MMAX, WPB, UNR><<<(unsigned)((c->sk.ne + WPB - 1) / WPB), 32 * WPB, 0, c->stream>>>(
-      c->sk.ne, c->vd->d_s_off, c->vd->d_m_off, c->vd->d_gint, S, sc, x, slot, done);
-}
-
-template <typename TV, typename ST = TV>
-void vd_apply_variant(hdg_ctx* c, int tile, const ST* S, const TV* x, TV* slot, const int* done,
-                      const float* sc = nullptr) {
-  switch (tile) {
-    case 0: vd_apply_tile<TV, ST, 4, 4>(c, S, sc, x, slot, done); break;
-    case 1: vd_apply_tile<TV, ST, 4, 8>(c, S, sc, x, slot, done); break;
-    case 2: vd_apply_tile<TV, ST, 4, 16>(c, S, sc, x, slot, done); break;
-    case 3: vd_apply_tile<TV, ST, 8, 4>(c, S, sc, x, slot, done); break;
-    case 4: vd_apply_tile<TV, ST, 8, 8>(c, S, sc, x, slot, done); break;
-    default: vd_apply_tile<TV, ST, 8, 16>(c, S, sc, x, slot, done); break;
-  }
-}
-
 template <int WPB, int UNR>
-void vd_apply_df_tile(hdg_ctx* c, const double* x, double* slot) {
-  apply_vd_df_kernel<VD_MMAX, WPB, UNR><<<(unsigned)((c->sk.ne + WPB - 1) / WPB), 32 * WPB, 0, c->stream>>>(
-      c->sk.ne, c->vd->d_s_off, c->vd->d_m_off, c->vd->d_gint, c->vd->d_S32, c->vd->d_S32lo, x, slot);
+void vd_apply_tile(hdg_ctx* c, const double* x, double* slot, const int* done) {
+  apply_vd_kernel<VD_MMAX, WPB, UNR><<<(unsigned)((c->sk.ne + WPB - 1) / WPB), 32 * WPB, 0, c->stream>>>(
+      c->sk.ne, c->vd->d_s_off, c->vd->d_m_off, c->vd->d_gint, c->d_S, x, slot, done);
 }
 
-void vd_apply_df_variant(hdg_ctx* c, int tile, const double* x, double* slot) {
+void vd_apply_variant(hdg_ctx* c, int tile, const double* x, double* slot, const int* done) {
   switch (tile) {
-    case 0: vd_apply_df_tile<4, 4>(c, x, slot); break;
-    case 1: vd_apply_df_tile<4, 8>(c, x, slot); break;
-    case 2: vd_apply_df_tile<4, 16>(c, x, slot); break;
-    case 3: vd_apply_df_tile<8, 4>(c, x, slot); break;
-    case 4: vd_apply_df_tile<8, 8>(c, x, slot); break;
-    default: vd_apply_df_tile<8, 16>(c, x, slot); break;
+    case 0: vd_apply_tile<4, 4>(c, x, slot, done); break;
+    case 1: vd_apply_tile<4, 8>(c, x, slot, done); break;
+    case 2: vd_apply_tile<4, 16>(c, x, slot, done); break;
+    case 3: vd_apply_tile<8, 4>(c, x, slot, done); break;
+    case 4: vd_apply_tile<8, 8>(c, x, slot, done); break;
+    default: vd_apply_tile<8, 16>(c, x, slot, done); break;
   }
 }
+
+SymIdxVd vd_sym(const hdg_ctx* c) { return SymIdxVd{c->vd->d_p_off, c->vd->d_s_off, c->vd->d_m_off, c->vd->d_gint}; }
 
 // Autotuner: times every candidate tile (run(t) launches candidate t) on the context's own
 // operator (the slot output is a workspace that the next use overwrites) and keeps the
@@ -223,7 +208,7 @@ void vd_local(hdg_ctx* c, int mode, const double* F, const double* hist, const d
 void vd_apply64(hdg_ctx* c, const double* x, double* slot, const int* done, int iter) {
   c->n_launch += 1;
   cudaEvent_t stop = apply_begin(c, 0, iter);
-  vd_apply_variant<double>(c, c->vd->tile64 < 0 ? 1 : c->vd->tile64, c->d_S, x, slot, done);
+  vd_apply_variant(c, c->vd->tile64 < 0 ? 1 : c->vd->tile64, x, slot, done);
   apply_end(c, stop);
 }
 
@@ -231,23 +216,30 @@ void vd_apply64(hdg_ctx* c, const double* x, double* slot, const int* done, int 
 void vd_apply_df(hdg_ctx* c, const double* x, double* slot) {
   c->n_launch += 1;
   cudaEvent_t stop = apply_begin(c, 2, -1);
-  vd_apply_df_variant(c, c->vd->tiledf < 0 ? 1 : c->vd->tiledf, x, slot);
+  sym_apply_df_kernel<<<(unsigned)((c->sk.ne + 3) / 4), 128, 0, c->stream>>>(c->sk.ne, vd_sym(c), c->vd->d_S32,
+                                                                             c->vd->d_S32lo, x, slot);
   apply_end(c, stop);
 }
 
-void vd_apply32(hdg_ctx* c, const float* x, float* slot, const int* done, int iter) {
-  c->n_launch += 1;
-  cudaEvent_t stop = apply_begin(c, 1, iter);
-  vd_apply_variant<float>(c, c->vd->tile32 < 0 ? 1 : c->vd->tile32, c->vd->d_S32, x, slot, done);
+// one iteration of the FP32 inner PCG (two kernels, see Cg2State) with the FP32 or the FP16 copy of
+// S_K; dev != 0: device-driven loop with condition h
+void vd_inner_iter(hdg_ctx* c, bool use16, int par, int dev, cudaGraphConditionalHandle h, int iter) {
+  const VarDeg* v = c->vd;
+  // the partials of A's CTAs are read by every CTA of the update, so their number is capped
+  const int na = (int)std::max<int64_t>(1, std::min<int64_t>((c->sk.ne + 3) / 4, (int64_t)c->sms * 16));
+  const Cg2Args o{c->d_sc, c->d_two, c->d_twoA, c->d_twoB, na, c->nb_red, par, c->opt.maxit, dev, (float)c->sgn, h};
+  c->n_launch += 2;
+  cudaEvent_t stop = apply_begin(c, use16 ? 3 : 1, iter);
+  if (use16)
+    sym_apply_two_kernel<<<(unsigned)na, 128, 0, c->stream>>>(c->sk.ne, vd_sym(c), v->d_S16, v->d_sc16, c->d_z32, c->d_p32,
+                                                              c->d_slot32, o);
+  else
+    sym_apply_two_kernel<<<(unsigned)na, 128, 0, c->stream>>>(c->sk.ne, vd_sym(c), v->d_S32, (const float*)nullptr, c->d_z32,
+                                                              c->d_p32, c->d_slot32, o);
   apply_end(c, stop);
-}
-
-void vd_apply16(hdg_ctx* c, const float* x, float* slot, const int* done, int iter) {
-  c->n_launch += 1;
-  cudaEvent_t stop = apply_begin(c, 3, iter);
-  vd_apply_variant<float, __half>(c, c->vd->tile16 < 0 ? 1 : c->vd->tile16, c->vd->d_S16, x, slot, done,
-                                  c->vd->d_sc16);
-  apply_end(c, stop);
+  cg32_update_f_kernel<QSlots, true><<<c->nb_red, 256, 0, c->stream>>>(
+      c->nfe4 / 4, (float)c->sgn, par, QSlots{c->ntr, v->d_dslot}, c->d_slot32, (float4*)c->d_p32, (const float4*)c->d_dinv32,
+      (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32, nullptr, nullptr, c->d_sc, o);
 }
 
 hdg_status vd_gather(hdg_ctx* c, const double* slot, double scale, double* out) {
@@ -309,30 +301,18 @@ hdg_status vd_cg32(hdg_ctx* c, double tol, int* iters, bool use16) {
   const int64_t n4 = c->nfe4 / 4;
   c->n_launch += 2;
   cg32_init_kernel<<<nb, 256, 0, c->stream>>>(n4, (const float4*)c->d_b32, (const float4*)c->d_dinv32, (float4*)c->d_x32,
-                                              (float4*)c->d_r32, (float4*)c->d_z32, (float4*)c->d_p32, c->d_part);
-  cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, tol, c->d_sc, nullptr);
+                                              (float4*)c->d_r32, (float4*)c->d_z32, (float4*)c->d_p32, c->d_twoB);
+  cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_twoB, tol, c->d_sc, c->d_two, nullptr);
   hdg_status s = check_launch(c, "vd_cg32_init");
   if (s) return s;
   int it = 0;
   const int maxit = c->opt.maxit;
   const int chk = std::max(1, c->opt.check_every);
   c->h_sc->done = 0;
-  while (!c->h_sc->done && it < maxit) {
-    const int upto = std::min(maxit, it + chk);
-    for (; it < upto; ++it) {
-      const int par = it & 1;
-      if (use16) vd_apply16(c, c->d_p32, c->d_slot32, &c->d_sc->done, it);
-      else vd_apply32(c, c->d_p32, c->d_slot32, &c->d_sc->done, it);
-      c->n_launch += 3;
-      vd_face_q_kernel<float><<<nb, 256, 0, c->stream>>>(n, (float)c->sgn, c->vd->d_dslot, c->d_slot32, c->d_p32,
-                                                         c->d_q32, c->d_part, c->d_sc);
-      cg32_update_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, c->d_part, (const float4*)c->d_p32,
-                                                    (const float4*)c->d_q32, (const float4*)c->d_dinv32,
-                                                    (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                    c->d_part + nb, c->d_sc);
-      cg32_direction_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, it, c->d_part + nb, (const float4*)c->d_z32,
-                                                       (float4*)c->d_p32, c->d_sc, maxit, 0);
-    }
+  // an update is tested at the start of the next iteration: one more than maxit ends the loop
+  while (!c->h_sc->done && it <= maxit) {
+    const int upto = std::min(maxit + 1, it + chk);
+    for (; it < upto; ++it) vd_inner_iter(c, use16, it & 1, 0, 0, it);
     if ((s = check_launch(c, "vd_cg32_iter"))) return s;
     CUDA_TRY(c, cudaMemcpyAsync(c->h_sc, c->d_sc, sizeof(CgScal), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -438,19 +418,7 @@ void vd_build_solve(hdg_ctx* c, GraphBuild& gb, cudaGraph_t G, std::vector<cudaG
   const int64_t n4 = c->nfe4 / 4;
   const bool has16 = c->vd->d_S16 != nullptr;
   auto inner = [&](bool use16, cudaGraphConditionalHandle h) {
-    for (int par = 0; par < 2; ++par) {
-      if (use16) vd_apply16(c, c->d_p32, c->d_slot32, &c->d_sc->done, -1);
-      else vd_apply32(c, c->d_p32, c->d_slot32, &c->d_sc->done, -1);
-      c->n_launch += 3;
-      vd_face_q_kernel<float><<<nb, 256, 0, c->stream>>>(n, (float)c->sgn, c->vd->d_dslot, c->d_slot32, c->d_p32,
-                                                         c->d_q32, c->d_part, c->d_sc);
-      cg32_update_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, c->d_part, (const float4*)c->d_p32,
-                                                    (const float4*)c->d_q32, (const float4*)c->d_dinv32,
-                                                    (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                    c->d_part + nb, c->d_sc);
-      cg32_direction_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, -1, c->d_part + nb, (const float4*)c->d_z32,
-                                                       (float4*)c->d_p32, c->d_sc, maxit, h);
-    }
+    for (int par = 0; par < 2; ++par) vd_inner_iter(c, use16, par, 1, h, -1);
   };
   const int64_t n0 = c->n_launch;
   gb.seq(G, deps, [&] {
@@ -473,8 +441,8 @@ void vd_build_solve(hdg_ctx* c, GraphBuild& gb, cudaGraph_t G, std::vector<cudaG
     to32_scaled_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(n, c->d_res, c->d_rs, c->d_b32);
     cg32_init_kernel<<<nb, 256, 0, c->stream>>>(n4, (const float4*)c->d_b32, (const float4*)c->d_dinv32,
                                                 (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32,
-                                                (float4*)c->d_p32, c->d_part);
-    cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, 0.5, c->d_sc, &c->d_lc->tol);
+                                                (float4*)c->d_p32, c->d_twoB);
+    cg32_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_twoB, 0.5, c->d_sc, c->d_two, &c->d_lc->tol);
   });
   const int64_t n2 = c->n_launch;
   if (has16) {
@@ -539,7 +507,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   std::vector<int64_t> t_off(nf + 1, 0);
   for (int64_t f = 0; f < nf; ++f) t_off[f + 1] = t_off[f] + dim * n_modes_h(dim - 1, fk[f]);
   c->ntr = t_off[nf];
-  std::vector<int64_t> u_off(ne + 1, 0), h_off(ne + 1, 0), s_off(ne + 1, 0);
+  std::vector<int64_t> u_off(ne + 1, 0), h_off(ne + 1, 0), s_off(ne + 1, 0), p_off(ne + 1, 0);
   std::vector<int32_t> m_off(ne + 1, 0);
   for (int64_t e = 0; e < ne; ++e) {
     const int np = n_modes_h(dim, elem_k[e]);
@@ -549,9 +517,11 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
     h_off[e + 1] = h_off[e] + (int64_t)(dim * np) * (dim * np);
     m_off[e + 1] = m_off[e] + me;
     s_off[e + 1] = s_off[e] + (int64_t)me * me;
+    p_off[e + 1] = p_off[e] + sym_units(me);
   }
   c->nfld = u_off[ne];
   v->m_tot = m_off[ne]; v->s_tot = s_off[ne]; v->h_tot = h_off[ne];
+  v->p_tot = p_off[ne];
   c->nschur = v->s_tot;
   c->nslot = v->m_tot;
   // compact local entries: faces in local order, components, active modes in the padded order
@@ -636,6 +606,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   if ((s = dalloc(c, &v->d_u_off, (size_t)ne + 1))) return s;
   if ((s = dalloc(c, &v->d_h_off, (size_t)ne + 1))) return s;
   if ((s = dalloc(c, &v->d_s_off, (size_t)ne + 1))) return s;
+  if ((s = dalloc(c, &v->d_p_off, (size_t)ne + 1))) return s;
   if ((s = dalloc(c, &v->d_m_off, (size_t)ne + 1))) return s;
   if ((s = dalloc(c, &v->d_gidx, (size_t)v->m_tot))) return s;
   if ((s = dalloc(c, &v->d_gint, (size_t)v->m_tot))) return s;
@@ -650,6 +621,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   CUDA_TRY(c, up(v->d_u_off, u_off.data(), u_off.size() * 8));
   CUDA_TRY(c, up(v->d_h_off, h_off.data(), h_off.size() * 8));
   CUDA_TRY(c, up(v->d_s_off, s_off.data(), s_off.size() * 8));
+  CUDA_TRY(c, up(v->d_p_off, p_off.data(), p_off.size() * 8));
   CUDA_TRY(c, up(v->d_m_off, m_off.data(), m_off.size() * 4));
   CUDA_TRY(c, up(v->d_gidx, gidx.data(), gidx.size() * 4));
   CUDA_TRY(c, up(v->d_gint, gint.data(), gint.size() * 4));
@@ -684,12 +656,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   CUDA_TRY(c, up(v->d_q_off, v->q_off.data(), v->q_off.size() * 8));
   // operators and workspaces
   const size_t ntr = (size_t)c->ntr, nfld = (size_t)c->nfld;
-  {
-    int per_sm = 4;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg32_update_kernel, 256, 0) != cudaSuccess || per_sm < 1)
-      per_sm = 4;
-    c->nb_red = std::max(1, std::min(per_sm * c->sms, (int)((ntr + 255) / 256)));
-  }
+  c->nb_red = std::max(1, std::min(3 * c->sms, (int)((ntr + 255) / 256)));   // one resident wave of the update
   if ((s = dalloc(c, &c->d_S, (size_t)v->s_tot))) return s;
   if ((s = dalloc(c, &c->d_Hinv, (size_t)v->h_tot))) return s;
   if ((s = dalloc(c, &c->d_dinv, ntr))) return s;
@@ -704,10 +671,10 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   for (double** p : {&c->d_u, &c->d_uprev, &c->d_h, &c->d_unew, &c->d_stage[0], &c->d_stage[1], &c->d_stage[2]})
     if ((s = dalloc(c, p, nfld))) return s;
   if (c->opt.prec != HDG_FP64) {
-    if ((s = dalloc(c, &v->d_S32, (size_t)v->s_tot))) return s;
-    if ((s = dalloc(c, &v->d_S32lo, (size_t)v->s_tot))) return s;
+    if ((s = dalloc(c, &v->d_S32, (size_t)v->p_tot * 256))) return s;
+    if ((s = dalloc(c, &v->d_S32lo, (size_t)v->p_tot * 256))) return s;
     if (c->opt.prec == HDG_MIXED16) {
-      if ((s = dalloc(c, &v->d_S16, (size_t)v->s_tot))) return s;
+      if ((s = dalloc(c, &v->d_S16, (size_t)v->p_tot * 256))) return s;
       if ((s = dalloc(c, &v->d_sc16, (size_t)ne))) return s;
     }
     if ((s = dalloc(c, &c->d_slot32, (size_t)v->m_tot))) return s;
@@ -716,6 +683,9 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
       if ((s = dalloc(c, p, (size_t)c->nfe4))) return s;
       CUDA_TRY(c, cudaMemsetAsync(*p, 0, (size_t)c->nfe4 * 4, c->stream));
     }
+    if ((s = dalloc(c, &c->d_two, 1))) return s;
+    if ((s = dalloc(c, &c->d_twoA, (size_t)c->sms * 16))) return s;
+    if ((s = dalloc(c, &c->d_twoB, (size_t)2 * c->nb_red))) return s;
     if ((s = dalloc(c, &c->d_res, ntr))) return s;
     if ((s = dalloc(c, &c->d_rs, 1))) return s;
     CUDA_TRY(c, cudaMallocHost((void**)&c->h_rs, sizeof(RefScal)));
@@ -746,31 +716,15 @@ hdg_status vd_condense(hdg_ctx* c, double alpha) {
                                                              c->d_dinv);
   if (c->opt.prec != HDG_FP64) {
     c->n_launch += 2;
-    to32_copy_kernel<<<grid_for(c, c->vd->s_tot), 256, 0, c->stream>>>(c->vd->s_tot, c->d_S, c->vd->d_S32);
-    c->n_launch += 1;
-    lo32_kernel<<<grid_for(c, c->vd->s_tot), 256, 0, c->stream>>>(c->vd->s_tot, c->d_S, c->vd->d_S32, c->vd->d_S32lo);
-    if (c->vd->d_S16) {
-      c->n_launch += 1;
-      pack16_vd_kernel<<<grid_for(c, c->sk.ne * 32), 256, 0, c->stream>>>(c->sk.ne, c->vd->d_s_off, c->d_S,
-                                                                          c->vd->d_sc16, c->vd->d_S16);
-    }
+    sym_pack_kernel<<<(unsigned)std::min<int64_t>(c->sk.ne, 1 << 20), 256, 0, c->stream>>>(
+        c->sk.ne, vd_sym(c), c->d_S, (float4*)c->vd->d_S32, (float4*)c->vd->d_S32lo, (uint4*)c->vd->d_S16, c->vd->d_sc16);
     to32_kernel<<<grid_for(c, c->ntr), 256, 0, c->stream>>>(c->ntr, c->d_dinv, c->d_dinv32);
   }
   if ((s = check_launch(c, "vd_diag"))) return s;
-  // tiles of the applies, tuned once per context on its own operator
+  // tile of the FP64 apply, tuned once per context on its own operator
   VarDeg* v = c->vd;
-  if (c->opt.prec == HDG_FP64) {
-    if (v->tile64 < 0)
-      v->tile64 = vd_tune(c, [&](int t) { vd_apply_variant<double>(c, t, c->d_S, c->d_lam, c->d_slot, nullptr); });
-  } else {
-    if (v->tile32 < 0)
-      v->tile32 = vd_tune(c, [&](int t) { vd_apply_variant<float>(c, t, v->d_S32, c->d_p32, c->d_slot32, nullptr); });
-    if (v->tiledf < 0) v->tiledf = vd_tune(c, [&](int t) { vd_apply_df_variant(c, t, c->d_lam, c->d_slot); });
-    if (v->d_S16 && v->tile16 < 0)
-      v->tile16 = vd_tune(c, [&](int t) {
-        vd_apply_variant<float, __half>(c, t, v->d_S16, c->d_p32, c->d_slot32, nullptr, v->d_sc16);
-      });
-  }
+  if (c->opt.prec == HDG_FP64 && v->tile64 < 0)
+    v->tile64 = vd_tune(c, [&](int t) { vd_apply_variant(c, t, c->d_lam, c->d_slot, nullptr); });
   if ((s = check_launch(c, "vd_tune"))) return s;
   int herr = 0;
   CUDA_TRY(c, cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -940,15 +894,14 @@ hdg_status vd_project_volume(hdg_ctx* c, const double* vals, double* u) {
 
 hdg_status vd_get_tuning(const hdg_ctx* c, hdg_tuning* o) {
   const VarDeg* v = c->vd;
-  // the FP64-accurate apply is the FP64 kernel on the plain path and the double-float kernel
-  // (residual of the refinement) on the mixed path
-  const int tr = c->opt.prec == HDG_FP64 ? v->tile64 : v->tiledf;
-  o->tuned = tr >= 0 ? 1 : 0;
-  const int t32 = v->tile32 < 0 ? 1 : v->tile32, t64 = tr < 0 ? 1 : tr;
-  o->apply32_warps = kApplyTiles[t32][0];
-  o->apply32_unroll = kApplyTiles[t32][1];
-  o->apply64_warps = kApplyTiles[t64][0];
-  o->apply64_unroll = kApplyTiles[t64][1];
+  // the packed applies of the mixed path have one shape: 4 warps, 8 entries of a column per lane
+  const bool fp64 = c->opt.prec == HDG_FP64;
+  const int t64 = v->tile64 < 0 ? 1 : v->tile64;
+  o->tuned = fp64 ? v->tile64 >= 0 : c->condensed;
+  o->apply32_warps = 4;
+  o->apply32_unroll = 8;
+  o->apply64_warps = fp64 ? kApplyTiles[t64][0] : 4;
+  o->apply64_unroll = fp64 ? kApplyTiles[t64][1] : 8;
   o->local_threads[0] = v->local_nth[0];
   o->local_threads[1] = v->local_nth[1];
   return HDG_OK;
