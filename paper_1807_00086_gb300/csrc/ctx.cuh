@@ -65,6 +65,7 @@ struct hdg_ctx {
   int tcp_per_sm = 1;           // resident CTAs per SM of the persistent tensor-core column-block apply
   // mixed precision
   float *d_S32 = nullptr, *d_dinv32 = nullptr, *d_slot32 = nullptr;
+  float* d_S32lo = nullptr;     // elastic: remainder of the packed FP32 copy (symapply.cuh); set where that is used
   float* d_Sdf = nullptr;       // double-float diagonal-major copy of S_K (refinement apply)
   df2 *d_Hinvdf = nullptr, *d_geodf = nullptr, *d_tabdf = nullptr;   // double-float local solves
   double* d_post = nullptr;       // post-processing tables K1 | E1 (PostTabs; built at the first hdg_postprocess)

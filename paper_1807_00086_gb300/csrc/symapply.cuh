@@ -10,6 +10,7 @@
 #pragma once
 
 #include "dflocal.cuh"
+#include "elastic.cuh"
 
 namespace hdg {
 
@@ -26,6 +27,23 @@ struct SymIdxVd {
   __device__ __forceinline__ int64_t unit0(int64_t e) const { return p_off[e]; }
   __device__ __forceinline__ int64_t s0(int64_t e) const { return s_off[e]; }
   __device__ __forceinline__ int64_t entry(int64_t, int64_t m0, int c) const { return gint[m0 + c]; }
+};
+
+// Uniform degree. The copies are used where their units hold fewer entries than the full block
+// (degrees 2 and 3 on tetrahedra and 4 on triangles; the padding of smaller blocks outweighs the half saved).
+__host__ __device__ constexpr bool sym_pays(int m) { return sym_units(m) * 256 < m * m; }
+template <class L>
+struct SymIdxUni {
+  static constexpr int M = L::M, NB = sym_blocks(L::M);
+  const int32_t *elem_face, *face_bnd;
+  __device__ __forceinline__ int64_t m0(int64_t e) const { return e * M; }
+  __device__ __forceinline__ int m(int64_t) const { return M; }
+  __device__ __forceinline__ int64_t unit0(int64_t e) const { return e * sym_units(M); }
+  __device__ __forceinline__ int64_t s0(int64_t e) const { return e * M * M; }
+  __device__ __forceinline__ int64_t entry(int64_t e, int64_t, int c) const {
+    const int f = elem_face[e * L::NFC + c / L::NF];
+    return face_bnd[f] < 0 ? (int64_t)f * L::NF + c % L::NF : -1;
+  }
 };
 
 // Sums of v[0..7] over the 16 lanes of a half-warp; lane l receives index l & 7
