@@ -65,16 +65,16 @@ void launch_local(hdg_ctx* c, int mode, const double* F, const double* hist, dou
   const SrcArgs sa = srcargs(c, t);
   c->n_launch += 1;
   if (c->d_Hinvdf) {
-    using LD = LocalDfCfg<DIM, K>;
+    using LD = LocalDfCfg<DIM, K, 0>;
     const unsigned gd = (unsigned)((c->sk.ne + LD::EPB - 1) / LD::EPB);
     const float th = (float)c->tau;
     const df2 tau{th, (float)(c->tau - (double)th)};
     if (mode == 0)
-      local_df_kernel<DIM, K, 0><<<gd, LD::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf, c->alpha,
-                                                               tau, F, hist, sa, lam, out);
+      local_df_kernel<DIM, K, 0, 0><<<gd, LD::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
+                                                                  tau, 1, F, hist, sa, lam, out);
     else
-      local_df_kernel<DIM, K, 1><<<gd, LD::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf, c->alpha,
-                                                               tau, F, hist, sa, lam, out);
+      local_df_kernel<DIM, K, 1, 0><<<gd, LD::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
+                                                                  tau, 1, F, hist, sa, lam, out);
     return;
   }
   using L = LocalCfg<DIM, K>;
@@ -385,7 +385,8 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
         if (c->d_S16) HDG_DISPATCH(c, prepare_apply16, c);
       }
       const int64_t nH = c->sk.ne * (int64_t)c->nv * c->nv;
-      c->n_launch += 1;
+      c->n_launch += 2;
+      local_co_kernel<<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_codf);
       to_df_kernel<<<grid_for(c, nH), 256, 0, c->stream>>>(nH, c->d_Hinv, c->d_Hinvdf);
     }
     const int64_t nfe = c->sk.nf * c->Nf;
@@ -993,16 +994,16 @@ void mlaunch_local_cw(hdg_ctx* c, int mode, const double* F, const double* hist,
 template <int DIM, int K, int CW>
 void mlaunch_local_df(hdg_ctx* c, int mode, const double* F, const double* hist, const SrcArgs& sa, const double* lam,
                       double* out) {
-  using L = LocalDfMCfg<DIM, K, CW>;
+  using L = LocalDfCfg<DIM, K, CW>;
   const dim3 grid((unsigned)((c->sk.ne + L::EPB - 1) / L::EPB), (unsigned)(c->R / CW));
   const float th = (float)c->tau;
   const df2 tau{th, (float)(c->tau - (double)th)};
   if (mode == 0)
-    local_df_multi_kernel<DIM, K, 0, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf,
-                                                                        c->alpha, tau, c->R, F, hist, sa, lam, out);
+    local_df_kernel<DIM, K, 0, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
+                                                                  tau, c->R, F, hist, sa, lam, out);
   else
-    local_df_multi_kernel<DIM, K, 1, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_Hinvdf,
-                                                                        c->alpha, tau, c->R, F, hist, sa, lam, out);
+    local_df_kernel<DIM, K, 1, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
+                                                                  tau, c->R, F, hist, sa, lam, out);
 }
 
 template <int DIM, int K>
@@ -2110,30 +2111,22 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
       if ((s = dalloc(c, &c->d_geodf, (size_t)ne * GEO_STRIDE))) return s;
       c->n_launch += 1;
       to_df_kernel<<<grid_for(c, ne * GEO_STRIDE), 256, 0, c->stream>>>(ne * GEO_STRIDE, c->d_geo, c->d_geodf);
-      const int NP = c->nv, NF = c->Nf, D = c->dim, NFC = c->dim + 1;
-      std::vector<df2> td((size_t)2 * D * NP * NP + 2 * NFC * NP * NF);
-      auto split = [](double v) { const float h = (float)v; return df2{h, (float)(v - (double)h)}; };
-      df2* DrT = td.data();
-      df2* Drd = DrT + D * NP * NP;
-      df2* FfT = Drd + D * NP * NP;
-      df2* Ffd = FfT + NFC * NP * NF;
-      for (int r = 0; r < D; ++r)
-        for (int l = 0; l < NP; ++l)
-          for (int i = 0; i < NP; ++i) {
-            DrT[(r * NP + l) * NP + i] = split(c->T.Dr[(r * NP + i) * NP + l]);
-            Drd[(r * NP + l) * NP + i] = split(c->T.Dr[(r * NP + l) * NP + i]);
-          }
-      for (int f = 0; f < NFC; ++f)
-        for (int i = 0; i < NP; ++i)
-          for (int mm = 0; mm < NF; ++mm) {
-            FfT[(f * NF + mm) * NP + i] = split(c->T.Ff[(f * NP + i) * NF + mm]);
-            Ffd[(f * NP + i) * NF + mm] = split(c->T.Ff[(f * NP + i) * NF + mm]);
-          }
-      if ((s = dalloc(c, &c->d_tabdf, td.size()))) return s;
-      CUDA_TRY(c, cudaMemcpyAsync(c->d_tabdf, td.data(), td.size() * sizeof(df2), cudaMemcpyHostToDevice, c->stream));
-      // the host copy is released below only after the stream has consumed it
+      if ((s = dalloc(c, &c->d_codf, (size_t)ne * 4))) return s;
+      const SparseRows sp = sparse_rows(c->T);
+      std::vector<SpDf> ent(sp.val.size());
+      for (size_t q = 0; q < ent.size(); ++q) {
+        const float h = (float)sp.val[q];
+        ent[q] = SpDf{h, (float)(sp.val[q] - (double)h), sp.idx[q], 0};
+      }
+      std::vector<int32_t> ip(sp.ptr);
+      ip.insert(ip.end(), sp.perm.begin(), sp.perm.end());
+      if ((s = dalloc(c, &c->d_tabdf, ent.size()))) return s;
+      if ((s = dalloc(c, &c->d_tabptr, ip.size()))) return s;
+      CUDA_TRY(c, cudaMemcpyAsync(c->d_tabdf, ent.data(), ent.size() * sizeof(SpDf), cudaMemcpyHostToDevice, c->stream));
+      CUDA_TRY(c, cudaMemcpyAsync(c->d_tabptr, ip.data(), ip.size() * 4, cudaMemcpyHostToDevice, c->stream));
+      // the host copies are released below only after the stream has consumed them
       CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-      c->tabsdf = TabsDf{c->d_tabdf, c->d_tabdf + (Drd - DrT), c->d_tabdf + (FfT - DrT), c->d_tabdf + (Ffd - DrT)};
+      c->tabsdf = TabsDf{c->d_tabdf, c->d_tabptr, c->d_tabptr + sp.ptr.size()};
     }
     if ((s = dalloc(c, &c->d_res, nfe * R))) return s;
     if ((s = dalloc(c, &c->d_rs, 1))) return s;

@@ -67,7 +67,10 @@ struct hdg_ctx {
   float *d_S32 = nullptr, *d_dinv32 = nullptr, *d_slot32 = nullptr;
   float* d_S32lo = nullptr;     // elastic: remainder of the packed FP32 copy (symapply.cuh); set where that is used
   float* d_Sdf = nullptr;       // double-float diagonal-major copy of S_K (refinement apply)
-  df2 *d_Hinvdf = nullptr, *d_geodf = nullptr, *d_tabdf = nullptr;   // double-float local solves
+  // double-float local solves: H^{-1}, geometry, coefficients at the mass shift, reference tables
+  df2 *d_Hinvdf = nullptr, *d_geodf = nullptr, *d_codf = nullptr;
+  SpDf* d_tabdf = nullptr;
+  int32_t* d_tabptr = nullptr;
   double* d_post = nullptr;       // post-processing tables K1 | E1 (PostTabs; built at the first hdg_postprocess)
   int64_t post_k1 = 0;            // entries of K1
   TabsDf tabsdf{};

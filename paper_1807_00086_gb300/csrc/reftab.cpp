@@ -3,6 +3,7 @@
 // lexicographically in (i, j[, l]). These realise the discrete spaces of Sec. 2.2.
 #include "reftab.h"
 
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <stdexcept>
@@ -159,6 +160,37 @@ std::vector<int> face_mode_degrees(int dim, int kf) {
       for (int j = 0; i + j <= kf; ++j) d.push_back(i + j);
   }
   return d;
+}
+
+SparseRows sparse_rows(const RefTables& T) {
+  const int dim = T.dim, Np = T.Np, Nf = T.Nf;
+  SparseRows S;
+  S.ptr.push_back(0);
+  auto put = [&](double v, int idx) {
+    if (std::fabs(v) < 1e-11) return;
+    S.val.push_back(v);
+    S.idx.push_back(idx);
+  };
+  auto end = [&] { S.ptr.push_back((int32_t)S.val.size()); };
+  for (int i = 0; i < Np; ++i, end())
+    for (int rl = 0; rl < dim * Np; ++rl) put(T.Dr[((size_t)(rl / Np) * Np + i) * Np + rl % Np], rl);
+  for (int r = 0; r < dim; ++r)
+    for (int i = 0; i < Np; ++i, end())
+      for (int l = 0; l < Np; ++l) put(T.Dr[((size_t)r * Np + l) * Np + i], l);
+  for (int fi = 0; fi < (dim + 1) * Np; ++fi, end())
+    for (int m = 0; m < Nf; ++m) put(T.Ff[(size_t)fi * Nf + m], m);
+  for (int f = 0; f <= dim; ++f)
+    for (int m = 0; m < Nf; ++m, end())
+      for (int q = 0; q < Np; ++q) put(T.Ff[((size_t)f * Np + q) * Nf + m], q);
+  std::vector<int> la(Np), lb(Np, 0);
+  for (int i = 0; i < Np; ++i) {
+    la[i] = S.ptr[i + 1] - S.ptr[i];
+    for (int r = 0; r < dim; ++r) lb[i] += S.ptr[Np + r * Np + i + 1] - S.ptr[Np + r * Np + i];
+    S.perm.push_back(i);
+  }
+  std::stable_sort(S.perm.begin(), S.perm.end(),
+                   [&](int a, int b) { return la[a] != la[b] ? la[a] > la[b] : lb[a] < lb[b]; });
+  return S;
 }
 
 RefTables build_tables(int dim, int k) { return build_tables_pair(dim, k, k); }
