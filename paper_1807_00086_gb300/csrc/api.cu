@@ -40,6 +40,8 @@ void launch_condense(hdg_ctx* c) {
     condense_el_kernel<DIM, K><<<(unsigned)c->sk.ne, 256, smem, c->stream>>>(devmesh(c), c->tabs, c->d_lame, c->d_mue,
                                                                             c->alpha, c->d_S, c->d_Hinv, c->d_err);
     diag_kernel<ElDims<DIM, K>><<<grid_for(c, c->sk.nf * c->Nf), 256, 0, c->stream>>>(devmesh(c), c->d_S, c->sgn, c->d_dinv);
+    c->n_launch += 1;
+    local_el_co_kernel<<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), DIM, c->d_lame, c->d_mue, c->alpha, c->d_elco);
     return;
   }
   using C = CondCfg<DIM, K>;
@@ -53,13 +55,15 @@ void launch_condense(hdg_ctx* c) {
 template <int DIM, int K>
 void launch_local(hdg_ctx* c, int mode, const double* F, const double* hist, double t, const double* lam, double* out) {
   if (c->phys == HDG_ELASTIC) {
+    constexpr int NTH = LocalElCfg<DIM, K>::NTH;
+    const double ia = 1.0 / c->alpha;
     c->n_launch += 1;
     if (mode == 0)
-      local_el_kernel<DIM, K, 0><<<(unsigned)c->sk.ne, 128, 0, c->stream>>>(devmesh(c), c->tabs, c->d_lame, c->d_mue,
-                                                                            c->d_Hinv, c->alpha, F, hist, lam, out);
+      local_el_kernel<DIM, K, 0><<<(unsigned)c->sk.ne, NTH, 0, c->stream>>>(devmesh(c), c->tabssp, c->d_elco, c->d_Hinv, ia,
+                                                                            F, hist, lam, out);
     else
-      local_el_kernel<DIM, K, 1><<<(unsigned)c->sk.ne, 128, 0, c->stream>>>(devmesh(c), c->tabs, c->d_lame, c->d_mue,
-                                                                            c->d_Hinv, c->alpha, F, hist, lam, out);
+      local_el_kernel<DIM, K, 1><<<(unsigned)c->sk.ne, NTH, 0, c->stream>>>(devmesh(c), c->tabssp, c->d_elco, c->d_Hinv, ia,
+                                                                            F, hist, lam, out);
     return;
   }
   const SrcArgs sa = srcargs(c, t);
@@ -1973,6 +1977,7 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   } else {
     if ((s = dalloc(c, &c->d_lame, (size_t)ne))) return s;
     if ((s = dalloc(c, &c->d_mue, (size_t)ne))) return s;
+    if (!svk && (s = dalloc(c, &c->d_elco, (size_t)ne * EL_CO))) return s;
     CUDA_TRY(c, cudaMemcpyAsync(c->d_lame, mat->lam, ne * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(c->d_mue, mat->mu, ne * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(c->d_c, mat->rho, ne * 8, cudaMemcpyHostToDevice, c->stream));   // sound-speed slot unused
@@ -2022,6 +2027,7 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   if ((s = dalloc(c, &c->d_qv_phi, c->T.qv_phi.size()))) return s;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_qv_w, c->T.qv_w.data(), c->T.qv_w.size() * 8, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(c->d_qv_phi, c->T.qv_phi.data(), c->T.qv_phi.size() * 8, cudaMemcpyHostToDevice, c->stream));
+  if (c->phys == HDG_ELASTIC && !svk && (s = upload_sparse(c, sparse_rows(c->T), c->tabssp))) return s;
   // condensed operators and workspaces
   const size_t nfe = (size_t)nf * c->Nf;
   const size_t R = (size_t)c->R;

@@ -14,6 +14,7 @@
 #include "kernels.cuh"
 #include "devloop.cuh"
 #include "dflocal.cuh"
+#include "ellocal.cuh"
 #include "multi.cuh"
 #include "mesh.h"
 #include "reftab.h"
@@ -69,6 +70,8 @@ struct hdg_ctx {
   float* d_Sdf = nullptr;       // double-float diagonal-major copy of S_K (refinement apply)
   // double-float local solves: H^{-1}, geometry, coefficients at the mass shift, reference tables
   df2 *d_Hinvdf = nullptr, *d_geodf = nullptr, *d_codf = nullptr;
+  TabsSp tabssp{};                     // nonzero rows of the reference tables
+  double* d_elco = nullptr;            // elastic: element coefficients at the mass shift
   SpDf* d_tabdf = nullptr;
   int32_t* d_tabptr = nullptr;
   double* d_post = nullptr;       // post-processing tables K1 | E1 (PostTabs; built at the first hdg_postprocess)
@@ -202,6 +205,25 @@ hdg_status dalloc(hdg_ctx* c, T** p, size_t count) {
   }
   c->allocs.push_back(*p);
   c->bytes += (int64_t)(count * sizeof(T));
+  return HDG_OK;
+}
+
+// device copy of the nonzero table rows (see SparseRows)
+inline hdg_status upload_sparse(hdg_ctx* c, const SparseRows& sp, TabsSp& T) {
+  std::vector<SpD> ent(sp.val.size());
+  for (size_t q = 0; q < ent.size(); ++q) ent[q] = SpD{sp.val[q], sp.idx[q], 0};
+  std::vector<int32_t> ip(sp.ptr);
+  ip.insert(ip.end(), sp.perm.begin(), sp.perm.end());
+  ip.insert(ip.end(), sp.permb.begin(), sp.permb.end());
+  SpD* d = nullptr;
+  int32_t* p = nullptr;
+  hdg_status s;
+  if ((s = dalloc(c, &d, ent.size()))) return s;
+  if ((s = dalloc(c, &p, ip.size()))) return s;
+  CUDA_TRY(c, cudaMemcpyAsync(d, ent.data(), ent.size() * sizeof(SpD), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(p, ip.data(), ip.size() * 4, cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));   // the host copies are released here
+  T = TabsSp{d, p, p + sp.ptr.size(), p + sp.ptr.size() + sp.perm.size()};
   return HDG_OK;
 }
 

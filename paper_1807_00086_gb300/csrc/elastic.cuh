@@ -235,163 +235,6 @@ __global__ void __launch_bounds__(256) condense_el_kernel(DevMesh mesh, Tabs T, 
   }
 }
 
-// ------------------------------------------------------------------ element-local solves
-// MODE 0: out = C_K A_K^{-1} (F_K - B_K lamD_K) [ne][M];  MODE 1: out = A_K^{-1} (F_K - B_K lam_K) [ne][N].
-// F_K = F[e] or alpha Mw_K hist[e] (no sources in the elastic path).
-template <int DIM, int K, int MODE>
-__global__ void __launch_bounds__(128) local_el_kernel(DevMesh mesh, Tabs T, const double* __restrict__ lamv,
-                                                        const double* __restrict__ muv, const double* __restrict__ Hinv,
-                                                        double alpha, const double* __restrict__ F,
-                                                        const double* __restrict__ hist, const double* __restrict__ lamt,
-                                                        double* __restrict__ out) {
-  using D = ElDims<DIM, K>;
-  constexpr int NP = D::NP, NFP = D::NFP, NF = D::NF, NFC = D::NFC, NT = D::NT, NV = D::NV, M = D::M, N = D::N;
-  constexpr int NTH = 128;
-  __shared__ double g[GEO_STRIDE];
-  __shared__ double ll[M];
-  __shared__ int fuse[NFC];
-  __shared__ double Fl[NFC * DIM * NP];
-  __shared__ double rv[NV], rs[NT * NP], y[NT * NP], tt[DIM * DIM * NP], rhs[NV], v[NV], z[DIM * DIM * NP];
-  __shared__ double w[NT * NP], sg[NT * NP];
-  __shared__ double Cm[NT * NT], Qm[NT * NT];
-  const int64_t e = blockIdx.x;
-  const int tid = threadIdx.x;
-  const double rho = mesh.rho[e], lam = lamv[e], mu = muv[e];
-  const double s = 2.0 * sqrt(rho * mu);
-  if (tid < GEO_STRIDE) g[tid] = mesh.geo[e * GEO_STRIDE + tid];
-  if (tid < NFC) {
-    int use = 0;
-    if (lamt) {
-      const int f = mesh.elem_face[e * NFC + tid];
-      use = (MODE == 1) || (mesh.face_bnd[f] >= 0);
-    }
-    fuse[tid] = use;
-  }
-  for (int t = tid; t < NT * NT; t += NTH) {
-    Cm[t] = cm_entry<DIM>(t / NT, t % NT, lam, mu);
-    Qm[t] = q_entry<DIM>(t / NT, t % NT, lam, mu);
-  }
-  __syncthreads();
-  for (int t = tid; t < M; t += NTH) {
-    const int f = mesh.elem_face[e * NFC + t / NF];
-    ll[t] = fuse[t / NF] ? lamt[(int64_t)f * NF + t % NF] : 0.0;
-  }
-  __syncthreads();
-  const double dJ = g[0];
-  for (int t = tid; t < NFC * DIM * NP; t += NTH) {
-    const int f = t / (DIM * NP), p = (t / NP) % DIM, l = t % NP;
-    double acc = 0.0;
-    if (fuse[f])
-      for (int mm = 0; mm < NFP; ++mm) acc += T.Ff[(f * NP + l) * NFP + mm] * ll[f * NF + p * NFP + mm];
-    Fl[t] = acc;
-  }
-  __syncthreads();
-  // right-hand sides r_v, r_sigma
-  for (int t = tid; t < N; t += NTH) {
-    const int comp = t / NP, l = t % NP;
-    if (comp < DIM) {
-      double val = hist ? alpha * rho * dJ * hist[e * N + t] : F[e * N + t];
-      double bl = 0.0;
-      for (int f = 0; f < NFC; ++f) bl += g[D::OJF + f] * Fl[(f * DIM + comp) * NP + l];
-      rv[t] = val + s * bl;
-    } else {
-      const int a = comp - DIM;
-      double val;
-      if (hist) {
-        val = 0.0;
-        for (int b = 0; b < NT; ++b) val += Qm[a * NT + b] * hist[e * N + (DIM + b) * NP + l];
-        val *= alpha * dJ;
-      } else {
-        val = F[e * N + t];
-      }
-      int ai, aj;
-      sym_ij<DIM>(a, ai, aj);
-      double bl = 0.0;
-      for (int f = 0; f < NFC; ++f) {
-        bl += g[D::ON + f * DIM + aj] * g[D::OJF + f] * Fl[(f * DIM + ai) * NP + l];
-        if (ai != aj) bl += g[D::ON + f * DIM + ai] * g[D::OJF + f] * Fl[(f * DIM + aj) * NP + l];
-      }
-      rs[a * NP + l] = val + bl;
-    }
-  }
-  __syncthreads();
-  for (int t = tid; t < NT * NP; t += NTH) {
-    const int a = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int b = 0; b < NT; ++b) acc += Cm[a * NT + b] * rs[b * NP + l];
-    y[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < DIM * DIM * NP; t += NTH) {
-    const int i = t / (DIM * NP), r = (t / NP) % DIM, l = t % NP;
-    double acc = 0.0;
-    for (int a = 0; a < NT; ++a) {
-      const int q = qa<DIM>(a, i);
-      if (q >= 0) acc += g[1 + r * DIM + q] * y[a * NP + l];
-    }
-    tt[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < NV; t += NTH) {
-    const int i = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int r = 0; r < DIM; ++r)
-      for (int m = 0; m < NP; ++m) acc += T.Dr[(r * NP + l) * NP + m] * tt[(i * DIM + r) * NP + m];
-    rhs[t] = rv[t] + acc / alpha;
-  }
-  __syncthreads();
-  const double* He = Hinv + e * (int64_t)(NV * NV);
-  for (int t = tid; t < NV; t += NTH) {
-    double acc = 0.0;
-    for (int l = 0; l < NV; ++l) acc += He[l * NV + t] * rhs[l];   // H^{-1} symmetric: column read
-    v[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < DIM * DIM * NP; t += NTH) {
-    const int r = t / (DIM * NP), p = (t / NP) % DIM, l = t % NP;
-    double acc = 0.0;
-    for (int m = 0; m < NP; ++m) acc += T.Dr[(r * NP + m) * NP + l] * v[p * NP + m];
-    z[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < NT * NP; t += NTH) {
-    const int b = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int p = 0; p < DIM; ++p) {
-      const int q = qa<DIM>(b, p);
-      if (q < 0) continue;
-      for (int r = 0; r < DIM; ++r) acc += g[1 + r * DIM + q] * z[(r * DIM + p) * NP + l];
-    }
-    w[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < NT * NP; t += NTH) {
-    const int a = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int b = 0; b < NT; ++b) acc += Cm[a * NT + b] * w[b * NP + l];
-    sg[t] = y[t] / (alpha * dJ) - acc / alpha;
-  }
-  __syncthreads();
-  if (MODE == 1) {
-    for (int t = tid; t < N; t += NTH) out[e * N + t] = t < NV ? v[t] : sg[t - NV];
-    return;
-  }
-  // g[f][i][mm] = J_f sum_l F^_f[l][mm] (-s v_i[l] + sum_j n_fj sigma_ij[l]); Fl reused for the weights
-  for (int t = tid; t < NFC * DIM * NP; t += NTH) {
-    const int f = t / (DIM * NP), i = (t / NP) % DIM, l = t % NP;
-    double acc = -s * v[i * NP + l];
-    for (int j = 0; j < DIM; ++j) acc += g[D::ON + f * DIM + j] * sg[sym_index<DIM>(i, j) * NP + l];
-    Fl[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < M; t += NTH) {
-    const int f = t / NF, i = (t % NF) / NFP, mm = t % NFP;
-    double acc = 0.0;
-    for (int l = 0; l < NP; ++l) acc += T.Ff[(f * NP + l) * NFP + mm] * Fl[(f * DIM + i) * NP + l];
-    out[e * M + t] = g[D::OJF + f] * acc;
-  }
-}
-
 // ------------------------------------------------------------------ FP32 apply for large blocks
 // warp per element, full FP32 S_K [e][M][M]; lane handles rows lane + 32 q; column c of the
 // symmetric S_K is read as row c (coalesced). Kernel A of the two-kernel iteration (Cg2State).

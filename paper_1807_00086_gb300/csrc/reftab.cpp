@@ -190,6 +190,9 @@ SparseRows sparse_rows(const RefTables& T) {
   }
   std::stable_sort(S.perm.begin(), S.perm.end(),
                    [&](int a, int b) { return la[a] != la[b] ? la[a] > la[b] : lb[a] < lb[b]; });
+  for (int rl = 0; rl < dim * Np; ++rl) S.permb.push_back(rl);
+  auto len = [&](int rl) { return S.ptr[Np + rl + 1] - S.ptr[Np + rl]; };
+  std::stable_sort(S.permb.begin(), S.permb.end(), [&](int a, int b) { return len(a) > len(b); });
   return S;
 }
 

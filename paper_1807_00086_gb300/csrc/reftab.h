@@ -39,9 +39,9 @@ RefTables build_tables(int dim, int k);
 //   B [dim][Np]     idx l,        Dr[r][l][i]
 //   C [dim+1][Np]   idx m,        Ff[f][i][m]
 //   D [dim+1][Nf]   idx q,        Ff[f][q][m]
-// perm: the volume rows i by falling length of A, then rising length of B.
+// perm: the volume rows i by falling length of A, then rising length of B; permb: the rows of B by length.
 struct SparseRows {
-  std::vector<int32_t> ptr, idx, perm;
+  std::vector<int32_t> ptr, idx, perm, permb;
   std::vector<double> val;
 };
 SparseRows sparse_rows(const RefTables& T);

@@ -81,7 +81,7 @@ VdIndex vd_index(const hdg_ctx* c, const VarDeg::Cls& k) {
 
 template <int K, int KT>
 void vd_local_smem(size_t& s) {
-  s = std::max(s, sizeof(double) * (size_t)LocalVdSmem<3, K, KT>::TOTAL);
+  s = std::max(s, sizeof(double) * (size_t)LocalElSmem<3, K, KT>::TOTAL);
 }
 
 template <int K, int KT>
@@ -159,16 +159,17 @@ void vd_local_launch(hdg_ctx* c, int nth, const double* F, const double* hist, c
   const VarDeg* v = c->vd;
   const VdIndex X{v->d_elist, v->d_u_off, v->d_h_off, v->d_s_off, v->d_m_off, v->d_gidx, v->d_pidx};
   const unsigned grid = (unsigned)c->sk.ne;
+  const double ia = 1.0 / c->alpha;
   c->n_launch += 1;
   if (nth == 64)
-    local_vd_all_kernel<MODE, 64><<<grid, 64, v->local_smem, c->stream>>>(devmesh(c), v->table, c->d_lame, c->d_mue,
-                                                                          c->d_Hinv, c->alpha, X, F, hist, lam, out);
+    local_vd_all_kernel<MODE, 64><<<grid, 64, v->local_smem, c->stream>>>(devmesh(c), v->table, c->d_elco, c->d_Hinv, ia, X,
+                                                                          F, hist, lam, out);
   else if (nth == 128)
-    local_vd_all_kernel<MODE, 128><<<grid, 128, v->local_smem, c->stream>>>(devmesh(c), v->table, c->d_lame, c->d_mue,
-                                                                            c->d_Hinv, c->alpha, X, F, hist, lam, out);
+    local_vd_all_kernel<MODE, 128><<<grid, 128, v->local_smem, c->stream>>>(devmesh(c), v->table, c->d_elco, c->d_Hinv, ia, X,
+                                                                            F, hist, lam, out);
   else
-    local_vd_all_kernel<MODE, 256><<<grid, 256, v->local_smem, c->stream>>>(devmesh(c), v->table, c->d_lame, c->d_mue,
-                                                                            c->d_Hinv, c->alpha, X, F, hist, lam, out);
+    local_vd_all_kernel<MODE, 256><<<grid, 256, v->local_smem, c->stream>>>(devmesh(c), v->table, c->d_elco, c->d_Hinv, ia, X,
+                                                                            F, hist, lam, out);
 }
 
 // The element-local solves of every class in one launch. The first call of each mode times
@@ -562,6 +563,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   std::vector<int32_t> elist;
   std::vector<double> tab;
   std::vector<std::array<size_t, 6>> toff;
+  std::vector<SparseRows> sparse;
   // heaviest classes first (descending 10 K + KT): the one-launch local solves start them first
   for (auto it = groups.rbegin(); it != groups.rend(); ++it) {
     auto& g = *it;
@@ -579,6 +581,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
     const std::vector<double>* parts[6] = {&T.Dr, &T.Ff, &T.Ef, &T.Trs, &T.DFrf, &T.Pfg};
     for (int i = 0; i < 6; ++i) { o[i] = tab.size(); tab.insert(tab.end(), parts[i]->begin(), parts[i]->end()); }
     toff.push_back(o);
+    sparse.push_back(sparse_rows(T));
     v->cls.push_back(k);
   }
   hdg_status s;
@@ -592,7 +595,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
   for (size_t i = 0; i < v->cls.size(); ++i) {
     v->table.start[i] = v->cls[i].first;
     v->table.key[i] = v->cls[i].K * 10 + v->cls[i].KT;
-    v->table.tabs[i] = v->cls[i].tabs;
+    if ((s = upload_sparse(c, sparse[i], v->table.tabs[i]))) return s;
     VD_DISPATCH(v->cls[i].K, v->cls[i].KT, vd_local_smem, v->local_smem);
   }
   v->table.start[v->cls.size()] = ne;
@@ -711,6 +714,8 @@ hdg_status vd_condense(hdg_ctx* c, double alpha) {
   for (const auto& k : c->vd->cls) VD_DISPATCH(k.K, k.KT, vd_launch_condense, c, k);
   hdg_status s = check_launch(c, "vd_condense");
   if (s) return s;
+  c->n_launch += 1;
+  local_el_co_kernel<<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), 3, c->d_lame, c->d_mue, alpha, c->d_elco);
   c->n_launch += 1;
   vd_diag_kernel<<<grid_for(c, c->ntr), 256, 0, c->stream>>>(c->ntr, c->sgn, c->vd->d_dslot, c->vd->d_sdiag, c->d_S,
                                                              c->d_dinv);

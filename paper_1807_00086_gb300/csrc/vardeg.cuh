@@ -15,23 +15,9 @@
 //   pidx[...]           padded local index (class layout) of compact entry a,
 //   dslot[2 d + s]      the two slot positions summed into trace entry d (-1: boundary).
 #pragma once
-#include "elastic.cuh"
+#include "ellocal.cuh"
 
 namespace hdg {
-
-template <int DIM, int K, int KT>
-struct VdDims {
-  static constexpr int NP = Dims<DIM, K>::NP;
-  static constexpr int NFP = Dims<DIM, KT>::NF;   // scalar face modes of the padded layout
-  static constexpr int NF = DIM * NFP;
-  static constexpr int NFC = DIM + 1;
-  static constexpr int NT = DIM * (DIM + 1) / 2;
-  static constexpr int NV = DIM * NP;
-  static constexpr int N = (DIM + NT) * NP;
-  static constexpr int M = NFC * NF;
-  static constexpr int OJF = 1 + DIM * DIM;
-  static constexpr int ON = 1 + DIM * DIM + DIM + 1;
-};
 
 struct VdIndex {
   const int32_t* elist;   // elements of the class
@@ -205,173 +191,16 @@ __global__ void __launch_bounds__(256) condense_vd_kernel(DevMesh mesh, Tabs T, 
   }
 }
 
-// Shared workspace of one element of class (K, KT) in the local solves (offsets in doubles).
-template <int DIM, int K, int KT>
-struct LocalVdSmem {
-  using D = VdDims<DIM, K, KT>;
-  static constexpr int G = 0, LL = G + GEO_STRIDE, FL = LL + D::M, RV = FL + D::NFC * DIM * D::NP,
-                       RS = RV + D::NV, Y = RS + D::NT * D::NP, TT = Y + D::NT * D::NP,
-                       RHS = TT + DIM * DIM * D::NP, V = RHS + D::NV, Z = V + D::NV, W = Z + DIM * DIM * D::NP,
-                       SG = W + D::NT * D::NP, CM = SG + D::NT * D::NP, QM = CM + D::NT * D::NT,
-                       FUSE = QM + D::NT * D::NT, TOTAL = FUSE + 4;
+// fields, H^{-1} and compact trace entries of an element in the local solves
+struct ElIdxVd {
+  VdIndex X;
+  __device__ __forceinline__ int64_t u0(int64_t e) const { return X.u_off[e]; }
+  __device__ __forceinline__ int64_t h0(int64_t e) const { return X.h_off[e]; }
+  __device__ __forceinline__ int64_t m0(int64_t e) const { return X.m_off[e]; }
+  __device__ __forceinline__ int m(int64_t e) const { return X.m_off[e + 1] - X.m_off[e]; }
+  __device__ __forceinline__ int pad(int64_t m0, int a) const { return X.pidx[m0 + a]; }
+  __device__ __forceinline__ int64_t trace(int64_t, int64_t m0, int a) const { return X.gidx[m0 + a]; }
 };
-
-// Element-local solves of one element of class (K, KT), NTH threads. MODE 0:
-// out[m_off[e] + a] = (C_K A_K^{-1}(F_K - B_K lamD_K)) at the compact entries; MODE 1:
-// out[u_off[e] ..] = A_K^{-1}(F_K - B_K lam_K). F_K = F[u_off[e] ..] or alpha Mw_K hist[u_off[e] ..].
-template <int DIM, int K, int KT, int MODE, int NTH>
-__device__ __forceinline__ void local_vd_body(const DevMesh& mesh, const Tabs& T, const double* __restrict__ lamv,
-                                              const double* __restrict__ muv, const double* __restrict__ Hinv,
-                                              double alpha, const VdIndex& X, int64_t e, const double* __restrict__ F,
-                                              const double* __restrict__ hist, const double* __restrict__ lamt,
-                                              double* __restrict__ out, double* sm) {
-  using D = VdDims<DIM, K, KT>;
-  using SM = LocalVdSmem<DIM, K, KT>;
-  constexpr int NP = D::NP, NFP = D::NFP, NF = D::NF, NFC = D::NFC, NT = D::NT, NV = D::NV, M = D::M, N = D::N;
-  double* g = sm + SM::G;
-  double* ll = sm + SM::LL;
-  double* Fl = sm + SM::FL;
-  double *rv = sm + SM::RV, *rs = sm + SM::RS, *y = sm + SM::Y, *tt = sm + SM::TT, *rhs = sm + SM::RHS,
-         *v = sm + SM::V, *z = sm + SM::Z, *w = sm + SM::W, *sg = sm + SM::SG, *Cm = sm + SM::CM, *Qm = sm + SM::QM;
-  int* fuse = reinterpret_cast<int*>(sm + SM::FUSE);
-  const int tid = threadIdx.x;
-  const double rho = mesh.rho[e], lam = lamv[e], mu = muv[e];
-  const double s = 2.0 * sqrt(rho * mu);
-  const int64_t u0 = X.u_off[e];
-  const int m0 = X.m_off[e], me = X.m_off[e + 1] - m0;
-  if (tid < GEO_STRIDE) g[tid] = mesh.geo[e * GEO_STRIDE + tid];
-  if (tid < NFC) {
-    int use = 0;
-    if (lamt) {
-      const int f = mesh.elem_face[e * NFC + tid];
-      use = (MODE == 1) || (mesh.face_bnd[f] >= 0);
-    }
-    fuse[tid] = use;
-  }
-  for (int t = tid; t < NT * NT; t += NTH) {
-    Cm[t] = cm_entry<DIM>(t / NT, t % NT, lam, mu);
-    Qm[t] = q_entry<DIM>(t / NT, t % NT, lam, mu);
-  }
-  for (int t = tid; t < M; t += NTH) ll[t] = 0.0;
-  __syncthreads();
-  for (int a = tid; a < me; a += NTH) {
-    const int pc = X.pidx[m0 + a];
-    if (fuse[pc / NF]) ll[pc] = lamt[X.gidx[m0 + a]];
-  }
-  __syncthreads();
-  const double dJ = g[0];
-  for (int t = tid; t < NFC * DIM * NP; t += NTH) {
-    const int f = t / (DIM * NP), p = (t / NP) % DIM, l = t % NP;
-    double acc = 0.0;
-    if (fuse[f])
-      for (int mm = 0; mm < NFP; ++mm) acc += T.Ff[(f * NP + l) * NFP + mm] * ll[f * NF + p * NFP + mm];
-    Fl[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < N; t += NTH) {
-    const int comp = t / NP, l = t % NP;
-    if (comp < DIM) {
-      double val = hist ? alpha * rho * dJ * hist[u0 + t] : F[u0 + t];
-      double bl = 0.0;
-      for (int f = 0; f < NFC; ++f) bl += g[D::OJF + f] * Fl[(f * DIM + comp) * NP + l];
-      rv[t] = val + s * bl;
-    } else {
-      const int a = comp - DIM;
-      double val;
-      if (hist) {
-        val = 0.0;
-        for (int b = 0; b < NT; ++b) val += Qm[a * NT + b] * hist[u0 + (DIM + b) * NP + l];
-        val *= alpha * dJ;
-      } else {
-        val = F[u0 + t];
-      }
-      int ai, aj;
-      sym_ij<DIM>(a, ai, aj);
-      double bl = 0.0;
-      for (int f = 0; f < NFC; ++f) {
-        bl += g[D::ON + f * DIM + aj] * g[D::OJF + f] * Fl[(f * DIM + ai) * NP + l];
-        if (ai != aj) bl += g[D::ON + f * DIM + ai] * g[D::OJF + f] * Fl[(f * DIM + aj) * NP + l];
-      }
-      rs[a * NP + l] = val + bl;
-    }
-  }
-  __syncthreads();
-  for (int t = tid; t < NT * NP; t += NTH) {
-    const int a = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int b = 0; b < NT; ++b) acc += Cm[a * NT + b] * rs[b * NP + l];
-    y[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < DIM * DIM * NP; t += NTH) {
-    const int i = t / (DIM * NP), r = (t / NP) % DIM, l = t % NP;
-    double acc = 0.0;
-    for (int a = 0; a < NT; ++a) {
-      const int q = qa<DIM>(a, i);
-      if (q >= 0) acc += g[1 + r * DIM + q] * y[a * NP + l];
-    }
-    tt[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < NV; t += NTH) {
-    const int i = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int r = 0; r < DIM; ++r)
-      for (int m = 0; m < NP; ++m) acc += T.Dr[(r * NP + l) * NP + m] * tt[(i * DIM + r) * NP + m];
-    rhs[t] = rv[t] + acc / alpha;
-  }
-  __syncthreads();
-  const double* He = Hinv + X.h_off[e];
-  for (int t = tid; t < NV; t += NTH) {
-    double acc = 0.0;
-    for (int l = 0; l < NV; ++l) acc += He[l * NV + t] * rhs[l];
-    v[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < DIM * DIM * NP; t += NTH) {
-    const int r = t / (DIM * NP), p = (t / NP) % DIM, l = t % NP;
-    double acc = 0.0;
-    for (int m = 0; m < NP; ++m) acc += T.Dr[(r * NP + m) * NP + l] * v[p * NP + m];
-    z[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < NT * NP; t += NTH) {
-    const int b = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int p = 0; p < DIM; ++p) {
-      const int q = qa<DIM>(b, p);
-      if (q < 0) continue;
-      for (int r = 0; r < DIM; ++r) acc += g[1 + r * DIM + q] * z[(r * DIM + p) * NP + l];
-    }
-    w[t] = acc;
-  }
-  __syncthreads();
-  for (int t = tid; t < NT * NP; t += NTH) {
-    const int a = t / NP, l = t % NP;
-    double acc = 0.0;
-    for (int b = 0; b < NT; ++b) acc += Cm[a * NT + b] * w[b * NP + l];
-    sg[t] = y[t] / (alpha * dJ) - acc / alpha;
-  }
-  __syncthreads();
-  if (MODE == 1) {
-    for (int t = tid; t < N; t += NTH) out[u0 + t] = t < NV ? v[t] : sg[t - NV];
-    return;
-  }
-  for (int t = tid; t < NFC * DIM * NP; t += NTH) {
-    const int f = t / (DIM * NP), i = (t / NP) % DIM, l = t % NP;
-    double acc = -s * v[i * NP + l];
-    for (int j = 0; j < DIM; ++j) acc += g[D::ON + f * DIM + j] * sg[sym_index<DIM>(i, j) * NP + l];
-    Fl[t] = acc;
-  }
-  __syncthreads();
-  for (int a = tid; a < me; a += NTH) {
-    const int t = X.pidx[m0 + a];
-    const int f = t / NF, i = (t % NF) / NFP, mm = t % NFP;
-    double acc = 0.0;
-    for (int l = 0; l < NP; ++l) acc += T.Ff[(f * NP + l) * NFP + mm] * Fl[(f * DIM + i) * NP + l];
-    out[m0 + a] = g[D::OJF + f] * acc;
-  }
-}
 
 // All classes of a variable-degree mesh in one launch: block b handles element elist[b]; the
 // element list is grouped by class, heaviest classes first, and the class ranges are
@@ -380,13 +209,12 @@ struct VdClassTable {
   int n;
   int64_t start[11];
   int key[10];     // 10 K + KT
-  Tabs tabs[10];
+  TabsSp tabs[10];
 };
 
 template <int MODE, int NTH>
-__global__ void __launch_bounds__(NTH) local_vd_all_kernel(DevMesh mesh, VdClassTable C, const double* __restrict__ lamv,
-                                                           const double* __restrict__ muv,
-                                                           const double* __restrict__ Hinv, double alpha, VdIndex X,
+__global__ void __launch_bounds__(NTH) local_vd_all_kernel(DevMesh mesh, VdClassTable C, const double* __restrict__ coef,
+                                                           const double* __restrict__ Hinv, double ia, VdIndex X,
                                                            const double* __restrict__ F, const double* __restrict__ hist,
                                                            const double* __restrict__ lamt, double* __restrict__ out) {
   extern __shared__ double sm[];
@@ -396,7 +224,7 @@ __global__ void __launch_bounds__(NTH) local_vd_all_kernel(DevMesh mesh, VdClass
   const int64_t e = X.elist[b];
 #define HDG_VD_BODY(KK, KKT)                                                                                      \
   case KK * 10 + KKT:                                                                                             \
-    local_vd_body<3, KK, KKT, MODE, NTH>(mesh, C.tabs[c], lamv, muv, Hinv, alpha, X, e, F, hist, lamt, out, sm); \
+    local_el_body<3, KK, KKT, MODE, NTH>(mesh, C.tabs[c], coef, Hinv, ia, ElIdxVd{X}, e, F, hist, lamt, out, sm); \
     break;
   switch (C.key[c]) {
     HDG_VD_BODY(4, 4)
