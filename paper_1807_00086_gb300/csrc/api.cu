@@ -129,14 +129,39 @@ void launch_sym_pack(hdg_ctx* c) {
       c->sk.ne, sym_idx<DIM, K>(c), c->d_S, (float4*)c->d_S32, (float4*)c->d_S32lo, (uint4*)nullptr, (float*)nullptr);
 }
 
+// one FP64 iteration; dev != 0: device-driven loop with condition h. Two kernels where A's CTAs are at most
+// four per SM: each sums B's partials first, about 2000 cycles of an SM's FP64 pipe. At 41,154 tets, k = 2 (45
+// per SM), that made an apply 68 us instead of 45 us, and striding over the elements with 4 per SM 89 us: there
+// the iteration is four kernels, apply, face pass with (p, q), update, direction.
+template <class L>
+void launch_iter64_l(hdg_ctx* c, double* x, int par, int dev, cudaGraphConditionalHandle h, int iter) {
+  using C = ApplyTwoCfg<L>;
+  const int64_t na = std::max<int64_t>(1, (c->sk.ne + C::EPB - 1) / C::EPB);
+  const int nb = c->nb_red;
+  if (na > 4 * c->sms) {
+    const int64_t nfe = c->sk.nf * c->Nf;
+    launch_apply_l<L>(c, c->d_p, c->d_slot, &c->d_sc->done, iter);
+    c->n_launch += 3;
+    cg_face_q_kernel<L><<<nb, 256, 0, c->stream>>>((int)c->sk.nf, c->sgn, c->d_face_slot, c->d_face_bnd, c->d_slot, c->d_p,
+                                                   c->d_q, c->d_part, c->d_sc);
+    cg_update_kernel<<<nb, 256, 0, c->stream>>>(nfe, nb, par, c->d_part, c->d_p, c->d_q, c->d_dinv, x, c->d_r, c->d_z,
+                                                c->d_part + nb, c->d_sc);
+    cg_direction_kernel<<<nb, 256, 0, c->stream>>>(nfe, nb, par, dev ? -1 : iter, c->d_part + nb, c->d_z, c->d_p, c->d_sc,
+                                                   c->opt.maxit, h);
+    return;
+  }
+  const Cg64Args o{c->d_sc, c->d_two64, c->d_two64A, c->d_two64B, (int)na, nb, par, c->opt.maxit, dev, c->sgn, h};
+  c->n_launch += 2;
+  cudaEvent_t stop = apply_begin(c, 0, iter);
+  apply_two64_kernel<L><<<(unsigned)na, C::NT, 0, c->stream>>>(devmesh(c), c->d_S, c->d_z, c->d_p, c->d_slot, o);
+  apply_end(c, stop);
+  cg_update_two64_kernel<L><<<nb, 256, 0, c->stream>>>(c->sk.nf * c->Nf, (const int2*)c->d_face_slot, c->d_face_bnd,
+                                                       c->d_slot, c->d_p, c->d_dinv, x, c->d_r, c->d_z, o);
+}
 template <int DIM, int K>
-void launch_face_q64(hdg_ctx* c) {
-  if (c->phys == HDG_ELASTIC)
-    cg_face_q_kernel<ElDims<DIM, K>><<<c->nb_red, 256, 0, c->stream>>>((int)c->sk.nf, c->sgn, c->d_face_slot, c->d_face_bnd,
-                                                                       c->d_slot, c->d_p, c->d_q, c->d_part, c->d_sc);
-  else
-    cg_face_q_kernel<Dims<DIM, K>><<<c->nb_red, 256, 0, c->stream>>>((int)c->sk.nf, c->sgn, c->d_face_slot, c->d_face_bnd,
-                                                                     c->d_slot, c->d_p, c->d_q, c->d_part, c->d_sc);
+void launch_iter64(hdg_ctx* c, double* x, int par, int dev, cudaGraphConditionalHandle h, int iter) {
+  if (c->phys == HDG_ELASTIC) launch_iter64_l<ElDims<DIM, K>>(c, x, par, dev, h, iter);
+  else launch_iter64_l<Dims<DIM, K>>(c, x, par, dev, h, iter);
 }
 
 // zero the device-side launch timers (start stamps to the maximum, so the first CTA lowers them)
@@ -519,7 +544,7 @@ hdg_status solve_mixed(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info
 // FP64 PCG on (sgn K) x = bvec: the initial residual, then a WHILE loop of two iterations per trip.
 hdg_status cg_solve_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info* info) {
   const int64_t nfe = c->sk.nf * c->Nf;
-  const int nb = c->nb_red, maxit = c->opt.maxit;
+  const int nb = c->nb_red;
   auto build = [&](GraphBuild& gb, cudaGraph_t G, hdg_ctx::DevGraph& dg) {
     std::vector<cudaGraphNode_t> deps, bd;
     const int64_t n0 = c->n_launch;
@@ -528,20 +553,13 @@ hdg_status cg_solve_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solve_i
       c->n_launch += 2;
       cg_init_kernel<<<nb, 256, 0, c->stream>>>(c->sk.nf, c->Nf, c->sgn, c->d_face_slot, c->d_face_bnd, c->d_slot, bvec,
                                                 c->d_dinv, c->d_r, c->d_z, c->d_p, c->d_part);
-      cg_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, c->opt.rtol, c->d_sc);
+      cg_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, c->opt.rtol, c->d_sc, c->d_two64);
     });
     const cudaGraphConditionalHandle h = gb.handle(G, 1, true);
     cudaGraph_t B = gb.loop(G, deps, h);
     const int64_t n1 = c->n_launch;
     gb.seq(B, bd, [&] {
-      for (int par = 0; par < 2; ++par) {
-        HDG_DISPATCH(c, launch_apply, c, c->d_p, c->d_slot, &c->d_sc->done, -1);
-        c->n_launch += 3;
-        HDG_DISPATCH(c, launch_face_q64, c);
-        cg_update_kernel<<<nb, 256, 0, c->stream>>>(nfe, nb, par, c->d_part, c->d_p, c->d_q, c->d_dinv, x, c->d_r, c->d_z,
-                                                    c->d_part + nb, c->d_sc);
-        cg_direction_kernel<<<nb, 256, 0, c->stream>>>(nfe, nb, par, -1, c->d_part + nb, c->d_z, c->d_p, c->d_sc, maxit, h);
-      }
+      for (int par = 0; par < 2; ++par) HDG_DISPATCH(c, launch_iter64, c, x, par, 1, h, -1);
     });
     const int64_t n2 = c->n_launch;
     gb.seq(G, deps, [&] {
@@ -927,7 +945,7 @@ hdg_status cg_solve(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info* i
   c->n_launch += 2;
   cg_init_kernel<<<nb, 256, 0, c->stream>>>(c->sk.nf, c->Nf, c->sgn, c->d_face_slot, c->d_face_bnd, c->d_slot, bvec, c->d_dinv, c->d_r,
                                             c->d_z, c->d_p, c->d_part);
-  cg_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, c->opt.rtol, c->d_sc);
+  cg_init_scalars<<<1, 256, 0, c->stream>>>(nb, c->d_part, c->opt.rtol, c->d_sc, c->d_two64);
   hdg_status s = check_launch(c, "cg_init");
   if (s) return s;
   CUDA_TRY(c, cudaMemcpyAsync(c->h_sc, c->d_sc, sizeof(CgScal), cudaMemcpyDeviceToHost, c->stream));
@@ -942,17 +960,10 @@ hdg_status cg_solve(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info* i
   const int maxit = c->opt.maxit;
   const int chk = std::max(1, c->opt.check_every);
   int first = std::max(2, std::min(chk, c->last_it64 - 1));   // first poll near the last solve's count
-  while (!c->h_sc->done && it < maxit) {
-    const int upto = std::min(maxit, it + (it == 0 ? first : (c->stats_on ? chk : std::min(chk, 4))));
-    for (; it < upto; ++it) {
-      const int par = it & 1;
-      HDG_DISPATCH(c, launch_apply, c, c->d_p, c->d_slot, &c->d_sc->done, it);
-      c->n_launch += 3;
-      HDG_DISPATCH(c, launch_face_q64, c);
-      cg_update_kernel<<<nb, 256, 0, c->stream>>>(nfe, nb, par, c->d_part, c->d_p, c->d_q, c->d_dinv, x, c->d_r, c->d_z,
-                                                  c->d_part + nb, c->d_sc);
-      cg_direction_kernel<<<nb, 256, 0, c->stream>>>(nfe, nb, par, it, c->d_part + nb, c->d_z, c->d_p, c->d_sc, maxit, 0);
-    }
+  // the iteration tests an update at the start of the next one: one more than maxit ends it
+  while (!c->h_sc->done && it <= maxit) {
+    const int upto = std::min(maxit + 1, it + (it == 0 ? first : (c->stats_on ? chk : std::min(chk, 4))));
+    for (; it < upto; ++it) HDG_DISPATCH(c, launch_iter64, c, x, it & 1, 0, cudaGraphConditionalHandle{}, it);
     s = check_launch(c, "cg_iter");
     if (s) return s;
     CUDA_TRY(c, cudaMemcpyAsync(c->h_sc, c->d_sc, sizeof(CgScal), cudaMemcpyDeviceToHost, c->stream));
@@ -2041,6 +2052,11 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   if ((s = dalloc(c, &c->d_slot, (size_t)ne * std::max(c->m, 1) + c->Nf))) return s;
   CUDA_TRY(c, cudaMemsetAsync(c->d_slot, 0, ((size_t)ne * std::max(c->m, 1) + c->Nf) * 8, c->stream));
   if ((s = dalloc(c, &c->d_part, (size_t)c->nb_red * 3 * R))) return s;
+  if (c->opt.prec == HDG_FP64 && c->R == 1) {
+    if ((s = dalloc(c, &c->d_two64, 1))) return s;
+    if ((s = dalloc(c, &c->d_two64A, (size_t)c->sms * 4))) return s;
+    if ((s = dalloc(c, &c->d_two64B, (size_t)2 * c->nb_red))) return s;
+  }
   if (c->R > 1) {
     if ((s = dalloc(c, &c->d_mslot, (size_t)ne * c->m * R))) return s;
     for (double** p : {&c->d_mrho0, &c->d_mrho1, &c->d_malpha, &c->d_mbeta, &c->d_mrr, &c->d_mbb, &c->d_mtol2, &c->d_mscale,

@@ -86,6 +86,8 @@ struct hdg_ctx {
   DevTiming* d_dtime = nullptr;   // device-side launch timing: [0] FP32 apply, [1] FP16 apply
   Cg2State* d_two = nullptr;    // two-kernel FP32 iteration: state, and the partials of its kernels
   float2 *d_twoA = nullptr, *d_twoB = nullptr;
+  Cg64State* d_two64 = nullptr;   // FP64 iteration: state and partials
+  double *d_two64A = nullptr, *d_two64B = nullptr;
   Cg2MState* d_twom = nullptr;  // the same for a narrow column block
   float *d_r32 = nullptr, *d_z32 = nullptr, *d_p32 = nullptr, *d_q32 = nullptr, *d_x32 = nullptr, *d_b32 = nullptr;
   double* d_res = nullptr;   // FP64 refinement residual

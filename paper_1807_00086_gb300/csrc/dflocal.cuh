@@ -107,7 +107,7 @@ static __global__ void local_co_kernel(DevMesh mesh, double alpha, df2* __restri
 // is read along its rows instead. One column: F, the history and the results pass through shared memory,
 // so that the global accesses are contiguous.
 // What bounds it: the instructions of the double-float products (11 each) and of the
-// pointwise steps. k = 3 tetrahedra, modes 0 / 1: 82,944 elements, one column 0.68 / 0.68 ms (0.75 / 0.72
+// pointwise steps. k = 3 tetrahedra, modes 0 / 1: 196,608 elements, one column 0.68 / 0.68 ms (0.75 / 0.72
 // with dense tables), 24,576 x 64 columns 3.3 / 4.1 ms (5.1 / 4.9), 16,464 x 4 columns 0.16 / 0.20 ms (0.24).
 template <int DIM, int K, int CW>
 struct LocalDfCfg {
