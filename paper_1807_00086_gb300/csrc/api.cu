@@ -1061,10 +1061,10 @@ void mlaunch_apply(hdg_ctx* c, const TV* x, TV* slot, const int* done, int iter)
 }
 template <int DIM, int K, int CWN>
 void mlaunch_apply_df_cw(hdg_ctx* c, const double* x, double* slot) {
-  constexpr int EPB = ApplyDfMCfg<DIM, K>::WPB * (32 / CWN);
-  dim3 grid((unsigned)((c->sk.ne + EPB - 1) / EPB), (unsigned)((c->R + CWN - 1) / CWN));
-  apply_df_multi_kernel<DIM, K, CWN><<<grid, 32 * ApplyDfMCfg<DIM, K>::WPB, 0, c->stream>>>(
-      c->sk.ne, c->R, c->d_elem_face, c->d_face_bnd, c->d_mShi, c->d_mSlo, x, slot);
+  constexpr int WPB = ApplyDfMCfg<DIM, K, CWN>::WPB;
+  dim3 grid((unsigned)((c->sk.ne + WPB - 1) / WPB), (unsigned)(c->R / CWN));
+  apply_df_multi_kernel<DIM, K, CWN><<<grid, 32 * WPB, 0, c->stream>>>(c->sk.ne, c->R, c->d_elem_face, c->d_face_bnd, c->d_mShi,
+                                                                       c->d_mSlo, x, slot);
 }
 
 // FP64-accurate R-column apply of the mixed refinement (double-float on the FP32 pipe)

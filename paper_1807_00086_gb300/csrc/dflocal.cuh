@@ -11,39 +11,8 @@
 #pragma once
 
 #include "kernels.cuh"
-#include "multi.cuh"
 
 namespace hdg {
-
-__device__ __forceinline__ df2 df_two_sum(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ df2 df_mul(df2 a, df2 b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
-  const float s = p + e;
-  return {s, e - (s - p)};
-}
-__device__ __forceinline__ df2 df_add(df2 a, df2 b) {
-  df2 s = df_two_sum(a.h, b.h);
-  const float err = s.l + (a.l + b.l);
-  const float h = s.h + err;
-  return {h, err - (h - s.h)};
-}
-__device__ __forceinline__ df2 df_neg(df2 a) { return {-a.h, -a.l}; }
-// normalised value of a compensated accumulator
-__device__ __forceinline__ df2 df_of(const DfAcc& a) { return df_two_sum(a.s, a.c); }
-
-// conversions of the local solves, on the integer pipe (see split_f64)
-__device__ __forceinline__ df2 dfl_from(double x) {
-  df2 v;
-  split_f64(x, v.h, v.l);
-  return v;
-}
-__device__ __forceinline__ double dfl_to(df2 v) { return join_f64(v.h, v.l); }
 
 // Reference tables as rows of their nonzero entries (sparse_rows): the derivative of a mode has a lower
 // degree, and the collapsed-coordinate basis is orthonormal, so Dr holds 202 of 1200 entries and Ff 320 of

@@ -231,77 +231,78 @@ __global__ void __launch_bounds__(128) apply_multi_kernel(int64_t ne, int R, con
 
 // FP64-accurate R-column apply on the FP32 pipe (the refinement residual of the mixed
 // multi-column path): S_K = hi + lo as full row-major FP32 pairs [e][m][m], x split into
-// double-floats and staged lane-contiguous in shared memory. Warp = 32 / CWN elements x CWN columns.
-// Four rows (three where M is no multiple of four) share each x from shared memory, and four
-// entries of a row one 16-byte load, so that the kernel is bounded by its FP32 instructions (11 per
-// product) and not by the load unit: one row and one entry at a time took
-// 1.81 ms for 24,576 tets x 64 columns (k = 3), against 1.29 ms; R = 4, 16,464 tets: 0.255 -> 0.173 ms.
-template <int DIM, int K>
-struct ApplyDfMCfg {   // warps per block: the staged x (M x 32 double-floats per warp) stays under 48 KB
-  static constexpr int WPB = Dims<DIM, K>::M * 32 * 8 * 4 <= 48 * 1024 ? 4 : 2;
+// double-floats and staged in shared memory. A warp multiplies one element by CWN columns: lane = (row
+// lane, column), rows rl + RL i for a lane, so that a warp reads few rows of one element at a time. RB
+// rows share each x from shared memory and, where rows are 16-byte aligned, four entries of a row one
+// load. Bounded by the FP32 instructions (11 per product) and the loads beside them; the conversions run on
+// the integer pipe, for 32 columns on the FP64 pipe, which is idle beside that many products. 24,576
+// tets, k = 3, 64 columns: 1.29 ms; 16,464 x 4 columns: 0.089 ms (0.174 ms with eight elements per warp,
+// whose rows share no cache line).
+template <int DIM, int K, int CWN>
+struct ApplyDfMCfg {
+  static constexpr int M = Dims<DIM, K>::M;
+  static constexpr int WPB = M * CWN * 8 * 4 <= 48 * 1024 ? 4 : 2;   // the staged x stays under 48 KB
+  static constexpr int RL = 32 / CWN;
+  static constexpr int RPL = (M + RL - 1) / RL;                       // rows per lane
+  static constexpr int RB = CWN < 32 && RPL % 5 == 0 ? 5 : RPL % 4 == 0 ? 4 : RPL % 3 == 0 ? 3 : RPL <= 5 ? RPL : 4;
 };
 
 template <int DIM, int K, int CWN>
-__global__ void __launch_bounds__(32 * ApplyDfMCfg<DIM, K>::WPB) apply_df_multi_kernel(int64_t ne, int R, const int32_t* __restrict__ elem_face,
-                                                             const int32_t* __restrict__ face_bnd,
-                                                             const float* __restrict__ Shi,
-                                                             const float* __restrict__ Slo,
-                                                             const double* __restrict__ x, double* __restrict__ slot) {
+__global__ void __launch_bounds__(32 * ApplyDfMCfg<DIM, K, CWN>::WPB)
+    apply_df_multi_kernel(int64_t ne, int R, const int32_t* __restrict__ elem_face, const int32_t* __restrict__ face_bnd,
+                          const float* __restrict__ Shi, const float* __restrict__ Slo, const double* __restrict__ x,
+                          double* __restrict__ slot) {
   using Dm = Dims<DIM, K>;
-  constexpr int NF = Dm::NF, M = Dm::M, NFC = Dm::NFC, EPW = 32 / CWN, WPB = ApplyDfMCfg<DIM, K>::WPB;
-  __shared__ df2 xs[WPB][M][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t e = ((int64_t)blockIdx.x * WPB + w) * EPW + lane / CWN;
-  const int j = blockIdx.y * CWN + lane % CWN;
-  const bool live = e < ne && j < R;
-#pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    const int fid = live ? elem_face[e * NFC + f] : 0;
-    const bool use = live && face_bnd[fid] < 0;
-#pragma unroll
-    for (int mm = 0; mm < NF; ++mm) xs[w][f * NF + mm][lane] = df_from(use ? x[((int64_t)fid * NF + mm) * R + j] : 0.0);
+  using C = ApplyDfMCfg<DIM, K, CWN>;
+  constexpr int NF = Dm::NF, M = Dm::M, NFC = Dm::NFC, WPB = C::WPB, RL = C::RL, RB = C::RB;
+  __shared__ df2 xs[WPB][M][CWN];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, jc = lane % CWN, rl = lane / CWN;
+  const int64_t e = (int64_t)blockIdx.x * WPB + w;
+  const int cb = blockIdx.y * CWN;
+  if (e >= ne) return;
+  for (int r = rl; r < M; r += RL) {
+    const int fid = elem_face[e * NFC + r / NF];
+    const double v = face_bnd[fid] < 0 ? x[((int64_t)fid * NF + r % NF) * R + cb + jc] : 0.0;
+    xs[w][r][jc] = CWN == 32 ? df_from(v) : dfl_from(v);
   }
   __syncwarp();
-  if (!live) return;
   const float* Sh = Shi + e * (int64_t)(M * M);
   const float* Sl = Slo + e * (int64_t)(M * M);
-  double* out = slot + e * (int64_t)M * R + j;
-  if constexpr (M % 4 == 0) {
-    for (int r = 0; r < M; r += 4) {
-      DfAcc acc[4];
+  double* out = slot + e * (int64_t)M * R + cb + jc;
+  for (int r0 = rl; r0 < M; r0 += RL * RB) {
+    DfAcc acc[RB];
+    int row[RB];   // a row past the last one repeats it
+#pragma unroll
+    for (int b = 0; b < RB; ++b) row[b] = min(r0 + RL * b, M - 1) * M;
+    if constexpr (M % 4 == 0) {
 #pragma unroll 2
       for (int c = 0; c < M; c += 4) {
-        float h[4][4], l[4][4];
+        float h[RB][4], l[RB][4];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const float4 u = __ldg(reinterpret_cast<const float4*>(Sh + (r + b) * M + c));
-          const float4 v = __ldg(reinterpret_cast<const float4*>(Sl + (r + b) * M + c));
+        for (int b = 0; b < RB; ++b) {
+          const float4 u = __ldg(reinterpret_cast<const float4*>(Sh + row[b] + c));
+          const float4 v = __ldg(reinterpret_cast<const float4*>(Sl + row[b] + c));
           h[b][0] = u.x; h[b][1] = u.y; h[b][2] = u.z; h[b][3] = u.w;
           l[b][0] = v.x; l[b][1] = v.y; l[b][2] = v.z; l[b][3] = v.w;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const df2 xc = xs[w][c + k][lane];
+          const df2 xc = xs[w][c + k][jc];
 #pragma unroll
-          for (int b = 0; b < 4; ++b) acc[b].fma(df2{h[b][k], l[b][k]}, xc);
+          for (int b = 0; b < RB; ++b) acc[b].fma(df2{h[b][k], l[b][k]}, xc);
         }
       }
-#pragma unroll
-      for (int b = 0; b < 4; ++b) out[(int64_t)(r + b) * R] = acc[b].value();
-    }
-  } else {
-    static_assert(M % 3 == 0, "rows in threes");
-    for (int r = 0; r < M; r += 3) {
-      DfAcc acc[3];
-#pragma unroll
+    } else {
+#pragma unroll 3
       for (int c = 0; c < M; ++c) {
-        const df2 xc = xs[w][c][lane];
+        const df2 xc = xs[w][c][jc];
 #pragma unroll
-        for (int b = 0; b < 3; ++b) acc[b].fma(df2{__ldg(Sh + (r + b) * M + c), __ldg(Sl + (r + b) * M + c)}, xc);
+        for (int b = 0; b < RB; ++b) acc[b].fma(df2{__ldg(Sh + row[b] + c), __ldg(Sl + row[b] + c)}, xc);
       }
-#pragma unroll
-      for (int b = 0; b < 3; ++b) out[(int64_t)(r + b) * R] = acc[b].value();
     }
+#pragma unroll
+    for (int b = 0; b < RB; ++b)
+      if (r0 + RL * b < M) out[(int64_t)(r0 + RL * b) * R] = CWN == 32 ? acc[b].value() : dfl_to(df_of(acc[b]));
   }
 }
 
