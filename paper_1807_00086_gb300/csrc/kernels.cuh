@@ -1307,39 +1307,59 @@ static __global__ void cg32_init_scalars(int nb, const float2* __restrict__ part
 // is folded in): q = sgn (slot0 + slot1) on interior faces (0 on the boundary),
 // x += alpha p, r -= alpha q, z = Dinv r; partials (r.z, r.r). alpha = rho / pq with pq
 // from the apply's reduction. Vectors are processed as float4 (coalesced); the two slot
-// values of each entry are gathered per entry (runs of NF consecutive floats). Two float4
+// values of each entry are gathered by runs within a face. Two float4
 // per trip, and the face flags and slot pairs loaded before the branch on them, keep two
 // independent load chains in flight per thread; a thread visits its entries in the same order
 // as with one float4 per trip, so the sums are the same.
 template <class LD>
 __device__ __forceinline__ float4 q_entries4(int64_t t, int64_t nfe, float sgn, const int2* __restrict__ face_slot2,
                                              const int32_t* __restrict__ face_bnd, const float* __restrict__ slot) {
-  constexpr int NF = LD::NF;
+  // V consecutive entries never leave a face: one face lookup and two V-wide loads serve them
+  constexpr int NF = LD::NF, V = NF % 4 == 0 ? 4 : NF % 2 == 0 ? 2 : 1, G = 4 / V;
   const int64_t d0 = 4 * t;
   uint32_t f = (uint32_t)(d0 / NF);   // n_faces * NF < 2^32
   int mm = (int)(d0 - (int64_t)f * NF);
-  uint32_t fi[4];
-  int mi[4], fb[4];
-  int2 fs[4];
-  bool ok[4];
+  uint32_t fi[G];
+  int mi[G], fb[G];
+  int2 fs[G];
+  bool ok[G];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < G; ++i) {
     fi[i] = f;
     mi[i] = mm;
-    if (++mm == NF) { mm = 0; ++f; }
+    mm += V;
+    if (mm == NF) { mm = 0; ++f; }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    ok[i] = d0 + i < nfe;
+  for (int i = 0; i < G; ++i) {
+    ok[i] = d0 + V * i < nfe;
     fb[i] = ok[i] ? face_bnd[fi[i]] : 0;
     fs[i] = ok[i] ? face_slot2[fi[i]] : make_int2(0, 0);
   }
   float q[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    q[i] = (ok[i] && fb[i] < 0)
-               ? sgn * (slot[(int64_t)fs[i].x * NF + mi[i]] + slot[(int64_t)fs[i].y * NF + mi[i]])
-               : 0.f;
+  for (int i = 0; i < G; ++i) {
+    float a[V], b[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) a[v] = b[v] = 0.f;
+    if (ok[i] && fb[i] < 0) {
+      const float *sa = slot + (int64_t)fs[i].x * NF + mi[i], *sb = slot + (int64_t)fs[i].y * NF + mi[i];
+      if constexpr (V == 4) {
+        const float4 u = *reinterpret_cast<const float4*>(sa), w = *reinterpret_cast<const float4*>(sb);
+        a[0] = u.x; a[1] = u.y; a[2] = u.z; a[3] = u.w;
+        b[0] = w.x; b[1] = w.y; b[2] = w.z; b[3] = w.w;
+      } else if constexpr (V == 2) {
+        const float2 u = *reinterpret_cast<const float2*>(sa), w = *reinterpret_cast<const float2*>(sb);
+        a[0] = u.x; a[1] = u.y;
+        b[0] = w.x; b[1] = w.y;
+      } else {
+        a[0] = *sa;
+        b[0] = *sb;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) q[V * i + v] = sgn * (a[v] + b[v]);
+  }
   return make_float4(q[0], q[1], q[2], q[3]);
 }
 
