@@ -1048,17 +1048,6 @@ void mlaunch_apply_cw(hdg_ctx* c, const TV* x, TV* slot, const int* done) {
                                                                    c->d_S32, c->d_S, x, slot, done);
 }
 
-template <int DIM, int K, typename TV>
-void mlaunch_apply(hdg_ctx* c, const TV* x, TV* slot, const int* done, int iter) {
-  c->n_launch += 1;
-  cudaEvent_t stop = apply_begin(c, sizeof(TV) == 4 ? 1 : 0, iter);
-  if (c->R <= 2) mlaunch_apply_cw<DIM, K, TV, 2>(c, x, slot, done);
-  else if (c->R <= 4) mlaunch_apply_cw<DIM, K, TV, 4>(c, x, slot, done);
-  else if (c->R <= 8) mlaunch_apply_cw<DIM, K, TV, 8>(c, x, slot, done);
-  else if (c->R <= 16) mlaunch_apply_cw<DIM, K, TV, 16>(c, x, slot, done);
-  else mlaunch_apply_cw<DIM, K, TV, 32>(c, x, slot, done);
-  apply_end(c, stop);
-}
 template <int DIM, int K, int CWN>
 void mlaunch_apply_df_cw(hdg_ctx* c, const double* x, double* slot) {
   constexpr int WPB = ApplyDfMCfg<DIM, K, CWN>::WPB;
@@ -1082,13 +1071,23 @@ void mlaunch_apply_df(hdg_ctx* c, const double* x, double* slot) {
 
 template <int DIM, int K>
 void mlaunch_apply64(hdg_ctx* c, const double* x, double* slot, const int* done, int iter) {
-  mlaunch_apply<DIM, K, double>(c, x, slot, done, iter);
+  c->n_launch += 1;
+  cudaEvent_t stop = apply_begin(c, 0, iter);
+  if (c->R <= 2) mlaunch_apply_cw<DIM, K, double, 2>(c, x, slot, done);
+  else if (c->R <= 4) mlaunch_apply_cw<DIM, K, double, 4>(c, x, slot, done);
+  else if (c->R <= 8) mlaunch_apply_cw<DIM, K, double, 8>(c, x, slot, done);
+  else if (c->R <= 16) mlaunch_apply_cw<DIM, K, double, 16>(c, x, slot, done);
+  else mlaunch_apply_cw<DIM, K, double, 32>(c, x, slot, done);
+  apply_end(c, stop);
 }
 template <int DIM, int K>
 void mlaunch_apply32(hdg_ctx* c, const float* x, float* slot, const int* done, int iter) {
-  // fewer than 32 columns: several elements per warp over the group-layout FP32 S_K
+  // two columns: several elements per warp over the group-layout FP32 S_K (4, 8 and 16: m_iter_two)
   if (c->R < 32) {
-    mlaunch_apply<DIM, K, float>(c, x, slot, done, iter);
+    c->n_launch += 1;
+    cudaEvent_t stop = apply_begin(c, 1, iter);
+    mlaunch_apply_cw<DIM, K, float, 2>(c, x, slot, done);
+    apply_end(c, stop);
     return;
   }
   // 32 columns or more: S_K times the column block on the tensor cores

@@ -17,6 +17,7 @@
 
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <type_traits>
 
 #include <cstdint>
 
@@ -1124,6 +1125,15 @@ __global__ void __launch_bounds__(128, 4) apply32_kernel(int64_t ne, const int32
     timing_end(pqo);
   } else if (pqo.part) {
     pq_epilogue(pqo, a.value());
+  }
+}
+
+// f(0), .., f(N - 1) with compile-time arguments: loops too long for the unroller keep register arrays
+template <int I, int N, class F>
+__device__ __forceinline__ void static_for(F&& f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>{});
+    static_for<I + 1, N>(f);
   }
 }
 
