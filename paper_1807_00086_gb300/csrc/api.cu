@@ -52,6 +52,37 @@ void launch_condense(hdg_ctx* c) {
   diag_kernel<Dims<DIM, K>><<<grid_for(c, c->sk.nf * c->Nf), 256, 0, c->stream>>>(devmesh(c), c->d_S, c->sgn, c->d_dinv);
 }
 
+// the operands of the acoustic element-local solves in the arithmetic of the context
+template <class AR>
+struct LocalOps {
+  TabsRows<typename AR::T> tabs;
+  const typename AR::T *geo, *co, *Hinv;
+  typename AR::T tau;
+};
+template <class AR>
+LocalOps<AR> local_ops(const hdg_ctx* c) {
+  if constexpr (std::is_same<AR, ArDf>::value) {
+    const float th = (float)c->tau;
+    return {c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf, df2{th, (float)(c->tau - (double)th)}};
+  } else {
+    return {c->tabssp, c->d_geo, c->d_co64, c->d_Hinv, c->tau};
+  }
+}
+// CW = 0: one column; else blocks of CW columns
+template <class AR, int DIM, int K, int CW>
+void launch_local_ar(hdg_ctx* c, int mode, const double* F, const double* hist, const SrcArgs& sa, const double* lam,
+                     double* out) {
+  using L = LocalCfg<DIM, K, CW>;
+  const dim3 grid((unsigned)((c->sk.ne + L::EPB - 1) / L::EPB), CW ? (unsigned)(c->R / (CW ? CW : 1)) : 1u);
+  const LocalOps<AR> o = local_ops<AR>(c);
+  if (mode == 0)
+    local_kernel<AR, DIM, K, 0, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), o.tabs, o.geo, o.co, o.Hinv, o.tau, c->R, F,
+                                                                   hist, sa, lam, out);
+  else
+    local_kernel<AR, DIM, K, 1, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), o.tabs, o.geo, o.co, o.Hinv, o.tau, c->R, F,
+                                                                   hist, sa, lam, out);
+}
+
 template <int DIM, int K>
 void launch_local(hdg_ctx* c, int mode, const double* F, const double* hist, double t, const double* lam, double* out) {
   if (c->phys == HDG_ELASTIC) {
@@ -68,27 +99,8 @@ void launch_local(hdg_ctx* c, int mode, const double* F, const double* hist, dou
   }
   const SrcArgs sa = srcargs(c, t);
   c->n_launch += 1;
-  if (c->d_Hinvdf) {
-    using LD = LocalDfCfg<DIM, K, 0>;
-    const unsigned gd = (unsigned)((c->sk.ne + LD::EPB - 1) / LD::EPB);
-    const float th = (float)c->tau;
-    const df2 tau{th, (float)(c->tau - (double)th)};
-    if (mode == 0)
-      local_df_kernel<DIM, K, 0, 0><<<gd, LD::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
-                                                                  tau, 1, F, hist, sa, lam, out);
-    else
-      local_df_kernel<DIM, K, 1, 0><<<gd, LD::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
-                                                                  tau, 1, F, hist, sa, lam, out);
-    return;
-  }
-  using L = LocalCfg<DIM, K>;
-  const unsigned grid = (unsigned)((c->sk.ne + L::EPB - 1) / L::EPB);
-  if (mode == 0)
-    local_kernel<DIM, K, 0><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabs, c->d_Hinv, c->alpha, c->tau, F, hist, sa, lam,
-                                                            out);
-  else
-    local_kernel<DIM, K, 1><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabs, c->d_Hinv, c->alpha, c->tau, F, hist, sa, lam,
-                                                            out);
+  if (c->d_Hinvdf) launch_local_ar<ArDf, DIM, K, 0>(c, mode, F, hist, sa, lam, out);
+  else launch_local_ar<ArF64, DIM, K, 0>(c, mode, F, hist, sa, lam, out);
 }
 
 template <class L>
@@ -398,6 +410,10 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
   HDG_DISPATCH(c, launch_condense, c);
   hdg_status s = check_launch(c, "condense");
   if (s) return s;
+  if (c->d_co64) {
+    c->n_launch += 1;
+    local_co_kernel<ArF64><<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_co64);
+  }
   if (c->opt.prec != HDG_FP64) {
     if (c->d_S32lo) {
       HDG_DISPATCH(c, launch_sym_pack, c);
@@ -415,7 +431,7 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
       }
       const int64_t nH = c->sk.ne * (int64_t)c->nv * c->nv;
       c->n_launch += 2;
-      local_co_kernel<<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_codf);
+      local_co_kernel<ArDf><<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_codf);
       to_df_kernel<<<grid_for(c, nH), 256, 0, c->stream>>>(nH, c->d_Hinv, c->d_Hinvdf);
     }
     const int64_t nfe = c->sk.nf * c->Nf;
@@ -992,52 +1008,20 @@ MScal mscal(hdg_ctx* c) {
   return m;
 }
 
-template <int DIM, int K, int CWW>
-void mlaunch_local_cw(hdg_ctx* c, int mode, const double* F, const double* hist, const SrcArgs& sa, const double* lam,
-                      double* out) {
-  using L = LocalMultiCfg<DIM, K, CWW>;
-  dim3 grid((unsigned)c->sk.ne, (unsigned)((c->R + L::CW - 1) / L::CW));
-  if (mode == 0)
-    local_multi_kernel<DIM, K, 0, CWW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabs, c->d_Hinv, c->alpha, c->tau,
-                                                                       c->R, F, hist, sa, lam, out);
-  else
-    local_multi_kernel<DIM, K, 1, CWW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabs, c->d_Hinv, c->alpha, c->tau,
-                                                                       c->R, F, hist, sa, lam, out);
-}
-
-// mixed precision: double-float on the FP32 pipe
-template <int DIM, int K, int CW>
-void mlaunch_local_df(hdg_ctx* c, int mode, const double* F, const double* hist, const SrcArgs& sa, const double* lam,
-                      double* out) {
-  using L = LocalDfCfg<DIM, K, CW>;
-  const dim3 grid((unsigned)((c->sk.ne + L::EPB - 1) / L::EPB), (unsigned)(c->R / CW));
-  const float th = (float)c->tau;
-  const df2 tau{th, (float)(c->tau - (double)th)};
-  if (mode == 0)
-    local_df_kernel<DIM, K, 0, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
-                                                                  tau, c->R, F, hist, sa, lam, out);
-  else
-    local_df_kernel<DIM, K, 1, CW><<<grid, L::NT, 0, c->stream>>>(devmesh(c), c->tabsdf, c->d_geodf, c->d_codf, c->d_Hinvdf,
-                                                                  tau, c->R, F, hist, sa, lam, out);
-}
-
-template <int DIM, int K>
-void mlaunch_local(hdg_ctx* c, int mode, const double* F, const double* hist, double t, const double* lam, double* out) {
+template <class AR, int DIM, int K>
+void mlaunch_local_ar(hdg_ctx* c, int mode, const double* F, const double* hist, double t, const double* lam, double* out) {
   const SrcArgs sa = srcargs(c, t);
   c->n_launch += 1;
   // as many columns per CTA as the batch has (up to the kernel's width)
-  if (c->d_Hinvdf) {
-    if (c->R <= 2) mlaunch_local_df<DIM, K, 2>(c, mode, F, hist, sa, lam, out);
-    else if (c->R <= 4) mlaunch_local_df<DIM, K, 4>(c, mode, F, hist, sa, lam, out);
-    else if (c->R <= 8) mlaunch_local_df<DIM, K, 8>(c, mode, F, hist, sa, lam, out);
-    else mlaunch_local_df<DIM, K, 16>(c, mode, F, hist, sa, lam, out);
-    return;
-  }
-  if (c->R <= 2) mlaunch_local_cw<DIM, K, 2>(c, mode, F, hist, sa, lam, out);
-  else if (c->R <= 4) mlaunch_local_cw<DIM, K, 4>(c, mode, F, hist, sa, lam, out);
-  else if (c->R <= 8) mlaunch_local_cw<DIM, K, 8>(c, mode, F, hist, sa, lam, out);
-  else if (c->R <= 16) mlaunch_local_cw<DIM, K, 16>(c, mode, F, hist, sa, lam, out);
-  else mlaunch_local_cw<DIM, K, 32>(c, mode, F, hist, sa, lam, out);
+  if (c->R <= 2) launch_local_ar<AR, DIM, K, 2>(c, mode, F, hist, sa, lam, out);
+  else if (c->R <= 4) launch_local_ar<AR, DIM, K, 4>(c, mode, F, hist, sa, lam, out);
+  else if (c->R <= 8) launch_local_ar<AR, DIM, K, 8>(c, mode, F, hist, sa, lam, out);
+  else launch_local_ar<AR, DIM, K, 16>(c, mode, F, hist, sa, lam, out);
+}
+template <int DIM, int K>
+void mlaunch_local(hdg_ctx* c, int mode, const double* F, const double* hist, double t, const double* lam, double* out) {
+  if (c->d_Hinvdf) mlaunch_local_ar<ArDf, DIM, K>(c, mode, F, hist, t, lam, out);
+  else mlaunch_local_ar<ArF64, DIM, K>(c, mode, F, hist, t, lam, out);
 }
 
 template <int DIM, int K, typename TV, int CWN>
@@ -2037,7 +2021,9 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   if ((s = dalloc(c, &c->d_qv_phi, c->T.qv_phi.size()))) return s;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_qv_w, c->T.qv_w.data(), c->T.qv_w.size() * 8, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(c->d_qv_phi, c->T.qv_phi.data(), c->T.qv_phi.size() * 8, cudaMemcpyHostToDevice, c->stream));
-  if (c->phys == HDG_ELASTIC && !svk && (s = upload_sparse(c, sparse_rows(c->T), c->tabssp))) return s;
+  if (!svk && (c->phys == HDG_ELASTIC || c->opt.prec == HDG_FP64) && (s = upload_sparse(c, sparse_rows(c->T), c->tabssp)))
+    return s;
+  if (c->phys == HDG_ACOUSTIC && c->opt.prec == HDG_FP64 && (s = dalloc(c, &c->d_co64, (size_t)ne * 4))) return s;
   // condensed operators and workspaces
   const size_t nfe = (size_t)nf * c->Nf;
   const size_t R = (size_t)c->R;
@@ -2133,21 +2119,8 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
       c->n_launch += 1;
       to_df_kernel<<<grid_for(c, ne * GEO_STRIDE), 256, 0, c->stream>>>(ne * GEO_STRIDE, c->d_geo, c->d_geodf);
       if ((s = dalloc(c, &c->d_codf, (size_t)ne * 4))) return s;
-      const SparseRows sp = sparse_rows(c->T);
-      std::vector<SpDf> ent(sp.val.size());
-      for (size_t q = 0; q < ent.size(); ++q) {
-        const float h = (float)sp.val[q];
-        ent[q] = SpDf{h, (float)(sp.val[q] - (double)h), sp.idx[q], 0};
-      }
-      std::vector<int32_t> ip(sp.ptr);
-      ip.insert(ip.end(), sp.perm.begin(), sp.perm.end());
-      if ((s = dalloc(c, &c->d_tabdf, ent.size()))) return s;
-      if ((s = dalloc(c, &c->d_tabptr, ip.size()))) return s;
-      CUDA_TRY(c, cudaMemcpyAsync(c->d_tabdf, ent.data(), ent.size() * sizeof(SpDf), cudaMemcpyHostToDevice, c->stream));
-      CUDA_TRY(c, cudaMemcpyAsync(c->d_tabptr, ip.data(), ip.size() * 4, cudaMemcpyHostToDevice, c->stream));
-      // the host copies are released below only after the stream has consumed them
-      CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-      c->tabsdf = TabsDf{c->d_tabdf, c->d_tabptr, c->d_tabptr + sp.ptr.size()};
+      auto split = [](double v) { const float h = (float)v; return df2{h, (float)(v - (double)h)}; };
+      if ((s = upload_rows(c, sparse_rows(c->T), split, c->tabsdf, nullptr))) return s;
     }
     if ((s = dalloc(c, &c->d_res, nfe * R))) return s;
     if ((s = dalloc(c, &c->d_rs, 1))) return s;

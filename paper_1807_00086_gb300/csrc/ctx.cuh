@@ -72,11 +72,10 @@ struct hdg_ctx {
   df2 *d_Hinvdf = nullptr, *d_geodf = nullptr, *d_codf = nullptr;
   TabsSp tabssp{};                     // nonzero rows of the reference tables
   double* d_elco = nullptr;            // elastic: element coefficients at the mass shift
-  SpDf* d_tabdf = nullptr;
-  int32_t* d_tabptr = nullptr;
+  double* d_co64 = nullptr;            // the coefficients of the FP64 acoustic solves
   double* d_post = nullptr;       // post-processing tables K1 | E1 (PostTabs; built at the first hdg_postprocess)
   int64_t post_k1 = 0;            // entries of K1
-  TabsDf tabsdf{};
+  TabsRows<df2> tabsdf{};
   __half* d_S16 = nullptr;      // FP16 packed S_K (inner Krylov operator of HDG_MIXED16)
   float* d_sc16 = nullptr;      // its per-element scales
   int32_t* d_gface16 = nullptr; // its trace gather table [whole groups][nfc] (face id, -1: none)
@@ -210,23 +209,28 @@ hdg_status dalloc(hdg_ctx* c, T** p, size_t count) {
   return HDG_OK;
 }
 
-// device copy of the nonzero table rows (see SparseRows)
-inline hdg_status upload_sparse(hdg_ctx* c, const SparseRows& sp, TabsSp& T) {
-  std::vector<SpD> ent(sp.val.size());
-  for (size_t q = 0; q < ent.size(); ++q) ent[q] = SpD{sp.val[q], sp.idx[q], 0};
+// device copy of the nonzero table rows (see SparseRows); ints: ptr, perm, permb
+template <class T, class F>
+hdg_status upload_rows(hdg_ctx* c, const SparseRows& sp, F&& conv, TabsRows<T>& t, const int32_t** permb) {
+  std::vector<SpEnt<T>> ent(sp.val.size());
+  for (size_t q = 0; q < ent.size(); ++q) ent[q] = SpEnt<T>{conv(sp.val[q]), sp.idx[q], 0};
   std::vector<int32_t> ip(sp.ptr);
   ip.insert(ip.end(), sp.perm.begin(), sp.perm.end());
   ip.insert(ip.end(), sp.permb.begin(), sp.permb.end());
-  SpD* d = nullptr;
+  SpEnt<T>* d = nullptr;
   int32_t* p = nullptr;
   hdg_status s;
   if ((s = dalloc(c, &d, ent.size()))) return s;
   if ((s = dalloc(c, &p, ip.size()))) return s;
-  CUDA_TRY(c, cudaMemcpyAsync(d, ent.data(), ent.size() * sizeof(SpD), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(d, ent.data(), ent.size() * sizeof(SpEnt<T>), cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(p, ip.data(), ip.size() * 4, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));   // the host copies are released here
-  T = TabsSp{d, p, p + sp.ptr.size(), p + sp.ptr.size() + sp.perm.size()};
+  t = TabsRows<T>{d, p, p + sp.ptr.size()};
+  if (permb) *permb = p + sp.ptr.size() + sp.perm.size();
   return HDG_OK;
+}
+inline hdg_status upload_sparse(hdg_ctx* c, const SparseRows& sp, TabsSp& t) {
+  return upload_rows(c, sp, [](double v) { return v; }, static_cast<TabsRows<double>&>(t), &t.permb);
 }
 
 void dfree(hdg_ctx* c, void* p) {

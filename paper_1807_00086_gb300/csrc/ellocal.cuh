@@ -14,6 +14,7 @@
 // (0.20 ms).
 #pragma once
 
+#include "dflocal.cuh"
 #include "elastic.cuh"
 
 namespace hdg {
@@ -33,14 +34,9 @@ struct VdDims {
   static constexpr int ON = 1 + DIM * DIM + DIM + 1;
 };
 
-// nonzero rows of the reference tables (row groups and order of SparseRows)
-struct alignas(16) SpD {
-  double v;
-  int idx, pad;
-};
-struct TabsSp {
-  const SpD* ent;
-  const int32_t *ptr, *perm, *permb;
+// nonzero rows of the reference tables and the order of the rows of group B (see SparseRows)
+struct TabsSp : TabsRows<double> {
+  const int32_t* permb;
 };
 __device__ __forceinline__ double sp_row(const TabsSp& T, int row, const double* x) {
   double s = 0.0;

@@ -91,182 +91,6 @@ __global__ void diag_kernel(DevMesh mesh, const double* __restrict__ S, double s
   }
 }
 
-// ---------------------------------------------------------------- element-local solves
-// MODE 0 (condensed rhs): out = gslot [ne][M] = C_K A_K^{-1} (F_K - B_K lamD_K)
-// MODE 1 (recovery):      out = u     [ne][N] = A_K^{-1} (F_K - B_K lam_K)
-// F_K is F[e] when hist == nullptr, else alpha Mw_K hist[e] + r(t) sum_src phi(x_s).
-// EPB elements per CTA, one thread per (element, row i < NP); only three block-wide
-// barriers, the rest of each element's work is row-local.
-template <int DIM, int K>
-struct LocalCfg {
-  static constexpr int NP = Dims<DIM, K>::NP;
-  static constexpr int EPB = NP <= 10 ? 16 : (NP <= 20 ? 8 : 4);
-  static constexpr int NT = EPB * NP;
-};
-
-template <int DIM, int K, int MODE>
-__global__ void __launch_bounds__(LocalCfg<DIM, K>::NT) local_kernel(DevMesh mesh, Tabs T, const double* __restrict__ Hinv,
-                                                                    double alpha, double tau, const double* __restrict__ F,
-                                                                    const double* __restrict__ hist, SrcArgs src,
-                                                                    const double* __restrict__ lam, double* __restrict__ out) {
-  using D = Dims<DIM, K>;
-  using L = LocalCfg<DIM, K>;
-  constexpr int NP = D::NP, NF = D::NF, M = D::M, NFC = D::NFC, N = D::N, EPB = L::EPB, NT = L::NT;
-  __shared__ double g[EPB][GEO_STRIDE];
-  __shared__ double ll[EPB][M];
-  __shared__ double Tr[EPB][DIM * NP];   // reused for the face weights w_f in MODE 0
-  __shared__ double rp[EPB][NP];
-  __shared__ double pp[EPB][NP];
-  __shared__ double co[EPB][2];          // b = alpha rho, a' = alpha dJ / (rho c^2) (hist mode)
-  __shared__ int fuse[EPB][NFC];         // face contributes a trace (nonzero lam) to this element
-  const int tid = threadIdx.x;
-  const int64_t e0 = (int64_t)blockIdx.x * EPB;
-  for (int t = tid; t < EPB * GEO_STRIDE; t += NT) {
-    const int64_t e = e0 + t / GEO_STRIDE;
-    g[t / GEO_STRIDE][t % GEO_STRIDE] = e < mesh.ne ? mesh.geo[e * GEO_STRIDE + t % GEO_STRIDE] : (t % GEO_STRIDE == 0 ? 1.0 : 0.0);
-  }
-  for (int t = tid; t < EPB * NFC; t += NT) {
-    const int64_t e = e0 + t / NFC;
-    int use = 0;
-    if (e < mesh.ne && lam) {
-      const int f = mesh.elem_face[e * NFC + t % NFC];
-      use = (MODE == 1) || (mesh.face_bnd[f] >= 0);
-    }
-    fuse[t / NFC][t % NFC] = use;
-  }
-  for (int t = tid; t < EPB * M; t += NT) {
-    const int64_t e = e0 + t / M;
-    const int r = t % M;
-    double v = 0.0;
-    if (e < mesh.ne && lam) {
-      const int f = mesh.elem_face[e * NFC + r / NF];
-      if ((MODE == 1) || (mesh.face_bnd[f] >= 0)) v = lam[(int64_t)f * NF + r % NF];
-    }
-    ll[t / M][r] = v;
-  }
-  if (tid < EPB) {
-    const int64_t e = e0 + tid;
-    const double rho = e < mesh.ne ? mesh.rho[e] : 1.0, cc = e < mesh.ne ? mesh.c[e] : 1.0;
-    co[tid][0] = alpha * rho;
-    co[tid][1] = alpha / (rho * cc * cc);
-  }
-  __syncthreads();
-  const int el = tid / NP, i = tid % NP;
-  const int64_t e = e0 + el;
-  const bool live = e < mesh.ne;
-  const double* ge = g[el];
-  const double dJ = ge[0];
-  const double b = co[el][0];
-  // row i of F~ for all components (+ the F^ lam face products it needs)
-  double Fu[DIM + 1];
-  {
-    double Fl[NFC];
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      double s = 0.0;
-      if (fuse[el][f])
-        for (int mm = 0; mm < NF; ++mm) s += T.Ff[(f * NP + i) * NF + mm] * ll[el][f * NF + mm];
-      Fl[f] = s;
-    }
-#pragma unroll
-    for (int comp = 0; comp <= DIM; ++comp) {
-      double v = 0.0;
-      if (live) {
-        if (hist) {
-          const double sc = comp == 0 ? co[el][1] * dJ : b * dJ;
-          v = sc * hist[e * N + comp * NP + i];
-          if (comp == 0 && src.ptr)
-            for (int q = src.ptr[e]; q < src.ptr[e + 1]; ++q) v += ricker_at(src, q) * src.phi[(int64_t)q * NP + i];
-        } else {
-          v = F[e * N + comp * NP + i];
-        }
-      }
-      double bl = 0.0;
-      if (comp == 0) {
-#pragma unroll
-        for (int f = 0; f < NFC; ++f) bl += ge[D::OJF + f] * Fl[f];
-        v += tau * bl;
-      } else {
-#pragma unroll
-        for (int f = 0; f < NFC; ++f) bl += ge[D::ON + f * DIM + comp - 1] * ge[D::OJF + f] * Fl[f];
-        v -= bl;
-      }
-      Fu[comp] = v;
-    }
-  }
-  // Tr[r][i] = sum_j Jinv[r][j] F~v_j[i]
-#pragma unroll
-  for (int r = 0; r < DIM; ++r) {
-    double s = 0.0;
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) s += ge[1 + r * DIM + j] * Fu[j + 1];
-    Tr[el][r * NP + i] = s;
-  }
-  __syncthreads();
-  {
-    double s = 0.0;
-#pragma unroll
-    for (int r = 0; r < DIM; ++r)
-      for (int l = 0; l < NP; ++l) s += T.Dr[(r * NP + i) * NP + l] * Tr[el][r * NP + l];
-    rp[el][i] = Fu[0] - s / b;
-  }
-  __syncthreads();
-  {
-    // p = H^{-1} rp; H^{-1} is symmetric, so row i is read as column i (coalesced)
-    const double* He = Hinv + (live ? e : 0) * (int64_t)(NP * NP);
-    double s = 0.0;
-    for (int l = 0; l < NP; ++l) s += He[l * NP + i] * rp[el][l];
-    pp[el][i] = s;
-  }
-  __syncthreads();
-  double vv[DIM];
-  {
-    double qd[DIM];
-#pragma unroll
-    for (int r = 0; r < DIM; ++r) {
-      double s = 0.0;
-      for (int l = 0; l < NP; ++l) s += T.Dr[(r * NP + l) * NP + i] * pp[el][l];
-      qd[r] = s;
-    }
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) {
-      double s = 0.0;
-#pragma unroll
-      for (int r = 0; r < DIM; ++r) s += ge[1 + r * DIM + j] * qd[r];
-      vv[j] = Fu[j + 1] / (b * dJ) + s / b;
-    }
-  }
-  if (MODE == 1) {
-    if (live) {
-      out[e * N + i] = pp[el][i];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) out[e * N + (j + 1) * NP + i] = vv[j];
-    }
-    return;
-  }
-  // MODE 0: w_f[i] = tau p[i] + sum_j n_fj v_j[i]  (Tr reused: NFC*NP <= DIM*NP + NP)
-  double* w = &Tr[el][0];
-  __syncthreads();   // every thread is done reading Tr
-#pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    double s = tau * pp[el][i];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) s += ge[D::ON + f * DIM + j] * vv[j];
-    if (f < DIM) w[f * NP + i] = s;
-    else rp[el][i] = s;                   // last face's weights live in rp (no longer needed)
-  }
-  __syncthreads();
-  for (int t = tid; t < EPB * M; t += NT) {
-    const int el2 = t / M, r = t % M, f = r / NF, mm = r % NF;
-    const int64_t e2 = e0 + el2;
-    if (e2 >= mesh.ne) continue;
-    const double* wf = f < DIM ? &Tr[el2][f * NP] : &rp[el2][0];
-    double s = 0.0;
-    for (int q = 0; q < NP; ++q) s += T.Ff[(f * NP + q) * NF + mm] * wf[q];
-    out[e2 * M + r] = g[el2][D::OJF + f] * s;
-  }
-}
-
 // ---------------------------------------------------------------- matrix-free trace apply (d)
 // zslot[e][r] = sum_c S_K[r][c] x_K[c], x gathered from faces (boundary faces read as 0).
 // S_K is symmetric, so thread r reads column r (coalesced across the element's threads).
@@ -618,8 +442,8 @@ static __global__ void cg_direction_kernel(int64_t n, int nb, int parity, int it
 // ---- FP64 iteration in two kernels (one column, discontinuous traces): A = operator with the direction
 // p_K = z_K + beta p_K formed in the gather, B = update of p, x, r, z; the scheme of Cg2State with FP64
 // partials. For small systems, bounded by the latency of an iteration's dependent launches; each sum
-// is formed by the warps side by side, and one thread of a CTA divides. Triangles, k = 2, 2,048 to 4,050
-// elements: about 10 us an iteration (14.8 us in four kernels).
+// is formed by the warps side by side, and one thread of a CTA divides. 512 triangles, k = 2: 10 us an
+// iteration (14.8 us in four kernels).
 struct Cg64Args {
   CgScal* sc;
   Cg64State* st;

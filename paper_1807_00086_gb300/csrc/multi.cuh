@@ -9,163 +9,6 @@
 
 namespace hdg {
 
-// ------------------------------------------------------------------ element-local solves, R columns
-// CTA = one element x CW columns x NP rows; with CW = 32 a warp is one row over 32 columns, so
-// table, geometry and H^{-1} reads are warp-uniform and field reads are coalesced along columns.
-// CW = columns per CTA: min(R, 32) (16 when N_p > 32), so a narrow batch (a few serving slots)
-// keeps every thread busy.
-template <int DIM, int K, int CWW = 32>
-struct LocalMultiCfg {
-  static constexpr int NP = Dims<DIM, K>::NP;
-  static constexpr int CW = (NP <= 32 ? 32 : 16) < CWW ? (NP <= 32 ? 32 : 16) : CWW;
-  static constexpr int NT = NP * CW;
-};
-
-template <int DIM, int K, int MODE, int CWW = 32>
-__global__ void __launch_bounds__(LocalMultiCfg<DIM, K, CWW>::NT)
-    local_multi_kernel(DevMesh mesh, Tabs T, const double* __restrict__ Hinv, double alpha, double tau, int R,
-                       const double* __restrict__ F, const double* __restrict__ hist, SrcArgs src,
-                       const double* __restrict__ lam, double* __restrict__ out) {
-  using D = Dims<DIM, K>;
-  using L = LocalMultiCfg<DIM, K, CWW>;
-  constexpr int NP = D::NP, NF = D::NF, M = D::M, NFC = D::NFC, N = D::N, CW = L::CW;
-  __shared__ double g[GEO_STRIDE];
-  __shared__ double Tr[DIM * NP][CW];
-  __shared__ double rp[NP][CW];
-  __shared__ double pp[NP][CW];
-  __shared__ double ll[M][CW];
-  __shared__ int fuse[NFC];
-  const int64_t e = blockIdx.x;
-  const int jl = threadIdx.x % CW, i = threadIdx.x / CW;
-  const int j = blockIdx.y * CW + jl;
-  const bool col = j < R;
-  for (int t = threadIdx.x; t < GEO_STRIDE; t += L::NT) g[t] = mesh.geo[e * GEO_STRIDE + t];   // NT may be < 32
-  if (threadIdx.x < NFC) {
-    int use = 0;
-    if (lam) {
-      const int f = mesh.elem_face[e * NFC + threadIdx.x];
-      use = (MODE == 1) || (mesh.face_bnd[f] >= 0);
-    }
-    fuse[threadIdx.x] = use;
-  }
-  for (int t = threadIdx.x; t < M * CW; t += L::NT) {
-    const int r = t / CW, jj = blockIdx.y * CW + t % CW;
-    double v = 0.0;
-    if (lam && jj < R) {
-      const int f = mesh.elem_face[e * NFC + r / NF];
-      if ((MODE == 1) || (mesh.face_bnd[f] >= 0)) v = lam[((int64_t)f * NF + r % NF) * R + jj];
-    }
-    ll[r][t % CW] = v;
-  }
-  __syncthreads();
-  const double dJ = g[0];
-  const double rho = mesh.rho[e], cc = mesh.c[e];
-  const double b = alpha * rho;
-  double Fu[DIM + 1];
-  {
-    double Fl[NFC];
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      double s = 0.0;
-      if (fuse[f])
-        for (int mm = 0; mm < NF; ++mm) s += T.Ff[(f * NP + i) * NF + mm] * ll[f * NF + mm][jl];
-      Fl[f] = s;
-    }
-#pragma unroll
-    for (int comp = 0; comp <= DIM; ++comp) {
-      double v = 0.0;
-      if (col) {
-        const int64_t idx = (e * N + comp * NP + i) * R + j;
-        if (hist) {
-          v = (comp == 0 ? alpha * dJ / (rho * cc * cc) : b * dJ) * hist[idx];
-          if (comp == 0 && src.ptr)
-            for (int q = src.ptr[e]; q < src.ptr[e + 1]; ++q)
-              if (src.col[q] == j) v += ricker_at(src, q) * src.phi[(int64_t)q * NP + i];
-        } else {
-          v = F[idx];
-        }
-      }
-      double bl = 0.0;
-      if (comp == 0) {
-#pragma unroll
-        for (int f = 0; f < NFC; ++f) bl += g[D::OJF + f] * Fl[f];
-        v += tau * bl;
-      } else {
-#pragma unroll
-        for (int f = 0; f < NFC; ++f) bl += g[D::ON + f * DIM + comp - 1] * g[D::OJF + f] * Fl[f];
-        v -= bl;
-      }
-      Fu[comp] = v;
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < DIM; ++r) {
-    double s = 0.0;
-#pragma unroll
-    for (int jj = 0; jj < DIM; ++jj) s += g[1 + r * DIM + jj] * Fu[jj + 1];
-    Tr[r * NP + i][jl] = s;
-  }
-  __syncthreads();
-  {
-    double s = 0.0;
-#pragma unroll
-    for (int r = 0; r < DIM; ++r)
-      for (int l = 0; l < NP; ++l) s += T.Dr[(r * NP + i) * NP + l] * Tr[r * NP + l][jl];
-    rp[i][jl] = Fu[0] - s / b;
-  }
-  __syncthreads();
-  {
-    const double* He = Hinv + e * (int64_t)(NP * NP);
-    double s = 0.0;
-    for (int l = 0; l < NP; ++l) s += He[i * NP + l] * rp[l][jl];
-    pp[i][jl] = s;
-  }
-  __syncthreads();
-  double vv[DIM];
-  {
-    double qd[DIM];
-#pragma unroll
-    for (int r = 0; r < DIM; ++r) {
-      double s = 0.0;
-      for (int l = 0; l < NP; ++l) s += T.Dr[(r * NP + l) * NP + i] * pp[l][jl];
-      qd[r] = s;
-    }
-#pragma unroll
-    for (int jj = 0; jj < DIM; ++jj) {
-      double s = 0.0;
-#pragma unroll
-      for (int r = 0; r < DIM; ++r) s += g[1 + r * DIM + jj] * qd[r];
-      vv[jj] = Fu[jj + 1] / (b * dJ) + s / b;
-    }
-  }
-  if (MODE == 1) {
-    if (col) {
-      out[(e * N + i) * R + j] = pp[i][jl];
-#pragma unroll
-      for (int jj = 0; jj < DIM; ++jj) out[(e * N + (jj + 1) * NP + i) * R + j] = vv[jj];
-    }
-    return;
-  }
-  __syncthreads();   // all reads of Tr done: reuse it (and rp) for the face weights
-#pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    double s = tau * pp[i][jl];
-#pragma unroll
-    for (int jj = 0; jj < DIM; ++jj) s += g[D::ON + f * DIM + jj] * vv[jj];
-    if (f < DIM) Tr[f * NP + i][jl] = s;
-    else rp[i][jl] = s;
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < M * CW; t += L::NT) {
-    const int r = t / CW, jj2 = t % CW, f = r / NF, mm = r % NF;
-    const int jc = blockIdx.y * CW + jj2;
-    if (jc >= R) continue;
-    double s = 0.0;
-    for (int q = 0; q < NP; ++q) s += T.Ff[(f * NP + q) * NF + mm] * (f < DIM ? Tr[f * NP + q][jj2] : rp[q][jj2]);
-    out[(e * M + r) * R + jc] = g[D::OJF + f] * s;
-  }
-}
-
 // ------------------------------------------------------------------ trace apply, R columns
 // warp = (element, 32-column group); lane = column. S_K entries are warp-uniform loads.
 // FP32: S from the packed group layout of pack_kernel. FP64: S from [e][M][M].
