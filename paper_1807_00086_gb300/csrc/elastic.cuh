@@ -60,7 +60,7 @@ __device__ __forceinline__ int qa(int a, int i) {
   if (i == aj && ai != aj) return ai;
   return -1;
 }
-// Cm = compliance^{-1} in the component basis; Q = compliance (for the mass term)
+// Cm = compliance^{-1} in the component basis
 template <int DIM>
 __device__ __forceinline__ double cm_entry(int a, int b, double lam, double mu) {
   int ai, aj, bi, bj;
@@ -69,17 +69,6 @@ __device__ __forceinline__ double cm_entry(int a, int b, double lam, double mu) 
   if (ai == aj && bi == bj) return lam + (a == b ? 2.0 * mu : 0.0);
   return a == b ? mu : 0.0;
 }
-template <int DIM>
-__device__ __forceinline__ double q_entry(int a, int b, double lam, double mu) {
-  int ai, aj, bi, bj;
-  sym_ij<DIM>(a, ai, aj);
-  sym_ij<DIM>(b, bi, bj);
-  double v = 0.0;
-  if (a == b) v += (ai == aj ? 1.0 : 2.0) / (2.0 * mu);
-  if (ai == aj && bi == bj) v -= lam / ((DIM * lam + 2.0 * mu) * 2.0 * mu);
-  return v;
-}
-
 // ------------------------------------------------------------------ condensation
 template <int DIM, int K>
 struct CondElCfg {

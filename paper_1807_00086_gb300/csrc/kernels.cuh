@@ -1411,7 +1411,6 @@ __device__ __forceinline__ df2 df_from(double x) {
   const float h = __double2float_rn(x);
   return {h, __double2float_rn(x - (double)h)};
 }
-__device__ __forceinline__ double df_to(df2 a) { return (double)a.h + (double)a.l; }
 
 // hi = fl32(v), lo = fl32(v - hi), bit for bit as the FP64 conversions give them, on the integer
 // pipe: the four FP64 instructions of the other route cost a copy kernel more than its bytes do
@@ -1481,7 +1480,6 @@ __device__ __forceinline__ df2 df_add(df2 a, df2 b) {
   const float h = s.h + err;
   return {h, err - (h - s.h)};
 }
-__device__ __forceinline__ df2 df_neg(df2 a) { return {-a.h, -a.l}; }
 // normalised value of a compensated accumulator
 __device__ __forceinline__ df2 df_of(const DfAcc& a) { return df_two_sum(a.s, a.c); }
 

@@ -277,7 +277,7 @@ hdg_status vd_cg(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info* info
       const int par = it & 1;
       vd_apply64(c, c->d_p, c->d_slot, &c->d_sc->done, it);
       c->n_launch += 3;
-      vd_face_q_kernel<double><<<nb, 256, 0, c->stream>>>(n, c->sgn, c->vd->d_dslot, c->d_slot, c->d_p, c->d_q,
+      vd_face_q_kernel<<<nb, 256, 0, c->stream>>>(n, c->sgn, c->vd->d_dslot, c->d_slot, c->d_p, c->d_q,
                                                           c->d_part, c->d_sc);
       cg_update_kernel<<<nb, 256, 0, c->stream>>>(n, nb, par, c->d_part, c->d_p, c->d_q, c->d_dinv, x, c->d_r, c->d_z,
                                                   c->d_part + nb, c->d_sc);
@@ -396,7 +396,7 @@ void vd_build_solve(hdg_ctx* c, GraphBuild& gb, cudaGraph_t G, std::vector<cudaG
       for (int par = 0; par < 2; ++par) {
         vd_apply64(c, c->d_p, c->d_slot, &c->d_sc->done, -1);
         c->n_launch += 3;
-        vd_face_q_kernel<double><<<nb, 256, 0, c->stream>>>(n, c->sgn, c->vd->d_dslot, c->d_slot, c->d_p, c->d_q,
+        vd_face_q_kernel<<<nb, 256, 0, c->stream>>>(n, c->sgn, c->vd->d_dslot, c->d_slot, c->d_p, c->d_q,
                                                             c->d_part, c->d_sc);
         cg_update_kernel<<<nb, 256, 0, c->stream>>>(n, nb, par, c->d_part, c->d_p, c->d_q, c->d_dinv, x, c->d_r, c->d_z,
                                                     c->d_part + nb, c->d_sc);

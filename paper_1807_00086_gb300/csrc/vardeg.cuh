@@ -345,23 +345,20 @@ static __global__ void vd_cg_init_kernel(int64_t n, double sgn, const int32_t* _
   s = block_sum256(bb, red); if (threadIdx.x == 0) part[blockIdx.x * 3 + 2] = s;
 }
 
-// q = sgn K p through the slots; partial p.q (FP64, or compensated FP32 for float vectors)
-template <typename TV>
-__global__ void __launch_bounds__(256) vd_face_q_kernel(int64_t n, TV sgn, const int32_t* __restrict__ dslot,
-                                                        const TV* __restrict__ slot, const TV* __restrict__ p,
-                                                        TV* __restrict__ q, double* __restrict__ part,
-                                                        const CgScal* __restrict__ sc) {
+// q = sgn K p through the slots; partial p.q
+static __global__ void __launch_bounds__(256) vd_face_q_kernel(int64_t n, double sgn, const int32_t* __restrict__ dslot,
+                                                               const double* __restrict__ slot,
+                                                               const double* __restrict__ p, double* __restrict__ q,
+                                                               double* __restrict__ part, const CgScal* __restrict__ sc) {
   if (sc->done) return;
   __shared__ double red[8];
   double pq = 0.0;
-  Acc2 pq32;
   for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n; d += (int64_t)gridDim.x * blockDim.x) {
-    const TV qv = dslot[2 * d] >= 0 ? sgn * vd_sum(dslot, slot, d) : TV(0);
+    const double qv = dslot[2 * d] >= 0 ? sgn * vd_sum(dslot, slot, d) : 0.0;
     q[d] = qv;
-    if (sizeof(TV) == 8) pq += (double)p[d] * (double)qv;
-    else pq32.dot((float)p[d], (float)qv);
+    pq += p[d] * qv;
   }
-  const double s = block_sum256(sizeof(TV) == 8 ? pq : pq32.value(), red);
+  const double s = block_sum256(pq, red);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
