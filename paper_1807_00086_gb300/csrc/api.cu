@@ -203,8 +203,8 @@ void launch_update_f32(hdg_ctx* c, int par) {
   cg32_update_f_kernel<Q, false><<<c->nb_red, 256, 0, c->stream>>>(
       c->nfe4 / 4, (float)c->sgn, par, Q{c->sk.nf * c->Nf, (const int2*)c->d_face_slot, c->d_face_bnd}, c->d_slot32,
       (float4*)c->d_p32,
-      (const float4*)c->d_dinv32, (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32, c->d_pq, c->d_part + c->nb_red,
-      c->d_sc, Cg2Args{});
+      (const float4*)c->d_dinv32, (float4*)c->d_x32, (float4*)c->d_r32, (float4*)c->d_z32, c->d_pq,
+      (float2*)(c->d_part + c->nb_red), c->d_sc, Cg2Args{});
 }
 template <class L>
 void launch_update_two_l(hdg_ctx* c, const Cg2Args& o) {
@@ -350,8 +350,9 @@ void inner32_iter(hdg_ctx* c, bool use16, int par, int dev, cudaGraphConditional
   HDG_DISPATCH(c, launch_apply16, c, c->d_p32, c->d_slot32, &c->d_sc->done, iter);
   c->n_launch += 2;
   HDG_DISPATCH(c, launch_update_f32, c, par);
-  cg32_direction_kernel<<<c->nb_red, 256, 0, c->stream>>>(c->nfe4 / 4, c->nb_red, par, iter, c->d_part + c->nb_red,
-                                                          (const float4*)c->d_z32, (float4*)c->d_p32, c->d_sc, c->opt.maxit, h);
+  cg32_direction_kernel<float2><<<c->nb_red, 256, 0, c->stream>>>(
+      c->nfe4 / 4, c->nb_red, par, iter, (const float2*)(c->d_part + c->nb_red), (const float4*)c->d_z32, (float4*)c->d_p32,
+      c->d_sc, c->opt.maxit, h);
 }
 
 // ---- continuous traces (IEDG / EDG): expansion lam = R mu and restriction R^T (face weights)
@@ -734,8 +735,8 @@ hdg_status edg_mixed_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solve_
       edg_update32_kernel<<<nb, 256, 0, c->stream>>>(n, (float)c->sgn, c->d_node_ptr, c->d_node_inc, c->d_w32, c->d_p32,
                                                      c->d_dinv32, c->d_x32, c->d_r32, c->d_z32, par, c->d_pq, c->d_part,
                                                      c->d_sc);
-      cg32_direction_kernel<<<nb, 256, 0, c->stream>>>(n4, nb, par, -1, c->d_part, (const float4*)c->d_z32,
-                                                       (float4*)c->d_p32, c->d_sc, maxit, h);
+      cg32_direction_kernel<double><<<nb, 256, 0, c->stream>>>(n4, nb, par, -1, c->d_part, (const float4*)c->d_z32,
+                                                               (float4*)c->d_p32, c->d_sc, maxit, h);
     }
   };
   auto build = [&](GraphBuild& gb, cudaGraph_t G, hdg_ctx::DevGraph& dg) {

@@ -242,6 +242,15 @@ __device__ __forceinline__ double reduce_partials(const double* __restrict__ par
   return bc;
 }
 
+// a / b by one thread for the CTA (once per kernel): by every thread of a full SM an FP64 division takes
+// about 4 us of its FP64 pipe
+__device__ __forceinline__ double cta_ratio(double a, double b) {
+  __shared__ double r;
+  if (threadIdx.x == 0) r = a / b;
+  __syncthreads();
+  return r;
+}
+
 // Scalars of an FP32 inner solve whose iteration is two kernels: A multiplies every element block by
 // its direction p_K = z_K + beta p_K, formed in the gather, and leaves block partials of (p, S p);
 // B forms alpha from them, advances p, x, r, z and leaves partials of (r, z) and (r, r), from which
@@ -366,7 +375,7 @@ static __global__ void cg_update_kernel(int64_t n, int nb, int parity, const dou
   if (sc->done) return;
   __shared__ double red[8];
   const double pq = reduce_partials(part_pq, nb, 1, red);
-  const double al = sc->rho[parity] / pq;
+  const double al = cta_ratio(sc->rho[parity], pq);
   double rz = 0, rr = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -416,7 +425,7 @@ static __global__ void cg_direction_kernel(int64_t n, int nb, int parity, int it
   // with a host index no block reads what block 0 writes; on the device only block 0 uses it
   const int it = iter >= 0 ? iter + 1 : sc->iters + 1;
   if (!conv && (iter < 0 || it < maxit)) {
-    const double be = rz / sc->rho[parity];
+    const double be = cta_ratio(rz, sc->rho[parity]);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (; t + 3 * stride < n; t += 4 * stride) {
@@ -1231,7 +1240,7 @@ __global__ void __launch_bounds__(256, 3) cg32_update_f_kernel(int64_t n4, float
                                                                const float4* __restrict__ dinv, float4* __restrict__ x,
                                                                float4* __restrict__ r, float4* __restrict__ z,
                                                                const double* __restrict__ pq_in,
-                                                               double* __restrict__ part, const CgScal* __restrict__ sc,
+                                                               float2* __restrict__ part, const CgScal* __restrict__ sc,
                                                                Cg2Args o2) {
   constexpr int U = TWO ? 1 : 2;
   if constexpr (!TWO) {
@@ -1265,8 +1274,8 @@ __global__ void __launch_bounds__(256, 3) cg32_update_f_kernel(int64_t n4, float
     al = pair_ratio(rho, make_float2(sgn * pq[0].s, sgn * pq[0].c));
     first = k == 0;
   } else {
-    al = (float)(sc->rho[parity] / *pq_in);
     load();
+    al = (float)cta_ratio(sc->rho[parity], *pq_in);
   }
   Acc2 a[2];   // (r, z), (r, r)
   while (t < n4) {
@@ -1291,26 +1300,48 @@ __global__ void __launch_bounds__(256, 3) cg32_update_f_kernel(int64_t n4, float
   }
   block_pairs<2, 8>(a);
   if (threadIdx.x < 2) {
-    if constexpr (TWO) o2.partB[threadIdx.x * gridDim.x + blockIdx.x] = make_float2(a[threadIdx.x].s, a[threadIdx.x].c);
-    else part[blockIdx.x * 2 + threadIdx.x] = a[threadIdx.x].value();
+    float2* o = TWO ? o2.partB : part;
+    o[threadIdx.x * gridDim.x + blockIdx.x] = make_float2(a[threadIdx.x].s, a[threadIdx.x].c);
   }
 }
 
-// as cg_direction_kernel, FP32 vectors (float4)
-static __global__ void cg32_direction_kernel(int64_t n4, int nb, int parity, int iter, const double* __restrict__ part,
-                                      const float4* __restrict__ z, float4* __restrict__ p, CgScal* sc, int maxit,
-                                      cudaGraphConditionalHandle h) {
+// as cg_direction_kernel, FP32 vectors (float4). PART: double (interleaved sums), or float2 (compensated
+// pairs [2][nb], as in the two-kernel iteration): the FP64 sums of every CTA and a division in every
+// thread were most of this kernel's time, 196,608 tets, k = 3: 11.7 us, now 7.8 us
+template <class PART>
+__global__ void __launch_bounds__(256) cg32_direction_kernel(int64_t n4, int nb, int parity, int iter,
+                                                             const PART* __restrict__ part, const float4* __restrict__ z,
+                                                             float4* __restrict__ p, CgScal* sc, int maxit,
+                                                             cudaGraphConditionalHandle h) {
   if (sc->done) {
     if (iter < 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
     return;
   }
-  __shared__ double red[8];
-  const double rz = reduce_partials(part + 0, nb, 2, red);
-  const double rr = reduce_partials(part + 1, nb, 2, red);
+  __shared__ double rzs, rrs;
+  __shared__ float bes;
+  if constexpr (std::is_same<PART, float2>::value) {
+    Acc2 a[2];
+    sum_pairs<2, 8>(part, nb, a);
+    if (threadIdx.x == 0) {
+      rzs = a[0].value();
+      rrs = a[1].value();
+    }
+  } else {
+    __shared__ double red[8];
+    const double rz0 = reduce_partials(part + 0, nb, 2, red);
+    const double rr0 = reduce_partials(part + 1, nb, 2, red);
+    if (threadIdx.x == 0) {
+      rzs = rz0;
+      rrs = rr0;
+    }
+  }
+  if (threadIdx.x == 0) bes = (float)(rzs / sc->rho[parity]);
+  __syncthreads();
+  const double rz = rzs, rr = rrs;
   const bool conv = rr <= sc->tol2;
   const int it = iter >= 0 ? iter + 1 : sc->iters + 1;
   if (!conv && (iter < 0 || it < maxit)) {
-    const float be = (float)(rz / sc->rho[parity]);
+    const float be = bes;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (; t + 3 * stride < n4; t += 4 * stride) {
@@ -1342,8 +1373,8 @@ static __global__ void refine_residual_kernel(int64_t nf, int NF, double sgn, co
   const int64_t n = nf * NF;
   double rr = 0, bb = 0;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t f = t / NF;
-    const int mm = (int)(t % NF);
+    const uint32_t f = (uint32_t)t / (uint32_t)NF;   // n < 2^32
+    const int mm = (int)((uint32_t)t - f * (uint32_t)NF);
     double v = 0.0;
     if (face_bnd[f] < 0) {
       const double bv = b[t];
@@ -1384,10 +1415,10 @@ static __global__ void to32_scaled_kernel(int64_t n, const double* __restrict__ 
 static __global__ void refine_update_kernel(int64_t nf, int NF, const int32_t* __restrict__ face_bnd,
                                      const float* __restrict__ delta, const RefScal* __restrict__ rs,
                                      double* __restrict__ lam) {
-  const double inv = 1.0 / rs->scale;
-  const int64_t n = nf * NF;
+  const double inv = cta_ratio(1.0, rs->scale);
+  const int64_t n = nf * NF;   // < 2^32
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-    if (face_bnd[t / NF] < 0) lam[t] += (double)delta[t] * inv;
+    if (face_bnd[(uint32_t)t / (uint32_t)NF] < 0) lam[t] += (double)delta[t] * inv;
 }
 
 static __global__ void to32_kernel(int64_t n, const double* __restrict__ a, float* __restrict__ b) {

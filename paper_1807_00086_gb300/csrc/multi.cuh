@@ -1364,18 +1364,22 @@ static __global__ void mto32_scaled4_kernel(int64_t n4, int R, const double2* __
 }
 
 // lam += delta |rho|_j (|rho|_j = 1 / scale_j) on interior entries of the columns still refined
-// (scale_j != 0), four columns per thread. The reciprocal is taken once per thread: an FP64
-// division per entry made this kernel FP64-ALU-bound (8x its streaming time).
+// (scale_j != 0), four columns per thread. The reciprocals are taken once per CTA (R <= 256 of them): an
+// FP64 division per entry made this kernel FP64-ALU-bound (8x its streaming time), and four per thread
+// still did for narrow blocks (16,464 tets, k = 3, four columns: 24.6 us, now 11.1 us).
 static __global__ void mrefine_update4_kernel(int64_t n4, int R, int NF, const int32_t* __restrict__ face_bnd,
                                               const float4* __restrict__ delta, const double* __restrict__ scale,
                                               double2* __restrict__ lam) {
   const int R4 = R >> 2, lg = __ffs(R4) - 1, jq = threadIdx.x & (R4 - 1);
+  __shared__ double inv[256];
+  if (threadIdx.x < R) {
+    const double sc = scale[threadIdx.x];
+    inv[threadIdx.x] = sc != 0.0 ? 1.0 / sc : 0.0;
+  }
+  __syncthreads();
   double s[4];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const double sc = scale[4 * jq + c];
-    s[c] = sc != 0.0 ? 1.0 / sc : 0.0;
-  }
+  for (int c = 0; c < 4; ++c) s[c] = inv[4 * jq + c];
   if (s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0 && s[3] == 0.0) return;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
     if (face_bnd[(uint32_t)(t >> lg) / (uint32_t)NF] >= 0) continue;

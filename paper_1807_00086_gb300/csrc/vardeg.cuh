@@ -384,7 +384,7 @@ static __global__ void vd_refine_residual_kernel(int64_t n, double sgn, const in
 
 static __global__ void vd_refine_update_kernel(int64_t n, const int32_t* __restrict__ dslot, const float* __restrict__ delta,
                                         const RefScal* __restrict__ rs, double* __restrict__ lam) {
-  const double inv = 1.0 / rs->scale;
+  const double inv = cta_ratio(1.0, rs->scale);
   for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n; d += (int64_t)gridDim.x * blockDim.x)
     if (dslot[2 * d] >= 0) lam[d] += (double)delta[d] * inv;
 }
