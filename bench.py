@@ -471,8 +471,8 @@ def run_ours(args):
         pm = ev0.elapsed_time(ev1) / 5
         d, Np, Nf = s.dim, s.Np, s.Nf
         na = math.comb(s.k + 1 + d, d) - 1
-        fl = (2 * d * Np * (d * Np + (d + 1) * Nf) + 2 * na * d * d * Np + d * d * na * (na + 1)
-              + na ** 3 / 3 + 2 * na * na)
+        fl = (2 * d * Np * Np + 2 * (d + 1) * Np * Nf + 2 * Np * d * (2 * d + 1) + 2 * na * d * Np
+              + d * (d + 1) // 2 * na * (na + 1) + na ** 3 / 3 + 2 * na * na)
         ach_p = fl * ne / (pm / 1e3) / 1e12
         post = {"kernel": "post_kernel<%d,%d> (p* in P_%d: discrete gradient, local Neumann problem, Cholesky)"
                 % (d, s.k, s.k + 1), "launch_ms": pm, "flops_per_elem": fl, "achieved_tflops": ach_p,
@@ -515,12 +515,13 @@ def run_ours(args):
             f16 = st.get("apply16_launches", 0) > 0
             a32 = (st["apply16_ms"] / st["apply16_launches"]) if f16 else \
                 st["apply32_ms"] / max(1, st["apply32_launches"])
-            byt = (nschur * 2 + ne * 4 if f16 else nschur * 4) + 2 * nslot * 4
+            npack = packed_entries(w["elem"], w["elem_k"])
+            byt = (npack * 2 + ne * 4 if f16 else npack * 4) + 2 * nslot * 4
             ach = byt / (a32 / 1e3) / 1e9
             roof = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                     "frac": ach / peaks["hbm_gbs"], "traffic": None,
-                    "kernel": ("apply_vd_kernel<float, __half> (compact FP16 S_K, per-element scale)" if f16 else
-                               "apply_vd_kernel<float> (compact FP32 S_K, per-element m_K)"),
+                    "kernel": "sym_apply_two_kernel<SymIdxVd, %s> (packed symmetric S_K, 16 x 16 units)"
+                              % ("__half" if f16 else "float"),
                     "peak_source": src + " (hbm_gbs: copy)",
                     "bytes_per_launch": byt, "launch_ms": a32,
                     "launches": st["apply16_launches"] if f16 else st["apply32_launches"],
@@ -530,21 +531,25 @@ def run_ours(args):
             if st.get("applydf_launches"):
                 adf = st["applydf_ms"] / st["applydf_launches"]
                 roof["df_refinement_apply"] = {
-                    "kernel": "apply_vd_df_kernel (double-float hi + lo compact S_K)", "launches": st["applydf_launches"],
-                    "launch_ms": adf, "bytes_per_launch": nschur * 8 + nslot * 16,
-                    "achieved_gbs": (nschur * 8 + nslot * 16) / (adf / 1e3) / 1e9}
+                    "kernel": "sym_apply_df_kernel<SymIdxVd> (packed symmetric S_K, hi + lo)",
+                    "launches": st["applydf_launches"],
+                    "launch_ms": adf, "bytes_per_launch": npack * 8 + nslot * 16,
+                    "achieved_gbs": (npack * 8 + nslot * 16) / (adf / 1e3) / 1e9}
         else:
             ach = 2 * nschur / (apply_avg_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": ach, "peak": 1.25, "unit": "TFLOP/s", "frac": ach / 1.25,
-                    "traffic": None, "kernel": "apply_vd_kernel<double> (compact FP64 S_K)",
+                    "traffic": None, "kernel": "apply_vd_kernel (compact FP64 S_K)",
                     "peak_source": "nominal GB300 FP64 1.25 TFLOP/s", "flops_per_launch": 2 * nschur,
                     "launch_ms": apply_avg_ms, "launches": st["apply_launches"]}
     elif elastic and args.prec != "fp64":
         a32 = st["apply32_ms"] / max(1, st["apply32_launches"])
-        bytes_el = m * m * 4 + 2 * m * 4
+        units = sym_units(m) * 256
+        packed = units < m * m   # the library's rule for the packed symmetric copy
+        bytes_el = (units if packed else m * m) * 4 + 2 * m * 4
         ach = bytes_el * ne / (a32 / 1e3) / 1e9
         roof = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": ach / peaks["hbm_gbs"],
-                "traffic": None, "kernel": "apply32f_kernel<ElDims<3,%d>> (FP32 S_K %dx%d)" % (args.k, m, m),
+                "traffic": None, "kernel": ("sym_apply_two_kernel<SymIdxUni<ElDims<3,%d>>, float> (packed symmetric S_K)" % args.k
+                                           if packed else "apply32f_kernel<ElDims<3,%d>> (FP32 S_K %dx%d)" % (args.k, m, m)),
                 "bytes_per_elem": bytes_el, "launch_ms": a32, "launches": st["apply32_launches"],
                 "fp64_refinement_apply": fp64_view}
 
@@ -623,6 +628,24 @@ def run_ours(args):
         print(json.dumps(out), flush=True)
     if dist is not None:
         dist.destroy_process_group()
+
+
+def sym_units(m):
+    """16 x 16 units on and above the diagonal of an m x m block."""
+    nb = (np.asarray(m) + 15) // 16
+    return nb * (nb + 1) // 2
+
+
+def packed_entries(elem, ek):
+    """Entries of the packed symmetric S_K copies of a mesh with per-element degrees ek: element
+    block sizes m_K = sum over faces of 3 N_f(k_F), k_F the larger degree of a face's elements."""
+    faces = np.sort(np.stack([np.delete(elem, j, axis=1) for j in range(4)], axis=1).reshape(-1, 3), axis=1)
+    _, inv = np.unique(faces, axis=0, return_inverse=True)
+    inv = inv.reshape(-1)
+    kf = np.zeros(inv.max() + 1, dtype=np.int64)
+    np.maximum.at(kf, inv, np.repeat(np.asarray(ek, dtype=np.int64), 4))
+    m = (3 * (kf + 1) * (kf + 2) // 2)[inv].reshape(-1, 4).sum(axis=1)
+    return int(sym_units(m).sum()) * 256
 
 
 def svk_condense_flops(k):
