@@ -45,10 +45,18 @@ void launch_condense(hdg_ctx* c) {
     return;
   }
   using C = CondCfg<DIM, K>;
-  cudaFuncSetAttribute(condense_kernel<DIM, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-  condense_kernel<DIM, K><<<(unsigned)((c->sk.ne + C::EPW - 1) / C::EPW), 32, C::SMEM, c->stream>>>(
-      devmesh(c), CondTabs{c->d_condtab, c->tabs.Ff, c->tabs.DFrf, c->tabs.Pfg}, c->alpha, c->tau, c->d_S, c->d_Hinv,
-      c->d_err);
+  if (c->sk.ne <= (int64_t)cond_cta_per_sm<DIM, K>() * c->sms) {
+    condense_cta_kernel<DIM, K><<<(unsigned)c->sk.ne, 128, 0, c->stream>>>(devmesh(c), c->tabs, c->alpha, c->tau, c->d_S,
+                                                                          c->d_Hinv, c->d_err, c->d_co64, c->d_codf);
+  } else {
+    c->n_launch += 1;
+    if (c->d_co64) local_co_kernel<ArF64><<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_co64);
+    else if (c->d_codf) local_co_kernel<ArDf><<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_codf);
+    cudaFuncSetAttribute(condense_kernel<DIM, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    condense_kernel<DIM, K><<<(unsigned)((c->sk.ne + C::EPW - 1) / C::EPW), 32, C::SMEM, c->stream>>>(
+        devmesh(c), CondTabs{c->d_condtab, c->tabs.Ff, c->tabs.DFrf, c->tabs.Pfg}, c->alpha, c->tau, c->d_S, c->d_Hinv,
+        c->d_err);
+  }
   diag_kernel<Dims<DIM, K>><<<grid_for(c, c->sk.nf * c->Nf), 256, 0, c->stream>>>(devmesh(c), c->d_S, c->sgn, c->d_dinv);
 }
 
@@ -411,10 +419,6 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
   HDG_DISPATCH(c, launch_condense, c);
   hdg_status s = check_launch(c, "condense");
   if (s) return s;
-  if (c->d_co64) {
-    c->n_launch += 1;
-    local_co_kernel<ArF64><<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_co64);
-  }
   if (c->opt.prec != HDG_FP64) {
     if (c->d_S32lo) {
       HDG_DISPATCH(c, launch_sym_pack, c);
@@ -431,8 +435,7 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
         if (c->d_S16) HDG_DISPATCH(c, prepare_apply16, c);
       }
       const int64_t nH = c->sk.ne * (int64_t)c->nv * c->nv;
-      c->n_launch += 2;
-      local_co_kernel<ArDf><<<grid_for(c, c->sk.ne), 256, 0, c->stream>>>(devmesh(c), c->alpha, c->d_codf);
+      c->n_launch += 1;
       to_df_kernel<<<grid_for(c, nH), 256, 0, c->stream>>>(nH, c->d_Hinv, c->d_Hinvdf);
     }
     const int64_t nfe = c->sk.nf * c->Nf;

@@ -207,6 +207,132 @@ __global__ void __launch_bounds__(32) condense_kernel(DevMesh mesh, CondTabs T, 
   }
 }
 
+// The same for small meshes: one CTA of four warps per element, which also writes the coefficients of the
+// local solves (local_co_kernel). A warp of condense_kernel that is alone on its SM partition takes 64 cycles
+// per FP64 instruction, for EPW elements, while other partitions are idle. hdg_condense with the read-back of S,
+// this kernel / condense_kernel: 162 tets, k = 2: 98 / 127 us, k = 4: 378 / 569 us; 750 tets, k = 2: 114 / 128,
+// k = 3: 224 / 307, k = 4: 652 / 616; 1,296 tets, k = 2: 145 / 131, k = 3: 335 / 333 us; 800 triangles: as fast.
+template <int DIM, int K>
+__host__ __device__ constexpr int cond_cta_per_sm() {
+  return DIM == 3 ? 2 * CondCfg<DIM, K>::EPW : 4;   // at most so many elements per SM
+}
+template <int DIM, int K>
+__global__ void __launch_bounds__(128) condense_cta_kernel(DevMesh mesh, Tabs T, double alpha, double tau,
+                                                          double* __restrict__ S, double* __restrict__ Hinv,
+                                                          int* __restrict__ err, double* __restrict__ co64,
+                                                          df2* __restrict__ codf) {
+  constexpr int NT = 128;
+  using D = Dims<DIM, K>;
+  constexpr int NP = D::NP, NF = D::NF, M = D::M, NFC = D::NFC;
+  __shared__ double H[NP * NP];
+  __shared__ double W[NP * M];
+  __shared__ double Li[NP * NP];
+  __shared__ double g[GEO_STRIDE];
+  __shared__ double Grs[DIM * DIM], Bfr[NFC * DIM], nn[NFC * NFC];
+  const int64_t e = blockIdx.x;
+  const int tid = threadIdx.x;
+  if (tid < GEO_STRIDE) g[tid] = mesh.geo[e * GEO_STRIDE + tid];
+  __syncthreads();
+  const double dJ = g[0];
+  const double rho = mesh.rho[e], cc = mesh.c[e];
+  const double a = alpha / (rho * cc * cc), b = alpha * rho;
+  if (tid == NT - 1) {
+    const double v[4] = {1.0 / b, a * dJ, b * dJ, 1.0 / (b * dJ)};
+    for (int i = 0; i < 4; ++i)
+      if (co64) co64[4 * e + i] = v[i];
+      else if (codf) codf[4 * e + i] = df_from(v[i]);
+  }
+  if (tid < DIM * DIM) {
+    int r = tid / DIM, s = tid % DIM;
+    double v = 0.0;
+    for (int j = 0; j < DIM; ++j) v += g[1 + r * DIM + j] * g[1 + s * DIM + j];
+    Grs[tid] = v;
+  } else if (tid < DIM * DIM + NFC * DIM) {
+    int t = tid - DIM * DIM, f = t / DIM, r = t % DIM;
+    double v = 0.0;
+    for (int j = 0; j < DIM; ++j) v += g[D::ON + f * DIM + j] * g[1 + r * DIM + j];
+    Bfr[t] = v;
+  } else if (tid < DIM * DIM + NFC * DIM + NFC * NFC) {
+    int t = tid - DIM * DIM - NFC * DIM, f = t / NFC, h = t % NFC;
+    double v = 0.0;
+    for (int j = 0; j < DIM; ++j) v += g[D::ON + f * DIM + j] * g[D::ON + h * DIM + j];
+    nn[t] = v;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < NP * NP; idx += NT) {
+    const int i = idx / NP, l = idx % NP;
+    double v = (i == l) ? a * dJ : 0.0;
+    double fe = 0.0;
+    for (int f = 0; f < NFC; ++f) fe += g[D::OJF + f] * T.Ef[(f * NP + i) * NP + l];
+    double dd = 0.0;
+    for (int rs = 0; rs < DIM * DIM; ++rs) dd += Grs[rs] * T.Trs[(rs * NP + i) * NP + l];
+    H[idx] = v + tau * fe + (dJ / b) * dd;
+    Li[idx] = (i == l) ? 1.0 : 0.0;
+  }
+  for (int idx = tid; idx < NP * M; idx += NT) {
+    const int i = idx / M, col = idx % M, f = col / NF, mm = col % NF;
+    double v = tau * T.Ff[(f * NP + i) * NF + mm];
+    double d2 = 0.0;
+    for (int r = 0; r < DIM; ++r) d2 += Bfr[f * DIM + r] * T.DFrf[((r * NFC + f) * NP + i) * NF + mm];
+    W[idx] = -g[D::OJF + f] * (v + d2 / b);
+  }
+  __syncthreads();
+  // Cholesky, right-looking, lower triangle in place
+  for (int j = 0; j < NP; ++j) {
+    if (tid == 0) {
+      double d = H[j * NP + j];
+      if (!(d > 0.0)) { atomicExch(err, 1); d = 1.0; }
+      H[j * NP + j] = sqrt(d);
+    }
+    __syncthreads();
+    for (int i = j + 1 + tid; i < NP; i += NT) H[i * NP + j] /= H[j * NP + j];
+    __syncthreads();
+    const int w = NP - j - 1;
+    for (int idx = tid; idx < w * w; idx += NT) {
+      const int i = j + 1 + idx / w, l = j + 1 + idx % w;
+      if (l <= i) H[i * NP + l] -= H[i * NP + j] * H[l * NP + j];
+    }
+    __syncthreads();
+  }
+  // forward substitution, one column per thread: W <- L^{-1} Bt, Li <- L^{-1}
+  for (int col = tid; col < M + NP; col += NT) {
+    if (col < M) {
+      for (int i = 0; i < NP; ++i) {
+        double s = W[i * M + col];
+        for (int l = 0; l < i; ++l) s -= H[i * NP + l] * W[l * M + col];
+        W[i * M + col] = s / H[i * NP + i];
+      }
+    } else {
+      const int c2 = col - M;
+      for (int i = c2; i < NP; ++i) {
+        double s = (i == c2) ? 1.0 : 0.0;
+        for (int l = c2; l < i; ++l) s -= H[i * NP + l] * Li[l * NP + c2];
+        Li[i * NP + c2] = s / H[i * NP + i];
+      }
+    }
+  }
+  __syncthreads();
+  double* Se = S + e * (int64_t)(M * M);
+  const double ib = 1.0 / (b * dJ);
+  for (int idx = tid; idx < M * M; idx += NT) {
+    const int ra = idx / M, cb = idx % M;
+    const int f = ra / NF, aa = ra % NF, h = cb / NF, bb = cb % NF;
+    double s = 0.0;
+    for (int i = 0; i < NP; ++i) s += W[i * M + ra] * W[i * M + cb];
+    if (ra == cb) s -= tau * g[D::OJF + f];
+    s -= ib * g[D::OJF + f] * g[D::OJF + h] * nn[f * NFC + h] * T.Pfg[((f * NFC + h) * NF + aa) * NF + bb];
+    Se[idx] = s;
+  }
+  double* He = Hinv + e * (int64_t)(NP * NP);
+  for (int idx = tid; idx < NP * NP; idx += NT) {
+    const int i = idx / NP, l = idx % NP;
+    const int q0 = i > l ? i : l;
+    double s = 0.0;
+    for (int q = q0; q < NP; ++q) s += Li[q * NP + i] * Li[q * NP + l];
+    He[idx] = s;
+  }
+}
+
 // Double-float copy of an FP64 array (H^{-1} after each condensation, the element geometry).
 static __global__ void to_df_kernel(int64_t n, const double* __restrict__ a, df2* __restrict__ out) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {

@@ -45,3 +45,27 @@ def test_partial_groups_schur_and_copies(dim, k, ne):
             ref = u
         for j in range(R):
             assert relerr(u if R == 1 else u[:, :, j], ref) < 1e-9, (prec, R, j)
+
+
+@pytest.mark.parametrize("dim,k", [(2, 2), (3, 1), (3, 3), (3, 4)])
+@pytest.mark.parametrize("over", [0, 1, 3])
+def test_either_side_of_the_small_mesh_rule(dim, k, over):
+    """The last meshes with a CTA per element (4 or 8 elements per SM), and the first whose elements share a warp
+    (partial last ones). The recovery checks the coefficients that either kernel leaves for the local solves."""
+    import torch
+    from paper_1807_00086_gb300 import hdg
+    ne = (8 if dim == 3 and k < 4 else 4) * torch.cuda.get_device_properties(0).multi_processor_count + over
+    vert, elem = mesh(dim, 20 if dim == 2 else 6)
+    elem = elem[:ne]
+    used, inv = np.unique(elem, return_inverse=True)
+    vert, elem = vert[used], inv.reshape(elem.shape).astype(np.int32)
+    rho, c = inputs.loguniform(ne, 0.5, 2.0, 3), inputs.loguniform(ne, 1.0, 3.0, 4)
+    prob = ac.build_problem(vert, elem, k, 1.0, rho, c)
+    cond = ac.condense(prob, 37.0)
+    s = hdg.Solver(vert, elem, k, 1.0, rho, c)
+    s.hdg_condense(37.0)
+    assert relerr(s.hdg_get_schur().cpu().numpy(), np.array(cond.S)) < 1e-12
+    F = inputs.random_state(ne, s.n, 11).reshape(ne, s.n)
+    lam = inputs.random_traces(s.n_faces, s.Nf, 5).reshape(s.n_faces, s.Nf)
+    u = s.hdg_recover(torch.tensor(F, device="cuda"), torch.tensor(lam, device="cuda")).cpu().numpy()
+    assert relerr(u, ac.recover(prob, cond, F, lam)) < 1e-12
