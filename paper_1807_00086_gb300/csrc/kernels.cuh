@@ -127,10 +127,15 @@ __global__ void __launch_bounds__(ApplyCfg<D>::NT) apply_kernel(DevMesh mesh, co
 }
 
 // ---------------------------------------------------------------- face passes and PCG
+// done: the stop code, for the kernels that follow and the host. halt[parity]: the same for the kernel of
+// the iteration with this parity that records the stop code. Its CTA 0 writes the other slot, so no CTA
+// reads what its own launch writes: read from `done`, the warps of a late CTA could disagree and part
+// at a barrier.
 struct CgScal {
   double rho[2];
   double bb, rr, tol2;
-  int done, iters, pad0, pad1;
+  int done, iters;
+  int halt[2];
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -330,7 +335,7 @@ static __global__ void cg_init_scalars(int nb, const double* __restrict__ part, 
     sc->tol2 = rtol * rtol * bb;
     sc->iters = 0;
     // a zero right-hand side ends the solve here (its solution is zero on interior faces)
-    sc->done = (bb == 0.0 || rr <= sc->tol2) ? 1 : 0;
+    sc->done = sc->halt[0] = sc->halt[1] = (bb == 0.0 || rr <= sc->tol2) ? 1 : 0;
     if (st) st->it[0] = st->it[1] = 0;
   }
 }
@@ -414,8 +419,11 @@ static __global__ void cg_update_kernel(int64_t n, int nb, int parity, const dou
 static __global__ void cg_direction_kernel(int64_t n, int nb, int parity, int iter, const double* __restrict__ part,
                                     const double* __restrict__ z, double* __restrict__ p, CgScal* sc, int maxit,
                                     cudaGraphConditionalHandle h) {
-  if (sc->done) {
-    if (iter < 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
+  if (sc->halt[parity]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      sc->halt[parity ^ 1] = 1;
+      if (iter < 0) cudaGraphSetConditional(h, 0u);
+    }
     return;
   }
   __shared__ double red[8];
@@ -443,7 +451,7 @@ static __global__ void cg_direction_kernel(int64_t n, int nb, int parity, int it
     sc->rr = rr;
     sc->iters = it;
     const int done = conv ? 1 : (it >= maxit ? 2 : 0);
-    if (done) sc->done = done;
+    if (done) sc->done = sc->halt[parity ^ 1] = done;
     if (iter < 0) cudaGraphSetConditional(h, done ? 0u : 1u);
   }
 }
@@ -530,12 +538,15 @@ __global__ void __launch_bounds__(ApplyTwoCfg<D>::NT) apply_two64_kernel(DevMesh
       pv = p[t];
     }
   }
-  const int over = o.sc->done, k = o.st->it[o.parity];
+  const int over = o.sc->halt[o.parity], k = o.st->it[o.parity];
   const double rho = o.sc->rho[o.parity], tol2 = o.sc->tol2;
   double a[2];
   partial_sums<2, C::NT>(o.partB, o.nb, a);   // at k = 0 for nothing
   if (over) {
-    if (o.dev && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(o.h, 0u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      o.sc->halt[o.parity ^ 1] = 1;
+      if (o.dev) cudaGraphSetConditional(o.h, 0u);
+    }
     return;
   }
   block_sums<2, C::NW>(a);
@@ -555,7 +566,7 @@ __global__ void __launch_bounds__(ApplyTwoCfg<D>::NT) apply_two64_kernel(DevMesh
       o.st->it[o.parity ^ 1] = k + 1;
       o.st->beta = beta;
       o.sc->iters = k;
-      if (done) o.sc->done = done;
+      if (done) o.sc->done = o.sc->halt[o.parity ^ 1] = done;
       if (o.dev) cudaGraphSetConditional(o.h, done ? 0u : 1u);
     }
   }
@@ -841,12 +852,15 @@ struct Cg2Args {
 template <int NW>
 __device__ __forceinline__ bool cg2_begin_a(const Cg2Args& o, float& beta, bool& first) {
   // everything is loaded before any of it is tested: at k = 0 the partials are loaded for nothing
-  const int over = o.sc->done, k = o.st->it[o.parity];
+  const int over = o.sc->halt[o.parity], k = o.st->it[o.parity];
   const float2 rho = o.st->rho[o.parity], t2 = o.st->tol2;
   Acc2 a[2];
   sum_pairs<2, NW>(o.partB, o.nb, a);
   if (over) {
-    if (o.dev && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(o.h, 0u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      o.sc->halt[o.parity ^ 1] = 1;
+      if (o.dev) cudaGraphSetConditional(o.h, 0u);
+    }
     return false;
   }
   first = k == 0;
@@ -864,7 +878,7 @@ __device__ __forceinline__ bool cg2_begin_a(const Cg2Args& o, float& beta, bool&
     o.st->it[o.parity ^ 1] = k + 1;
     o.st->beta = beta;
     o.sc->iters = k;
-    if (done) o.sc->done = done;
+    if (done) o.sc->done = o.sc->halt[o.parity ^ 1] = done;
     if (o.dev) cudaGraphSetConditional(o.h, done ? 0u : 1u);
   }
   return done == 0;
@@ -1138,7 +1152,7 @@ static __global__ void cg32_init_scalars(int nb, const float2* __restrict__ part
     sc->rho[0] = a[0].value(); sc->rho[1] = 0; sc->bb = rr; sc->rr = rr;
     sc->tol2 = t2;
     sc->iters = 0;
-    sc->done = (rr == 0.0) ? 1 : 0;
+    sc->done = sc->halt[0] = sc->halt[1] = (rr == 0.0) ? 1 : 0;
     st->rho[0] = st->rho[1] = make_float2(a[0].s, a[0].c);
     st->tol2 = make_float2((float)t2, (float)(t2 - (double)(float)t2));
     st->beta = 0.f;
@@ -1313,8 +1327,11 @@ __global__ void __launch_bounds__(256) cg32_direction_kernel(int64_t n4, int nb,
                                                              const PART* __restrict__ part, const float4* __restrict__ z,
                                                              float4* __restrict__ p, CgScal* sc, int maxit,
                                                              cudaGraphConditionalHandle h) {
-  if (sc->done) {
-    if (iter < 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
+  if (sc->halt[parity]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      sc->halt[parity ^ 1] = 1;
+      if (iter < 0) cudaGraphSetConditional(h, 0u);
+    }
     return;
   }
   __shared__ double rzs, rrs;
@@ -1358,7 +1375,7 @@ __global__ void __launch_bounds__(256) cg32_direction_kernel(int64_t n4, int nb,
     sc->rr = rr;
     sc->iters = it;
     const int done = conv ? 1 : (it >= maxit ? 2 : 0);
-    if (done) sc->done = done;
+    if (done) sc->done = sc->halt[parity ^ 1] = done;
     if (iter < 0) cudaGraphSetConditional(h, done ? 0u : 1u);
   }
 }

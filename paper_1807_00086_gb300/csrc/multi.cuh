@@ -588,7 +588,7 @@ struct Cg2MState {
   float2 rho[2][kTwoR], tol2[kTwoR];
   float beta[kTwoR];
   int conv[2][kTwoR];
-  int it[2];
+  int it[2], halt[2];   // halt: as in CgScal
 };
 struct Cg2MArgs {
   MScal sc;
@@ -642,13 +642,16 @@ template <int NW>
 __device__ __forceinline__ bool cg2m_begin_a(const Cg2MArgs& o, float* be, bool& first) {
   __shared__ int running;
   // loaded before any of it is tested, as in cg2_begin_a
-  const int over = *o.sc.done, k = o.st->it[o.parity], j = threadIdx.x;
+  const int over = o.st->halt[o.parity], k = o.st->it[o.parity], j = threadIdx.x;
   first = k == 0;
   if (j == 0) running = 0;
   Acc2 a[2];
   sum_pairs_cols<2, NW>(o.partB, o.nb, o.R, a);
   if (over) {
-    if (o.dev && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(o.h, 0u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      o.st->halt[o.parity ^ 1] = 1;
+      if (o.dev) cudaGraphSetConditional(o.h, 0u);
+    }
     return false;
   }
   if (j < o.R) {
@@ -676,7 +679,7 @@ __device__ __forceinline__ bool cg2m_begin_a(const Cg2MArgs& o, float* be, bool&
   if (blockIdx.x == 0 && j == 0) {
     o.st->it[o.parity ^ 1] = k + 1;
     *o.sc.iters = k;
-    if (done) *o.sc.done = done;
+    if (done) *o.sc.done = o.st->halt[o.parity ^ 1] = done;
     if (o.dev) cudaGraphSetConditional(o.h, done ? 0u : 1u);
   }
   return done == 0;
@@ -1471,6 +1474,7 @@ static __global__ void mcols_init(int nb, int R, double rtol, int tol_from_rr, c
   __syncthreads();
   if (threadIdx.x == 0) {
     *sc.done = notconv == 0 ? 1 : 0;
+    if (st) st->halt[0] = st->halt[1] = *sc.done;
     *sc.iters = 0;
   }
 }
