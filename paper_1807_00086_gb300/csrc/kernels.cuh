@@ -784,8 +784,10 @@ struct PqOut {
   DevTiming* timing;  // may be null
 };
 
-__device__ __forceinline__ void timing_start(const PqOut& o) {
-  if (o.timing && o.part && threadIdx.x == 0) atomicMin(&o.timing->start_ns, global_ns());
+// t: global_ns() at the start of the CTA, in thread 0. A launch that may still turn out to have nothing to
+// do stamps once it is known to be a live one.
+__device__ __forceinline__ void timing_start(const PqOut& o, unsigned long long t) {
+  if (o.timing && o.part && threadIdx.x == 0) atomicMin(&o.timing->start_ns, t);
 }
 
 // A kernel that leaves its partials to the next one still counts its CTAs for the launch timing.
@@ -913,8 +915,8 @@ __global__ void __launch_bounds__(128, 4) apply32_kernel(int64_t ne, const int32
   __shared__ float tr[4][32 * MP];
   if constexpr (!TWO) {
     if (done && *done) return;
+    timing_start(pqo, global_ns());
   }
-  timing_start(pqo);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t g0 = (int64_t)blockIdx.x * 4 + wid;
   const bool wact = g0 * 32 < ne;                 // the last block may hold idle warps
@@ -936,7 +938,9 @@ __global__ void __launch_bounds__(128, 4) apply32_kernel(int64_t ne, const int32
   if constexpr (TWO) {
     float beta;
     bool first;
+    const unsigned long long t0 = threadIdx.x == 0 ? global_ns() : 0ull;
     if (!cg2_begin_a<4>(o2, beta, first)) return;   // while the gather is in flight
+    timing_start(pqo, t0);
 #pragma unroll
     for (int r = 0; r < M; ++r) xl[r] = cg2_dir(first, beta, y[r], xl[r]);
   }
@@ -1039,7 +1043,7 @@ __global__ void __launch_bounds__(128, 4) apply16_kernel(int64_t ne, const int32
   constexpr int NF = D::NF, M = D::M, NFC = D::NFC, P8 = PK::P8, XS = C::XS, MP = C::MP, CPB = C::CPB;
   extern __shared__ __align__(16) float a16sm[];
   if (done && *done) return;
-  timing_start(pqo);
+  timing_start(pqo, global_ns());
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float* t = a16sm + wid * 32 * (XS + MP) + 32 * XS;
   const unsigned xrow = (unsigned)__cvta_generic_to_shared(a16sm + wid * 32 * (XS + MP) + lane * XS);
