@@ -132,21 +132,11 @@ SymIdxUni<ElDims<DIM, K>> sym_idx(const hdg_ctx* c) {
   return {c->d_elem_face, c->d_face_bnd};
 }
 
-// FP64-accurate elastic residual apply from the packed double-float copy
-template <int DIM, int K>
-void launch_apply_sym_df(hdg_ctx* c, const double* x, double* zslot) {
-  c->n_launch += 1;
-  cudaEvent_t stop = apply_begin(c, 2, -1);
-  sym_apply_df_kernel<<<(unsigned)((c->sk.ne + 3) / 4), 128, 0, c->stream>>>(c->sk.ne, sym_idx<DIM, K>(c), c->d_S32,
-                                                                             c->d_S32lo, x, zslot);
-  apply_end(c, stop);
-}
-
 template <int DIM, int K>
 void launch_sym_pack(hdg_ctx* c) {
   c->n_launch += 1;
   sym_pack_kernel<<<(unsigned)std::min<int64_t>(c->sk.ne, 1 << 20), 256, 0, c->stream>>>(
-      c->sk.ne, sym_idx<DIM, K>(c), c->d_S, (float4*)c->d_S32, (float4*)c->d_S32lo, (uint4*)nullptr, (float*)nullptr);
+      c->sk.ne, sym_idx<DIM, K>(c), c->d_S, (float4*)c->d_S32, (float4*)nullptr, (uint4*)nullptr, (float*)nullptr);
 }
 
 // one FP64 iteration; dev != 0: device-driven loop with condition h. Two kernels where A's CTAs are at most
@@ -331,7 +321,7 @@ template <int DIM, int K>
 void launch_apply_two(hdg_ctx* c, const Cg2Args& o, int iter) {
   c->n_launch += 1;
   cudaEvent_t stop = apply_begin(c, 1, iter);
-  if (c->d_S32lo)
+  if (c->sym32)
     sym_apply_two_kernel<<<(unsigned)o.na, 128, 0, c->stream>>>(c->sk.ne, sym_idx<DIM, K>(c), c->d_S32, (const float*)nullptr,
                                                                 c->d_z32, c->d_p32, c->d_slot32, o);
   else if (c->phys == HDG_ELASTIC)
@@ -420,7 +410,7 @@ hdg_status do_condense(hdg_ctx* c, double alpha) {
   hdg_status s = check_launch(c, "condense");
   if (s) return s;
   if (c->opt.prec != HDG_FP64) {
-    if (c->d_S32lo) {
+    if (c->sym32) {
       HDG_DISPATCH(c, launch_sym_pack, c);
     } else if (c->phys == HDG_ELASTIC) {
       const int64_t nS = c->sk.ne * (int64_t)c->m * c->m;
@@ -513,8 +503,6 @@ hdg_status solve_mixed(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info
   for (int sweep = 0;; ++sweep) {
     if (c->d_Sdf) {
       HDG_DISPATCH(c, launch_apply_df, c, x, c->d_slot);
-    } else if (c->d_S32lo) {
-      HDG_DISPATCH(c, launch_apply_sym_df, c, x, c->d_slot);
     } else {
       HDG_DISPATCH(c, launch_apply, c, x, c->d_slot, (const int*)nullptr);
     }
@@ -629,8 +617,6 @@ hdg_status solve_mixed_graph(hdg_ctx* c, const double* bvec, double* x, hdg_solv
     gb.seq(B, bd, [&] {
       if (c->d_Sdf) {
         HDG_DISPATCH(c, launch_apply_df, c, x, c->d_slot, skip);
-      } else if (c->d_S32lo) {
-        HDG_DISPATCH(c, launch_apply_sym_df, c, x, c->d_slot);
       } else {
         HDG_DISPATCH(c, launch_apply, c, x, c->d_slot, (const int*)nullptr, -1);
       }
@@ -2068,11 +2054,10 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
     const int P4 = (c->m * (c->m + 1) / 2 + 3) / 4;
     // elastic: packed copies where they are smaller; an SVK step copies S_K in every Newton iteration
     // and applies it a few times only
-    const bool sym = c->phys == HDG_ELASTIC && !svk && sym_pays(c->m);
-    const size_t nS32 = sym ? (size_t)ne * sym_units(c->m) * 256
-                            : c->phys == HDG_ELASTIC ? (size_t)ne * c->m * c->m : (size_t)ngroups * P4 * 128;
+    c->sym32 = c->phys == HDG_ELASTIC && !svk && sym_pays(c->m);
+    const size_t nS32 = c->sym32 ? (size_t)ne * sym_units(c->m) * 256
+                        : c->phys == HDG_ELASTIC ? (size_t)ne * c->m * c->m : (size_t)ngroups * P4 * 128;
     if ((s = dalloc(c, &c->d_S32, nS32))) return s;
-    if (sym && (s = dalloc(c, &c->d_S32lo, nS32))) return s;
     // element slots (whole 32-element groups) plus one zero slot past the last element (the
     // missing neighbour of an SVK traction face)
     if ((s = dalloc(c, &c->d_slot32, (size_t)ngroups * c->m * 32 + c->Nf))) return s;

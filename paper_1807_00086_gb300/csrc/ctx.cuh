@@ -66,7 +66,7 @@ struct hdg_ctx {
   int tcp_per_sm = 1;           // resident CTAs per SM of the persistent tensor-core column-block apply
   // mixed precision
   float *d_S32 = nullptr, *d_dinv32 = nullptr, *d_slot32 = nullptr;
-  float* d_S32lo = nullptr;     // elastic: remainder of the packed FP32 copy (symapply.cuh); set where that is used
+  bool sym32 = false;           // elastic, one degree: d_S32 is the packed copy of symapply.cuh
   float* d_Sdf = nullptr;       // double-float diagonal-major copy of S_K (refinement apply)
   // double-float local solves: H^{-1}, geometry, coefficients at the mass shift, reference tables
   df2 *d_Hinvdf = nullptr, *d_geodf = nullptr, *d_codf = nullptr;

@@ -177,9 +177,12 @@ __global__ void __launch_bounds__(128, 5) sym_apply_two_kernel(int64_t ne, IX ix
   cg2_end_a<4>(o2, pq);
 }
 
-// FP64-accurate refinement apply on the FP32 pipe: S_K = hi + lo (hi = fl32(S_K), lo = fl32(S_K - hi)),
-// x in double-floats, compensated sums. Bounded by the bytes of the two copies; pipelined as above.
-// 24,576 tets of degrees 1..4: 0.47 ms (0.72 to 1.47 ms, by the tile chosen, with the whole blocks).
+// Refinement apply of the per-element degrees on the FP32 pipe: S_K = hi + lo (hi = fl32(S_K), lo =
+// fl32(S_K - hi)), x in double-floats, compensated sums. Bounded by the bytes of the two copies; pipelined
+// as above. 24,576 tets of degrees 1..4: 0.47 ms (0.72 to 1.47 ms, by the tile chosen, with the whole blocks).
+// With one degree the residual comes from the FP64 blocks: this kernel was faster there (7,986 tets, k = 2: 57
+// instead of 95 us), but a solve stalled at a residual of 1e-13 to 2e-13 |b| at alpha = 0.2 (48 to 384 tets, k = 2
+// and 3; 4e-12 at alpha = 0.01), above the default tolerance, where FP64 reaches 1e-14 (1.6e-13).
 template <class IX>
 __global__ void __launch_bounds__(128, 4) sym_apply_df_kernel(int64_t ne, IX ix, const float* __restrict__ Shi,
                                                               const float* __restrict__ Slo, const double* __restrict__ x,
@@ -266,8 +269,9 @@ __global__ void __launch_bounds__(128, 4) sym_apply_df_kernel(int64_t ne, IX ix,
   }
 }
 
-// The packed copies of every S_K (row-major FP64): hi, lo and, with S16, the FP16 copy with one scale per
-// element (max |S_K| rounded up, so that every stored value lies in [-1, 1]). CTA per element.
+// The packed copies of every S_K (row-major FP64): hi; the remainder, where lo is given; and with S16 the FP16
+// copy with one scale per element (max |S_K| rounded up, so that every stored value lies in [-1, 1]). CTA
+// per element.
 template <class IX>
 __global__ void __launch_bounds__(256) sym_pack_kernel(int64_t ne, IX ix, const double* __restrict__ S, float4* __restrict__ hi,
                                                        float4* __restrict__ lo, uint4* __restrict__ S16,
@@ -304,7 +308,7 @@ __global__ void __launch_bounds__(256) sym_pack_kernel(int64_t ne, IX ix, const 
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         hi[o + 32 * q] = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-        lo[o + 32 * q] = make_float4(l[4 * q], l[4 * q + 1], l[4 * q + 2], l[4 * q + 3]);
+        if (lo) lo[o + 32 * q] = make_float4(l[4 * q], l[4 * q + 1], l[4 * q + 2], l[4 * q + 3]);
       }
       if (S16) {
         unsigned p[4];
