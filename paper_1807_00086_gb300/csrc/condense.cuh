@@ -209,12 +209,15 @@ __global__ void __launch_bounds__(32) condense_kernel(DevMesh mesh, CondTabs T, 
 
 // The same for small meshes: one CTA of four warps per element, which also writes the coefficients of the
 // local solves (local_co_kernel). A warp of condense_kernel that is alone on its SM partition takes 64 cycles
-// per FP64 instruction, for EPW elements, while other partitions are idle. hdg_condense with the read-back of S,
-// this kernel / condense_kernel: 162 tets, k = 2: 98 / 127 us, k = 4: 378 / 569 us; 750 tets, k = 2: 114 / 128,
-// k = 3: 224 / 307, k = 4: 652 / 616; 1,296 tets, k = 2: 145 / 131, k = 3: 335 / 333 us; 800 triangles: as fast.
+// per FP64 instruction, for EPW elements, while other partitions are idle. hdg_condense in mixed precision, this
+// kernel / condense_kernel, us: triangles, k = 2: 128: 53 / 59, 578: 61 / 63, 1,152: 72 / 63; k = 3: 128: 65 / 76,
+// 578: 75 / 76, 1,152: 91 / 76; k = 4: 128: 86 / 105, 578: 99 / 105, 1,152: 128 / 107. Tetrahedra, k = 1: 384:
+// 54 / 63, 750: 61 / 61, 1,296: 74 / 64; k = 2: 384: 85 / 105, 750: 95 / 107, 1,296: 128 / 113; k = 3: 384:
+// 162 / 286, 750: 209 / 287, 1,296: 321 / 298; k = 4: 384: 382 / 500, 750: 536 / 508. The lines lie where this
+// kernel still gains: at most so many elements per SM.
 template <int DIM, int K>
 __host__ __device__ constexpr int cond_cta_per_sm() {
-  return DIM == 3 ? 2 * CondCfg<DIM, K>::EPW : 4;   // at most so many elements per SM
+  return DIM == 3 && (K == 2 || K == 3) ? 6 : 4;
 }
 template <int DIM, int K>
 __global__ void __launch_bounds__(128) condense_cta_kernel(DevMesh mesh, Tabs T, double alpha, double tau,

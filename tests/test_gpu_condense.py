@@ -69,3 +69,33 @@ def test_either_side_of_the_small_mesh_rule(dim, k, over):
     lam = inputs.random_traces(s.n_faces, s.Nf, 5).reshape(s.n_faces, s.Nf)
     u = s.hdg_recover(torch.tensor(F, device="cuda"), torch.tensor(lam, device="cuda")).cpu().numpy()
     assert relerr(u, ac.recover(prob, cond, F, lam)) < 1e-12
+
+
+@pytest.mark.parametrize("dim,k", [(2, 1), (2, 2), (2, 3), (2, 4), (3, 1), (3, 2), (3, 3), (3, 4)])
+def test_both_kernels_agree_at_the_rule(dim, k):
+    """Up to a number of elements per SM a CTA condenses one element, above it a warp several: on both sides of
+    that line, with every number of elements in the last warp, the last elements' S_K and local solves against
+    those of a mesh of these elements alone (<= 1e-12: the same formulas in another order)."""
+    import torch
+    from paper_1807_00086_gb300 import hdg
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    line = (6 if dim == 3 and k in (2, 3) else 4) * sms
+    N = 1
+    while (2 * N * N if dim == 2 else 6 * N ** 3) < line + 4:
+        N += 1
+    vert, elem = mesh(dim, N)
+    rho, c = inputs.loguniform(line + 4, 0.5, 2.0, 3), inputs.loguniform(line + 4, 1.0, 3.0, 4)
+    n = (dim + 1) * ((k + 1) * (k + 2) // 2 if dim == 2 else (k + 1) * (k + 2) * (k + 3) // 6)
+    F = inputs.random_state(line + 4, n, 11)
+
+    def blocks(ids):
+        used, inv = np.unique(elem[ids], return_inverse=True)
+        s = hdg.Solver(vert[used], inv.reshape(elem[ids].shape).astype(np.int32), k, 1.0, rho[ids], c[ids])
+        s.hdg_condense(37.0)
+        u = s.hdg_recover(torch.tensor(F[ids], device="cuda"), s.empty_traces())
+        return s.hdg_get_schur().cpu().numpy(), u.cpu().numpy()
+
+    for ne in range(line, line + 5):
+        S, u = blocks(np.arange(ne))
+        Sl, ul = blocks(np.arange(ne - 7, ne))
+        assert relerr(S[-7:], Sl) < 1e-12 and relerr(u[-7:], ul) < 1e-12
