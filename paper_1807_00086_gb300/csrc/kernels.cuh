@@ -1481,7 +1481,7 @@ __device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
   hi = __uint_as_float(sign | ((((unsigned)(ex - 896) << 23) | m) + up));
   // the signed remainder in units of the last FP64 place, rounded once
   const float rl = (float)((int)rem - (int)(up << 29)) * __uint_as_float((unsigned)(ex - 948) << 23);
-  lo = sign ? -rl : rl;
+  lo = sign ? 0.f - rl : rl;   // an exact value leaves +0, as v - hi does
 }
 
 // (double)h + (double)l for a normalised pair, the same bits, on the integer pipe: l in units of the
