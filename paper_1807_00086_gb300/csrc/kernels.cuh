@@ -1492,11 +1492,13 @@ __device__ __forceinline__ double join_f64(float h, float l) {
   if (eh >= 80 && eh < 255) {
     const float ls = l * __uint_as_float((unsigned)(306 - eh) << 23);   // exact: a power of two
     const long long m = ((long long)((hb & 0x7fffffu) | 0x800000u) << 29) + __float2int_rn((int)hb < 0 ? -ls : ls);
-    if (m >= (1ll << 52) && fabsf(ls) < 1073741824.f)
+    if (m > (1ll << 52) && fabsf(ls) < 1073741824.f)
       return __hiloint2double((int)((hb & 0x80000000u) | ((unsigned)(m >> 32) - 0x100000u + ((unsigned)(eh + 896) << 20))),
                               (int)(unsigned)m);
   }
-  return (double)h + (double)l;   // zero, tiny, not finite, or a sum below the binade of h
+  // zero, tiny, not finite, a sum below the binade of h, or one that rounded up to its edge: the places there
+  // are half as far apart
+  return (double)h + (double)l;
 }
 
 // compensated accumulator of sum_i a_i b_i with a_i, b_i double-floats

@@ -1,6 +1,7 @@
-"""split_f64 (a double as a pair of floats, on the integer pipe) against the plain conversions, bit for bit:
-random signs, exponents and significands over the whole range of doubles, ties of the first rounding and their
-neighbours, carries into the next binade, and the exponents at which it changes over to the conversions."""
+"""split_f64 and join_f64 (a double as a pair of floats and back, on the integer pipe) against the plain
+conversions, bit for bit: random signs, exponents and significands over the whole range of doubles, ties of the
+first rounding and their neighbours, carries into the next binade, the exponents at which the routines change
+over to the conversions, and pairs whose sum lies below the binade of the head."""
 import ctypes
 import pathlib
 import subprocess
@@ -15,8 +16,15 @@ SOURCE = """
 __global__ void split_k(int64_t n, const double* v, float* h, float* l) {
   for (int64_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) hdg::split_f64(v[i], h[i], l[i]);
 }
+__global__ void join_k(int64_t n, const float* h, const float* l, double* v) {
+  for (int64_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) v[i] = hdg::join_f64(h[i], l[i]);
+}
 extern "C" int split(int64_t n, const double* v, float* h, float* l) {
   split_k<<<256, 256>>>(n, v, h, l);
+  return (int)cudaDeviceSynchronize();
+}
+extern "C" int join(int64_t n, const float* h, const float* l, double* v) {
+  join_k<<<256, 256>>>(n, h, l, v);
   return (int)cudaDeviceSynchronize();
 }
 """
@@ -75,3 +83,23 @@ def test_split(lib):
     dev = torch.tensor(v, device="cuda")
     gh, gl = _call(lib.split, v.size, [dev], [torch.empty(v.size, dtype=torch.float32, device="cuda") for _ in range(2)])
     assert _same(gh, h) and _same(gl, l)
+
+
+def test_join(lib):
+    import torch
+    rng = np.random.default_rng(18)
+    h, l = _pair(_doubles())
+    keep = np.isfinite(h)
+    h, l = h[keep], l[keep]
+    # normalised pairs of every size of l: up to half a unit of the head's last place, also exactly that
+    with np.errstate(all="ignore"):
+        ulp = np.spacing(np.abs(h)) / np.float32(2)
+        ulp = np.where(np.abs(h).view(np.uint32) & np.uint32((1 << 23) - 1), ulp, ulp / np.float32(2)).astype(np.float32)
+        part = np.ldexp(rng.uniform(-1, 1, h.size), -rng.integers(0, 60, h.size)).astype(np.float32)
+        part[::3] = rng.choice(np.array([-1, 1, 0, -0.5, 0.5], dtype=np.float32), part[::3].size)
+        l2 = (ulp * part).astype(np.float32)
+    h, l = np.concatenate([h, h]), np.concatenate([l, np.where(np.isfinite(l2), l2, np.float32(0))])
+    want = h.astype(np.float64) + l.astype(np.float64)
+    got, = _call(lib.join, h.size, [torch.tensor(h, device="cuda"), torch.tensor(l, device="cuda")],
+                 [torch.empty(h.size, dtype=torch.float64, device="cuda")])
+    assert _same(got, want)
