@@ -2065,6 +2065,7 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
     c->nfe4 = (int64_t)((nfe + 3) / 4) * 4;
     const size_t n32 = c->R > 1 ? nfe * R : (size_t)c->nfe4;
     for (float** p : {&c->d_dinv32, &c->d_r32, &c->d_z32, &c->d_p32, &c->d_q32, &c->d_x32, &c->d_b32}) {
+      if (p == &c->d_q32 && c->R == 1) continue;   // one column forms q in its update
       const size_t cnt = p == &c->d_dinv32 ? (size_t)c->nfe4 : n32;
       if ((s = dalloc(c, p, cnt))) return s;
       CUDA_TRY(c, cudaMemsetAsync(*p, 0, cnt * 4, c->stream));

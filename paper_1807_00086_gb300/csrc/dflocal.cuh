@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(LocalCfg<DIM, K, CW>::NT)
   }
   for (int t = tid; t < 4 * GW; t += NT) {
     const int64_t e = e0 + (ONE ? t / 4 : t / 8);
-    AR::set(co[t % 4], ONE ? t / 4 : t / 4, e < mesh.ne ? coef[4 * e + t % 4] : V{});
+    AR::set(co[t % 4], t / 4, e < mesh.ne ? coef[4 * e + t % 4] : V{});
   }
   for (int q = tid; q < EPB; q += NT) {
     int use = 0;

@@ -682,7 +682,7 @@ hdg_status vd_setup(hdg_ctx* c, const int32_t* elem_k) {
     }
     if ((s = dalloc(c, &c->d_slot32, (size_t)v->m_tot))) return s;
     c->nfe4 = (int64_t)((ntr + 3) / 4) * 4;
-    for (float** p : {&c->d_dinv32, &c->d_r32, &c->d_z32, &c->d_p32, &c->d_q32, &c->d_x32, &c->d_b32}) {
+    for (float** p : {&c->d_dinv32, &c->d_r32, &c->d_z32, &c->d_p32, &c->d_x32, &c->d_b32}) {
       if ((s = dalloc(c, p, (size_t)c->nfe4))) return s;
       CUDA_TRY(c, cudaMemsetAsync(*p, 0, (size_t)c->nfe4 * 4, c->stream));
     }
