@@ -406,7 +406,8 @@ hdg_status hdg_trace_apply_noalloc(int32_t dim, int32_t k, int64_t n_elem, int64
  * double-float refinement-residual kernel, apply32: the inner apply) read packed copies of S_K
  * and have one tile, 4 warps x 8 entries per lane. At the first local solve of
  * each kind it times the block size of the one-launch element-local solve (64, 128 or 256
- * threads per element). tuned = 0 before the first condensation; local_threads are 0 until
+ * threads per element). tuned = 0 before the first condensation, then 1: the apply tiles are those
+ * in use (timed in FP64, the fixed ones with mixed precision); local_threads are 0 until
  * the first condensed right-hand side (index 0) / recovery (index 1). HDG_EINVAL for a
  * context without per-element degrees. */
 typedef struct {

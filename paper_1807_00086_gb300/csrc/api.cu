@@ -490,9 +490,9 @@ hdg_status cg32_inner(hdg_ctx* c, int* iters, double tol, int* last, bool use16)
   return HDG_OK;
 }
 
-// Mixed precision: FP64 iterative refinement of (-K) x = bvec. Each sweep forms the FP64
-// residual with the FP64 S_K, solves for the correction with FP32 S_K (inner PCG with FP64
-// inner products) and adds it to x in FP64.
+// Mixed precision: iterative refinement of sgn K x = bvec. Each sweep forms the residual (acoustic: from the
+// double-float copy of S_K; elastic: from the FP64 blocks), solves for the correction with the FP32 or FP16
+// copy of S_K (inner PCG in FP32, its inner products as compensated pairs) and adds it to x in FP64.
 hdg_status solve_mixed(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info* info) {
   const int64_t nfe = c->sk.nf * c->Nf;
   const int nb = c->nb_red;
@@ -1935,8 +1935,10 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   CUDA_TRY(c, cudaGetDevice(&dev));
   CUDA_TRY(c, cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev));
   {
-    // reduction grid = one resident wave of the heaviest vector kernel (no partial second wave), three
-    // CTAs of 256 threads per SM
+    // reduction grid: three CTAs of 256 threads per SM, a resident wave of every vector kernel. Against four:
+    // IEDG mixed, 10,368 tets, 1.50 / 1.56 ms; GMRES + Jacobi 5.54 / 5.73; two columns 4.85 / 5.06; 128 columns,
+    // 16,464 tets, 46.8 / 48.7; elastic, k = 2, 11.7 / 11.9; 196,608 tets, k = 3, 91.1 / 92.9; 64 columns and
+    // FP64 columns as fast
     c->nb_red = std::max(1, std::min(3 * c->sms, (int)((c->sk.nf * c->Nf + 255) / 256)));
   }
   const int64_t ne = c->sk.ne, nf = c->sk.nf, nb = c->sk.nb, nc = c->nfc;
@@ -2052,8 +2054,8 @@ hdg_status hdg_setup(const hdg_mesh* mesh, int32_t k, double tau, const hdg_mate
   if (c->opt.prec != HDG_FP64) {
     const int64_t ngroups = (ne + 31) / 32;
     const int P4 = (c->m * (c->m + 1) / 2 + 3) / 4;
-    // elastic: packed copies where they are smaller; an SVK step copies S_K in every Newton iteration
-    // and applies it a few times only
+    // elastic: packed copies where they are smaller. SVK keeps whole blocks: packed ones, which every Newton
+    // iteration would have to write again for its 45 or so applies (1,536 tets, k = 2), were not tried
     c->sym32 = c->phys == HDG_ELASTIC && !svk && sym_pays(c->m);
     const size_t nS32 = c->sym32 ? (size_t)ne * sym_units(c->m) * 256
                         : c->phys == HDG_ELASTIC ? (size_t)ne * c->m * c->m : (size_t)ngroups * P4 * 128;

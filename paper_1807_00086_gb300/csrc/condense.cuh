@@ -349,6 +349,8 @@ static __global__ void to_df_kernel(int64_t n, const double* __restrict__ a, df2
 // (null: not wanted). One kernel per copy read S_K up to four times and searched the row of every
 // packed entry: 2.61 ms for the FP32, FP16 and double-float copies of 82,944 blocks of 40 x 40,
 // against 0.57 ms here; what remains is the shared-memory transposition and the 2.0 GB moved.
+// An FP16 entry is the FP32 quotient of hi and the scale, rounded: at most 2^-23 of it beside the 2^-11 of the
+// rounding.
 struct PackOut {
   float* Sdf;      // [e][hi | lo] diagonal-major upper triangles (refinement apply)
   float* S32;      // [group][P4][32][4] packed rows of the upper triangle

@@ -924,8 +924,8 @@ __device__ __forceinline__ void block_cols_v(const double (&v)[NV], int R, doubl
 }
 
 // q = (-K) p from the two slots of each interior entry; partial p.q per column. The reducing
-// kernels of this family are bounded to 64 registers, so four 256-thread CTAs are resident per
-// SM and the reduction grid (a multiple of the SM count) runs in whole waves.
+// kernels of this family are bounded to 64 registers: four 256-thread CTAs fit an SM, and the reduction
+// grid of at most three per SM is one wave.
 template <int DIM, int K>
 __global__ void __launch_bounds__(256, 4) mface_q4_kernel(int nf, int R, const int2* __restrict__ face_slot2,
                                                        const int32_t* __restrict__ face_bnd,

@@ -270,7 +270,8 @@ __global__ void __launch_bounds__(128, 4) sym_apply_df_kernel(int64_t ne, IX ix,
 }
 
 // The packed copies of every S_K (row-major FP64): hi; the remainder, where lo is given; and with S16 the FP16
-// copy with one scale per element (max |S_K| rounded up, so that every stored value lies in [-1, 1]). CTA
+// copy with one scale per element (max |S_K| rounded up, so that every stored value lies in [-1, 1]). An FP16 entry
+// is the FP32 quotient of hi and the scale, rounded: at most 2^-23 of it beside the 2^-11 of the rounding. CTA
 // per element.
 template <class IX>
 __global__ void __launch_bounds__(256) sym_pack_kernel(int64_t ne, IX ix, const double* __restrict__ S, float4* __restrict__ hi,

@@ -323,7 +323,7 @@ hdg_status vd_cg32(hdg_ctx* c, double tol, int* iters, bool use16) {
   return HDG_OK;
 }
 
-// FP64 iterative refinement: FP64 residual with the FP64 S_K, FP32 correction solves.
+// Iterative refinement: residual from the double-float copy of S_K, correction solves in FP32, x in FP64.
 hdg_status vd_refine(hdg_ctx* c, const double* bvec, double* x, hdg_solve_info* info) {
   const int64_t n = c->ntr;
   const int nb = c->nb_red;
