@@ -633,7 +633,8 @@ def run_ours(args):
 def sym_units(m):
     """16 x 16 units on and above the diagonal of an m x m block."""
     nb = (np.asarray(m) + 15) // 16
-    return nb * (nb + 1) // 2
+    u = nb * (nb + 1) // 2
+    return int(u) if u.ndim == 0 else u   # a NumPy integer is no JSON number
 
 
 def packed_entries(elem, ek):
