@@ -613,7 +613,7 @@ def run_ours(args):
                           "trace_space": args.trace_space, "solver": args.solver,
                           "precond": args.precond if args.solver == "gmres" else "jacobi",
                           "trace_unknowns": int(s.sizes.trace_unknowns) * R,
-                          "trace_solve": "host-driven loops" if (args.host_loops or R > 1) else
+                          "trace_solve": "host-driven loops" if args.host_loops else
                           "one CUDA-graph launch per trace solve (device-side loop conditions)"},
                "roofline": roof, "cpu_baseline": cpu, "fp64_gpu": fp64,
                "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 2 * field_bytes + trace_bytes,
