@@ -264,7 +264,7 @@ __device__ __forceinline__ double cta_ratio(double a, double b) {
 // of the other iteration parity, so that no CTA reads what it writes. A small system's iteration is
 // bounded by the latency of its dependent kernels and of their sums: 16,562 triangles, k = 3: 9.2 us
 // (21.0 us as apply, update and direction with FP64 sums). The pairs of a thread were summed in FP64 there: an error of
-// 1e-16 to 3e-15 of sum |terms| (300 to 4 million entries, factors over e^4), as pairs 1e-15 to 1.4e-14. alpha and
+// 1e-16 to 3e-15 of sum |terms| (300 to 4 million entries, lognormal factors), as pairs 1e-15 to 1.4e-14. alpha and
 // beta are FP32 either way, and the rounded sums were the same.
 struct Cg2State {
   float2 rho[2];     // (r, z) of the iteration with this parity
